@@ -69,13 +69,6 @@ __device__ __forceinline__ void face_cells(const Dims& d, long long f, long long
   }
 }
 
-__device__ __forceinline__ void q1_ref_grad(int a, double xi, double eta, double zeta, double g[3]) {
-  const double sx = (a & 1) ? 1.0 : -1.0, sy = ((a >> 1) & 1) ? 1.0 : -1.0, sz = ((a >> 2) & 1) ? 1.0 : -1.0;
-  g[0] = 0.125 * sx * (1.0 + sy * eta) * (1.0 + sz * zeta);
-  g[1] = 0.125 * sy * (1.0 + sx * xi) * (1.0 + sz * zeta);
-  g[2] = 0.125 * sz * (1.0 + sx * xi) * (1.0 + sy * eta);
-}
-
 __device__ __forceinline__ void load_cell_coords(const Dims& d, const double* __restrict__ coords, long long T,
                                                  double X[8][3]) {
   const int i = (int)(T % d.nx), j = (int)((T / d.nx) % d.ny), k = (int)(T / ((long long)d.nx * d.ny));
@@ -87,85 +80,138 @@ __device__ __forceinline__ void load_cell_coords(const Dims& d, const double* __
 }
 
 // ---------------------------------------------------------------- K1: Q1
-// One warp per cell.  Appendix A: [A_uu]_ab = (grad^s eta_a, C_dr grad^s
-// eta_b)_T; for isotropic C_dr the 3x3 block is
+// Appendix A: [A_uu]_ab = (grad^s eta_a, C_dr grad^s eta_b)_T; for isotropic
+// C_dr the 3x3 block is
 //   K_ab(i,j) = int lam d_i N_a d_j N_b + G d_j N_a d_i N_b + G delta_ij grad N_a . grad N_b,
 // [A_up]_(a,c) = -b int d_c N_a, |T| = int 1.  2x2x2 Gauss.
-constexpr int Q1_WARPS = 4;
-__global__ void __launch_bounds__(32 * Q1_WARPS) k_q1(Dims d, const double* __restrict__ coords,
-                                                      const double* __restrict__ E, const double* __restrict__ nu,
-                                                      const double* __restrict__ biot, double* __restrict__ Ke,
-                                                      double* __restrict__ Aup, double* __restrict__ vol,
-                                                      int* __restrict__ flag) {
-  __shared__ double sG[Q1_WARPS][8][8][3];
-  __shared__ double sW[Q1_WARPS][8];
-  __shared__ double sX[Q1_WARPS][8][3];
+//
+// The FP64 pipe (2 FMA per clock and SM) bounds this kernel, so it is written
+// for few FP64 operations: lam and G are constant in the cell, so the block
+// follows from H_ab = int grad N_a (x) grad N_b alone, K_ab = lam H + G H^T +
+// G tr(H) I, and only the 36 pairs a <= b are integrated (K_ba = K_ab^T, so
+// the stored element matrix is exactly symmetric): about 5,000 operations per
+// cell instead of 25,000 with the integrand summed term by term over all 64
+// pairs.  A block takes 32 consecutive cells, a lane per cell, so every store
+// is one full row segment; warp q first forms the gradients at Gauss point q
+// in shared memory, then warp a takes the pairs (a, a + d mod 8), d = 0..3,
+// and d = 4 for a < 4 (nine pairs per scheduler).  96^3 cells: 49.5 ms before
+// (one warp per cell, a store per lane and row), 7.93 ms now (590 G FP64 FMA-slots per second, 0.97 of the pipe).
+constexpr int Q1_CELLS = 32;
+constexpr size_t Q1_SMEM = (8 * 24 + 8) * Q1_CELLS * sizeof(double);
+
+// 0.125 (1 + s g)(1 + t g) of a Q1 derivative's two transverse factors, s, t =
+// whether the node and the Gauss point lie on the same side
+__device__ __forceinline__ double q1_trans(bool s, bool t) {
+  constexpr double P = 0.125 * (1.0 + kGP) * (1.0 + kGP), M = 0.125 * (1.0 + kGP) * (1.0 - kGP),
+                   N = 0.125 * (1.0 - kGP) * (1.0 - kGP);
+  return s ? (t ? P : M) : (t ? M : N);
+}
+
+__global__ void __launch_bounds__(256, 2) k_q1(Dims d, const double* __restrict__ coords,
+                                               const double* __restrict__ E, const double* __restrict__ nu,
+                                               const double* __restrict__ biot, double* __restrict__ Ke,
+                                               double* __restrict__ Aup, double* __restrict__ vol,
+                                               int* __restrict__ flag) {
+  extern __shared__ double q1_sh[];
+  double* sG = q1_sh;                       // [8 Gauss points][24 = 3 a + i][32 cells]
+  double* sW = q1_sh + 8 * 24 * Q1_CELLS;   // [8][32] det J (Gauss weight 1)
   const int wp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const long long T = (long long)blockIdx.x * Q1_WARPS + wp;
-  if (T >= d.nT) return;  // whole warp leaves together; only __syncwarp below
-  const int ci = (int)(T % d.nx), cj = (int)((T / d.nx) % d.ny), ck = (int)(T / ((long long)d.nx * d.ny));
-  if (lane < 24) {
-    const int a = lane / 3, c = lane % 3;
-    sX[wp][a][c] = coords[3 * node_id(d, ci + (a & 1), cj + ((a >> 1) & 1), ck + ((a >> 2) & 1)) + c];
-  }
-  __syncwarp();
-  if (lane < 8) {
-    const double xi = (lane & 1) ? kGP : -kGP, eta = ((lane >> 1) & 1) ? kGP : -kGP,
-                 zeta = ((lane >> 2) & 1) ? kGP : -kGP;
+  const long long T0 = (long long)blockIdx.x * Q1_CELLS + lane;
+  const bool valid = T0 < d.nT;
+  const long long T = valid ? T0 : d.nT - 1;
+  {
+    double X[8][3];
+    load_cell_coords(d, coords, T, X);
+    const bool qx = wp & 1, qy = (wp >> 1) & 1, qz = (wp >> 2) & 1;
+    // J(:, 0) = sum over the four x-edges of (transverse weight) (edge vector), and so on
     double J[3][3] = {{0, 0, 0}, {0, 0, 0}, {0, 0, 0}};
-    double gr[8][3];
-    for (int a = 0; a < 8; ++a) {
-      q1_ref_grad(a, xi, eta, zeta, gr[a]);
-      for (int i = 0; i < 3; ++i)
-        for (int j = 0; j < 3; ++j) J[i][j] += sX[wp][a][i] * gr[a][j];
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+      const bool u = e & 1, v = e >> 1;
+      const double wx = q1_trans(u == qy, v == qz), wy = q1_trans(u == qx, v == qz), wz = q1_trans(u == qx, v == qy);
+#pragma unroll
+      for (int i = 0; i < 3; ++i) {
+        J[i][0] += wx * (X[1 + 2 * e][i] - X[2 * e][i]);
+        J[i][1] += wy * (X[(e & 1) + 2 + 4 * (e >> 1)][i] - X[(e & 1) + 4 * (e >> 1)][i]);
+        J[i][2] += wz * (X[e + 4][i] - X[e][i]);
+      }
     }
     const double c00 = J[1][1] * J[2][2] - J[1][2] * J[2][1];
     const double c01 = J[1][2] * J[2][0] - J[1][0] * J[2][2];
     const double c02 = J[1][0] * J[2][1] - J[1][1] * J[2][0];
     const double det = J[0][0] * c00 + J[0][1] * c01 + J[0][2] * c02;
-    if (!(det > 0.0)) atomicOr(flag, 1);
+    if (valid && !(det > 0.0)) atomicOr(flag, 1);
     const double id = 1.0 / det;
     double Ji[3][3];
     Ji[0][0] = c00 * id; Ji[0][1] = (J[0][2] * J[2][1] - J[0][1] * J[2][2]) * id; Ji[0][2] = (J[0][1] * J[1][2] - J[0][2] * J[1][1]) * id;
     Ji[1][0] = c01 * id; Ji[1][1] = (J[0][0] * J[2][2] - J[0][2] * J[2][0]) * id; Ji[1][2] = (J[0][2] * J[1][0] - J[0][0] * J[1][2]) * id;
     Ji[2][0] = c02 * id; Ji[2][1] = (J[0][1] * J[2][0] - J[0][0] * J[2][1]) * id; Ji[2][2] = (J[0][0] * J[1][1] - J[0][1] * J[1][0]) * id;
-    for (int a = 0; a < 8; ++a)
+#pragma unroll
+    for (int a = 0; a < 8; ++a) {
+      const bool ax = a & 1, ay = (a >> 1) & 1, az = (a >> 2) & 1;
+      const double tx = q1_trans(ay == qy, az == qz), ty = q1_trans(ax == qx, az == qz), tz = q1_trans(ax == qx, ay == qy);
+      const double g0 = ax ? tx : -tx, g1 = ay ? ty : -ty, g2 = az ? tz : -tz;
+#pragma unroll
       for (int i = 0; i < 3; ++i)
-        sG[wp][lane][a][i] = gr[a][0] * Ji[0][i] + gr[a][1] * Ji[1][i] + gr[a][2] * Ji[2][i];
-    sW[wp][lane] = det;  // Gauss weight 1
-  }
-  __syncwarp();
-  const double e = E[T], v = nu[T];
-  const double lam = e * v / ((1.0 + v) * (1.0 - 2.0 * v));
-  const double G = e / (2.0 * (1.0 + v));
-  const long long nT = d.nT;
-#pragma unroll 1
-  for (int rep = 0; rep < 2; ++rep) {
-    const int a = (lane >> 3) + 4 * rep, b = lane & 7;
-    double K[3][3] = {{0, 0, 0}, {0, 0, 0}, {0, 0, 0}};
-    for (int q = 0; q < 8; ++q) {
-      const double w = sW[wp][q];
-      const double* ga = sG[wp][q][a];
-      const double* gb = sG[wp][q][b];
-      const double dot = ga[0] * gb[0] + ga[1] * gb[1] + ga[2] * gb[2];
-      for (int i = 0; i < 3; ++i)
-        for (int j = 0; j < 3; ++j)
-          K[i][j] += w * (lam * ga[i] * gb[j] + G * ga[j] * gb[i] + (i == j ? G * dot : 0.0));
+        sG[(wp * 24 + 3 * a + i) * Q1_CELLS + lane] = g0 * Ji[0][i] + g1 * Ji[1][i] + g2 * Ji[2][i];
     }
+    sW[wp * Q1_CELLS + lane] = det;
+  }
+  __syncthreads();
+  const int a = wp;
+  double H[5][9], ga_sum[3] = {0, 0, 0}, v = 0.0;
+#pragma unroll
+  for (int p = 0; p < 5; ++p)
+#pragma unroll
+    for (int e = 0; e < 9; ++e) H[p][e] = 0.0;
+#pragma unroll 1
+  for (int q = 0; q < 8; ++q) {
+    const double w = sW[q * Q1_CELLS + lane];
+    const double* g = sG + q * 24 * Q1_CELLS + lane;
+    double ga[3];
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+      ga[i] = w * g[(3 * a + i) * Q1_CELLS];
+      ga_sum[i] += ga[i];
+    }
+    v += w;
+#pragma unroll
+    for (int p = 0; p < 5; ++p) {
+      if (p == 4 && a >= 4) break;  // warp-uniform
+      const int b = (a + p) & 7;
+#pragma unroll
+      for (int j = 0; j < 3; ++j) {
+        const double gb = g[(3 * b + j) * Q1_CELLS];
+#pragma unroll
+        for (int i = 0; i < 3; ++i) H[p][3 * i + j] += ga[i] * gb;
+      }
+    }
+  }
+  if (!valid) return;
+  const double e = E[T], pr = nu[T];
+  const double lam = e * pr / ((1.0 + pr) * (1.0 - 2.0 * pr));
+  const double G = e / (2.0 * (1.0 + pr));
+  const double lamG = lam + G;
+  const long long nT = d.nT;
+#pragma unroll
+  for (int p = 0; p < 5; ++p) {
+    if (p == 4 && a >= 4) break;
+    const int b = (a + p) & 7;
+    const double gt = G * (H[p][0] + H[p][4] + H[p][8]);
+#pragma unroll
     for (int i = 0; i < 3; ++i)
-      for (int j = 0; j < 3; ++j) Ke[(long long)((3 * a + i) * 24 + 3 * b + j) * nT + T] = K[i][j];
+#pragma unroll
+      for (int j = 0; j < 3; ++j) {
+        if (p == 0 && j < i) continue;  // the (a, a) block is symmetric: its upper triangle, stored twice
+        const double k = i == j ? lamG * H[p][4 * i] + gt : lam * H[p][3 * i + j] + G * H[p][3 * j + i];
+        Ke[(long long)((3 * a + i) * 24 + 3 * b + j) * nT + T] = k;
+        if (p != 0 || i != j) Ke[(long long)((3 * b + j) * 24 + 3 * a + i) * nT + T] = k;
+      }
   }
-  if (lane < 24) {
-    const int a = lane / 3, c = lane % 3;
-    double s = 0.0;
-    for (int q = 0; q < 8; ++q) s += sW[wp][q] * sG[wp][q][a][c];
-    Aup[(long long)lane * nT + T] = -biot[T] * s;
-  }
-  if (lane == 0) {
-    double s = 0.0;
-    for (int q = 0; q < 8; ++q) s += sW[wp][q];
-    vol[T] = s;
-  }
+  const double bi = biot[T];
+#pragma unroll
+  for (int c = 0; c < 3; ++c) Aup[(long long)(3 * a + c) * nT + T] = -bi * ga_sum[c];
+  if (a == 0) vol[T] = v;
 }
 
 // ---------------------------------------------------------------- K2: RT0
@@ -174,89 +220,158 @@ __global__ void __launch_bounds__(32 * Q1_WARPS) k_q1(Dims d, const double* __re
 // reference basis (phi_hat of local face 2d / 2d+1 is -(1-xi_d)/8 e_d /
 // (1+xi_d)/8 e_d).  Condensation (Eq. hmfeSys): W_T = A_ww,T^-1, W_T 1,
 // 1^T W_T 1, Abar_pp,T = S_eps|T| + dt 1^T W_T 1.
-__global__ void k_rt0(Dims d, const double* __restrict__ coords, const double* __restrict__ mu,
+//
+// Bound by the FP64 pipe: column d of J depends on the two other coordinates
+// of the Gauss point only (12 columns per cell instead of 24), A_ww is
+// symmetric (21 entries, the reference basis' products are constants), and
+// W = L^-T L^-1 from the Cholesky factor needs six reciprocal square roots
+// and no division: about 1,000 FP64 operations per cell against 4,000 for
+// the plain sums and column-by-column solves.  96^3 cells: 4.97 ms before,
+// 1.46 ms now.
+__global__ void __launch_bounds__(128) k_rt0(Dims d, const double* __restrict__ coords, const double* __restrict__ mu,
                       const double* __restrict__ kappa, const double* __restrict__ Seps,
                       const double* __restrict__ vol, double dt, double* __restrict__ Wout,
                       double* __restrict__ W1out, double* __restrict__ sWout, double* __restrict__ Abar,
                       int* __restrict__ flag, double* __restrict__ Aww_out = nullptr) {
   const long long T = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (T >= d.nT) return;
-  double X[8][3];
-  load_cell_coords(d, coords, T, X);
+  // col[ax][c]: column ax of J where the Gauss point's other two coordinates
+  // (in axis order) have the sides c & 1 and c >> 1
+  double col[3][4][3];
+  {
+    double X[8][3];
+    load_cell_coords(d, coords, T, X);
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+      double ed[3][4];
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        ed[0][e] = X[1 + 2 * e][i] - X[2 * e][i];
+        ed[1][e] = X[(e & 1) + 2 + 4 * (e >> 1)][i] - X[(e & 1) + 4 * (e >> 1)][i];
+        ed[2][e] = X[e + 4][i] - X[e][i];
+      }
+#pragma unroll
+      for (int ax = 0; ax < 3; ++ax)
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+          double s = 0.0;
+#pragma unroll
+          for (int e = 0; e < 4; ++e) s += q1_trans((e & 1) == (c & 1), (e >> 1) == (c >> 1)) * ed[ax][e];
+          col[ax][c][i] = s;
+        }
+    }
+  }
   const double m = mu[T];
   const double kinv[3] = {m / kappa[3 * T], m / kappa[3 * T + 1], m / kappa[3 * T + 2]};
-  double A[6][6];
+  double A[6][6];  // lower triangle
+#pragma unroll
   for (int f = 0; f < 6; ++f)
+#pragma unroll
     for (int g = 0; g < 6; ++g) A[f][g] = 0.0;
-  for (int q = 0; q < 8; ++q) {
-    const double xq[3] = {(q & 1) ? kGP : -kGP, ((q >> 1) & 1) ? kGP : -kGP, ((q >> 2) & 1) ? kGP : -kGP};
-    double J[3][3] = {{0, 0, 0}, {0, 0, 0}, {0, 0, 0}};
-    for (int a = 0; a < 8; ++a) {
-      double gr[3];
-      q1_ref_grad(a, xq[0], xq[1], xq[2], gr);
-      for (int i = 0; i < 3; ++i)
-        for (int j = 0; j < 3; ++j) J[i][j] += X[a][i] * gr[j];
+  bool bad = false;
+#pragma unroll
+  for (int qz = 0; qz < 2; ++qz)
+#pragma unroll
+  for (int qy = 0; qy < 2; ++qy)
+#pragma unroll
+  for (int qx = 0; qx < 2; ++qx) {
+    const int bit[3] = {qx, qy, qz};
+    double J[3][3], KJ[3][3];
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+      J[i][0] = col[0][qy + 2 * qz][i];
+      J[i][1] = col[1][qx + 2 * qz][i];
+      J[i][2] = col[2][qx + 2 * qy][i];
+#pragma unroll
+      for (int p = 0; p < 3; ++p) KJ[i][p] = kinv[i] * J[i][p];
     }
     const double det = J[0][0] * (J[1][1] * J[2][2] - J[1][2] * J[2][1]) -
                        J[0][1] * (J[1][0] * J[2][2] - J[1][2] * J[2][0]) +
                        J[0][2] * (J[1][0] * J[2][1] - J[1][1] * J[2][0]);
-    if (!(det > 0.0)) atomicOr(flag, 1);
-    // M_dd' = sum_i J_id J_id' (mu/kappa_i) / det
-    double M[3][3];
+    bad = bad || !(det > 0.0);
+    const double rd = 1.0 / det;
+    // the basis functions' factors at this point: lower face -(1 - xi)/8, upper (1 + xi)/8
+    constexpr double HI = (1.0 + kGP) * 0.125, LO = (1.0 - kGP) * 0.125;
+#pragma unroll
     for (int p = 0; p < 3; ++p)
-      for (int r = 0; r < 3; ++r) M[p][r] = (J[0][p] * J[0][r] * kinv[0] + J[1][p] * J[1][r] * kinv[1] + J[2][p] * J[2][r] * kinv[2]) / det;
-    double val[6];
-    for (int f = 0; f < 6; ++f) {
-      const int dd = f >> 1;
-      val[f] = (f & 1) ? (1.0 + xq[dd]) * 0.125 : -(1.0 - xq[dd]) * 0.125;
-    }
-    for (int f = 0; f < 6; ++f)
-      for (int g = 0; g < 6; ++g) A[f][g] += M[f >> 1][g >> 1] * val[f] * val[g];
+#pragma unroll
+      for (int r = 0; r < 3; ++r) {
+        if (r > p) continue;
+        // M_pr = sum_i J_ip J_ir (mu/kappa_i) / det
+        const double M = (KJ[0][p] * J[0][r] + KJ[1][p] * J[1][r] + KJ[2][p] * J[2][r]) * rd;
+#pragma unroll
+        for (int s = 0; s < 2; ++s)
+#pragma unroll
+          for (int t = 0; t < 2; ++t) {
+            if (2 * p + s < 2 * r + t) continue;
+            const double vs = s ? (bit[p] ? HI : LO) : (bit[p] ? -LO : -HI);
+            const double vt = t ? (bit[r] ? HI : LO) : (bit[r] ? -LO : -HI);
+            A[2 * p + s][2 * r + t] += M * (vs * vt);
+          }
+      }
   }
+  if (bad) atomicOr(flag, 1);
   if (Aww_out)
+#pragma unroll
     for (int f = 0; f < 6; ++f)
-      for (int g = 0; g < 6; ++g) Aww_out[(long long)(6 * f + g) * d.nT + T] = A[f][g];
-  // Cholesky A = L L^T, then W = A^-1 column by column
-  double L[6][6];
-  for (int i = 0; i < 6; ++i)
-    for (int j = 0; j < 6; ++j) L[i][j] = 0.0;
+#pragma unroll
+      for (int g = 0; g < 6; ++g) Aww_out[(long long)(6 * f + g) * d.nT + T] = f >= g ? A[f][g] : A[g][f];
+  // Cholesky A = L L^T in place (the diagonal holds 1 / L_jj), then L^-1 in place
+#pragma unroll
   for (int j = 0; j < 6; ++j) {
     double s = A[j][j];
-    for (int k = 0; k < j; ++k) s -= L[j][k] * L[j][k];
+#pragma unroll
+    for (int k = 0; k < 6; ++k)
+      if (k < j) s -= A[j][k] * A[j][k];
     if (!(s > 0.0)) { atomicOr(flag, 2); s = 1e-300; }
-    const double ljj = sqrt(s);
-    L[j][j] = ljj;
-    for (int i = j + 1; i < 6; ++i) {
-      double t = A[i][j];
-      for (int k = 0; k < j; ++k) t -= L[i][k] * L[j][k];
-      L[i][j] = t / ljj;
-    }
-  }
-  double W[6][6];
-  for (int c = 0; c < 6; ++c) {
-    double y[6];
+    const double rl = rsqrt(s);
+    A[j][j] = rl;
+#pragma unroll
     for (int i = 0; i < 6; ++i) {
-      double t = (i == c) ? 1.0 : 0.0;
-      for (int k = 0; k < i; ++k) t -= L[i][k] * y[k];
-      y[i] = t / L[i][i];
-    }
-    for (int i = 5; i >= 0; --i) {
-      double t = y[i];
-      for (int k = i + 1; k < 6; ++k) t -= L[k][i] * W[k][c];
-      W[i][c] = t / L[i][i];
+      if (i <= j) continue;
+      double t = A[i][j];
+#pragma unroll
+      for (int k = 0; k < 6; ++k)
+        if (k < j) t -= A[i][k] * A[j][k];
+      A[i][j] = t * rl;
     }
   }
-  // symmetrise (exact symmetry of the stored inverse)
-  double s1 = 0.0;
-  for (int f = 0; f < 6; ++f) {
-    double r = 0.0;
-    for (int g = 0; g < 6; ++g) {
-      const double wfg = 0.5 * (W[f][g] + W[g][f]);
-      Wout[(long long)(6 * f + g) * d.nT + T] = wfg;
-      r += wfg;
+#pragma unroll
+  for (int j = 0; j < 6; ++j)
+#pragma unroll
+    for (int i = 0; i < 6; ++i) {
+      if (i <= j) continue;
+      // (L^-1)_ij = -(sum_{k=j}^{i-1} L_ik (L^-1)_kj) / L_ii; row i of L is still
+      // whole to the right of column j, column j above row i is already inverted
+      double t = 0.0;
+#pragma unroll
+      for (int k = 0; k < 6; ++k)
+        if (k >= j && k < i) t += A[i][k] * A[k][j];
+      A[i][j] = -t * A[i][i];
     }
-    W1out[(long long)f * d.nT + T] = r;
-    s1 += r;
+  // W = L^-T L^-1 (stored exactly symmetric)
+  double W1[6] = {0, 0, 0, 0, 0, 0};
+#pragma unroll
+  for (int f = 0; f < 6; ++f)
+#pragma unroll
+    for (int g = 0; g < 6; ++g) {
+      if (g > f) continue;
+      double w = 0.0;
+#pragma unroll
+      for (int k = 0; k < 6; ++k)
+        if (k >= f) w += A[k][f] * A[k][g];
+      Wout[(long long)(6 * f + g) * d.nT + T] = w;
+      W1[f] += w;
+      if (g != f) {
+        Wout[(long long)(6 * g + f) * d.nT + T] = w;
+        W1[g] += w;
+      }
+    }
+  double s1 = 0.0;
+#pragma unroll
+  for (int f = 0; f < 6; ++f) {
+    W1out[(long long)f * d.nT + T] = W1[f];
+    s1 += W1[f];
   }
   sWout[T] = s1;
   Abar[T] = Seps[T] * vol[T] + dt * s1;
@@ -1270,8 +1385,9 @@ void assemble_all(Ctx& c) {
   double* Ke = dalloc_n<double>(c, (size_t)576 * c.nT);
   c.Aup = dalloc_n<double>(c, (size_t)24 * c.nT);
   c.vol = dalloc_n<double>(c, c.nT);
-  k_q1<<<grid_for(c.nT, Q1_WARPS), 32 * Q1_WARPS, 0, c.stream>>>(d, c.coords, c.E, c.nu, c.biot, Ke, c.Aup, c.vol,
-                                                                 c.d_flag);
+  MHFP_CUDA(cudaFuncSetAttribute(k_q1, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Q1_SMEM));
+  k_q1<<<grid_for(c.nT, Q1_CELLS), 256, Q1_SMEM, c.stream>>>(d, c.coords, c.E, c.nu, c.biot, Ke, c.Aup, c.vol,
+                                                             c.d_flag);
   MHFP_LAUNCH_CHECK();
   c.W = dalloc_n<double>(c, (size_t)36 * c.nT);
   c.W1 = dalloc_n<double>(c, (size_t)6 * c.nT);
