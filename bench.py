@@ -610,7 +610,7 @@ def run_ours(args):
 
     # roofline of the dominant sweep of the headline form
     headline_mixed = precisions[-1] == 1
-    kname = "k_cheb_u0_sym<float>" if headline_mixed else "k_cheb_u0<double>"
+    kname = "k_cheb_u0_sym<float>" if headline_mixed else "k_cheb_u0"
     avg_ms, gbs = _sweep_roofline(r32["kt"], peak)
     roofline = {"bound": "hbm", "achieved": gbs, "peak": peak, "unit": "GB/s",
                 "frac": gbs / peak if gbs else None,
@@ -635,7 +635,7 @@ def run_ours(args):
     op_tf = operator_flops(n_mesh) / (op_ms * 1e-3) / 1e12 if op["launches"] and op_ms > 0 else None
     roofline_fp64 = {"bound": "alu", "achieved": op_tf, "peak": fpk, "unit": "TFLOP/s",
                      "frac": op_tf / fpk if op_tf else None, "traffic": None,
-                     "kernel": "operator A_H x (k_apply_u + k_apply_p + k_apply_pi, FP64"
+                     "kernel": "operator A_H x (k_u64 + k_apply_p + k_apply_pi, FP64"
                                + (", FP64 form's run)" if r_op is not r32 else ")"),
                      "launches": op["launches"], "avg_launch_us": op_ms * 1e3,
                      "flops_per_launch": operator_flops(n_mesh),
@@ -671,7 +671,7 @@ def run_ours(args):
         sb64 = step_bytes(n_mesh, r64["hu"], r64["hpi"], 0, r64["restart"], int(round(statistics.mean(r64["iters"]))))
         fp64_plain = {"ms_per_step": r64["ms"], "iterations_per_step": r64["iters"], "setup_ms": r64["setup_ms"],
                       "gpu_launches": r64["launches"], "cheb_degree": r64["cheb_degree"],
-                      "sweep_roofline": {"kernel": "k_cheb_u0<double>", "bound": "alu", "achieved": t64, "peak": fpk,
+                      "sweep_roofline": {"kernel": "k_cheb_u0", "bound": "alu", "achieved": t64, "peak": fpk,
                                          "unit": "TFLOP/s", "frac": t64 / fpk if t64 else None,
                                          "hbm_achieved_gbs": g64, "avg_launch_us": a64 * 1e3},
                       "step_frac_of_hbm": sb64 / (r64["ms"] * 1e-3) / 1e9 / peak}

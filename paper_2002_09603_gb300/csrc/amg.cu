@@ -18,6 +18,7 @@
 // on the fine lattice and A_c = P^T Q per coarse point: no atomics, no
 // sparse-matrix hashing.
 #include "lattice.cuh"
+#include "u64.cuh"
 
 #include <type_traits>
 
@@ -29,67 +30,52 @@ namespace mhfp {
 namespace {
 
 // <hot:k_cheb_u0> (bench.py hashes this region to tell whether profiles/traffic.json still applies)
-// Chebyshev step: r = b - A xin (r = b when xin is null), d = cd d + cr D^-1 r,
-// xout = xin + d.
-template <int BS, int KIND, typename T>
-__device__ __forceinline__ void cheb_body(const Lat& L, const T* __restrict__ val, const T* __restrict__ dinv,
-                                          const T* __restrict__ b, const T* __restrict__ xin, T* __restrict__ xout,
-                                          T* __restrict__ d, T cd, T cr) {
-  const long long p = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (p >= L.N) return;
-  T r[BS];
+// Chebyshev step of the finest displacement level in FP64 (the rows and the
+// two forms: u64.cuh): r = b - A xin, d = cd d + cr D^-1 r, xout = xin + d.
+template <int SPLIT>
+__global__ void __launch_bounds__(SPLIT ? 9 * U64_NODES : U64_NODES_1)
+    k_cheb_u0(Lat32 L, const double* __restrict__ val, const double* __restrict__ dinv, const double* __restrict__ b,
+              const double* __restrict__ xin, double* __restrict__ xout, double* __restrict__ d, double cd, double cr,
+              long long lb) {
+  b = lane_ptr(b, lb);
+  xin = lane_ptr(xin, lb);
+  xout = lane_ptr(xout, lb);
+  d = lane_ptr(d, lb);
+  const long long N = L.N;
+  if (SPLIT) {
+    __shared__ double rs[3][U64_NODES];
+    const unsigned n = blockIdx.x * U64_NODES + threadIdx.x;
+    const int comp = threadIdx.y % 3, s = threadIdx.y / 3;
+    const bool valid = n < (unsigned)N;
+    const double v = u64_row_split(L, n, valid, comp, s, val, xin, nullptr, 0.0);
+    const long long r = 3LL * n + comp;
+    if (s == 0) rs[comp][threadIdx.x] = valid ? b[r] - v : 0.0;
+    __syncthreads();
+    if (!valid || s != 0) return;
+    double z = 0.0;
 #pragma unroll
-  for (int q = 0; q < BS; ++q) r[q] = b[BS * p + q];
-  if (xin) {
-    int i, j, k;
-    L.ijk(p, i, j, k);
-#pragma unroll 1
-    for (int o = 0; o < St<KIND>::N; ++o) {
-      int dx, dy, dz;
-      St<KIND>::off(o, dx, dy, dz);
-      if (!L.in(i + dx, j + dy, k + dz)) continue;
-      const long long q = p + dx + (long long)L.Lx * (dy + (long long)L.Ly * dz);
-      const T* v = val + (long long)o * BS * BS * L.N + p;
+    for (int t = 0; t < 3; ++t) z += dinv[(3 * comp + t) * N + n] * rs[t][threadIdx.x];
+    const double dn = (cd != 0.0) ? cd * d[r] + cr * z : cr * z;
+    d[r] = dn;
+    xout[r] = xin[r] + dn;
+  } else {
+    const unsigned n = blockIdx.x * U64_NODES_1 + threadIdx.x;
+    if (n >= (unsigned)N) return;
+    double acc[3] = {0.0, 0.0, 0.0};
+    u64_rows(L, n, val, xin, nullptr, 0.0, acc);
 #pragma unroll
-      for (int a = 0; a < BS; ++a)
+    for (int a = 0; a < 3; ++a) acc[a] = b[3LL * n + a] - acc[a];
 #pragma unroll
-        for (int s = 0; s < BS; ++s) r[a] -= v[(long long)(a * BS + s) * L.N] * xin[BS * q + s];
+    for (int a = 0; a < 3; ++a) {
+      const long long r = 3LL * n + a;
+      double z = 0.0;
+#pragma unroll
+      for (int t = 0; t < 3; ++t) z += dinv[(3 * a + t) * N + n] * acc[t];
+      const double dn = (cd != 0.0) ? cd * d[r] + cr * z : cr * z;
+      d[r] = dn;
+      xout[r] = xin[r] + dn;
     }
   }
-#pragma unroll
-  for (int a = 0; a < BS; ++a) {
-    T z = T(0);
-#pragma unroll
-    for (int s = 0; s < BS; ++s) z += dinv[(long long)(a * BS + s) * L.N + p] * r[s];
-    const T dn = (cd != T(0)) ? cd * d[BS * p + a] + cr * z : cr * z;
-    d[BS * p + a] = dn;
-    xout[BS * p + a] = (xin ? xin[BS * p + a] : T(0)) + dn;
-  }
-}
-
-template <int BS, int KIND, typename T>
-__global__ void __launch_bounds__(256) k_spmv(Lat L, const T* __restrict__ val, const T* __restrict__ x,
-                                              const T* __restrict__ b, T* __restrict__ y) {
-  spmv_body<BS, KIND, T>(L, val, x, b, y);
-}
-template <int BS, int KIND, typename T>
-__global__ void __launch_bounds__(256) k_cheb(Lat L, const T* __restrict__ val, const T* __restrict__ dinv,
-                                              const T* __restrict__ b, const T* __restrict__ xin, T* __restrict__ xout,
-                                              T* __restrict__ d, T cd, T cr) {
-  cheb_body<BS, KIND, T>(L, val, dinv, b, xin, xout, d, cd, cr);
-}
-// the finest displacement level (the dominant sweeps) under names of their own
-template <typename T>
-__global__ void __launch_bounds__(256) k_resid_u0(Lat L, const T* __restrict__ val, const T* __restrict__ x,
-                                                  const T* __restrict__ b, T* __restrict__ y, long long lb) {
-  spmv_body<3, ST_BOX1, T>(L, val, lane_ptr(x, lb), lane_ptr(b, lb), lane_ptr(y, lb));
-}
-template <typename T>
-__global__ void __launch_bounds__(256) k_cheb_u0(Lat L, const T* __restrict__ val, const T* __restrict__ dinv,
-                                                 const T* __restrict__ b, const T* __restrict__ xin,
-                                                 T* __restrict__ xout, T* __restrict__ d, T cd, T cr, long long lb) {
-  cheb_body<3, ST_BOX1, T>(L, val, dinv, lane_ptr(b, lb), lane_ptr(xin, lb), lane_ptr(xout, lb), lane_ptr(d, lb), cd,
-                           cr);
 }
 // </hot:k_cheb_u0>
 
@@ -1957,9 +1943,15 @@ void smooth(Ctx& c, std::vector<Level>& H, int l, const T* b, const T* x0, T* ds
       if constexpr (std::is_same<T, float>::value) {
         launch_cheb_sym(c, L, b, xin, out, v.d, (T)cd, (T)cr);
       } else {
-        const Lat lat = lat_of(L.A);
-        k_cheb_u0<T><<<lgrid(grid_for(lat.N, 256)), 256, 0, c.stream>>>(lat, v.val, v.dinv, b, xin, out, v.d, (T)cd,
-                                                                         (T)cr, lbytes());
+        const Lat32 lat = lat32_of(L.A);
+        if (!xin)  // the first step from zero has no stencil work
+          sweep_cheb_zero<T>(c.stream, lat.N, 3, v.dinv, b, out, v.d, (T)cr);
+        else if (lat.N <= U64_SPLIT_NODES)
+          k_cheb_u0<1><<<lgrid(grid_for(lat.N, U64_NODES)), dim3(U64_NODES, 9), 0, c.stream>>>(
+              lat, v.val, v.dinv, b, xin, out, v.d, cd, cr, lbytes());
+        else
+          k_cheb_u0<0><<<lgrid(grid_for(lat.N, U64_NODES_1)), U64_NODES_1, 0, c.stream>>>(
+              lat, v.val, v.dinv, b, xin, out, v.d, cd, cr, lbytes());
       }
     } else {
       launch_cheb<T>(c, L, v, b, xin, out, (T)cd, (T)cr, L.tpp ? L.tpp : default_schedule(L.A.N, L.bs));
@@ -1994,8 +1986,8 @@ void vcycle_level(Ctx& c, std::vector<Level>& H, int l, const T* b, T* x, bool p
     if constexpr (std::is_same<T, float>::value) {
       launch_resid_sym(c, L, s_buf, b, v.r);
     } else {
-      const Lat lat = lat_of(L.A);
-      k_resid_u0<T><<<lgrid(grid_for(lat.N, 256)), 256, 0, c.stream>>>(lat, v.val, s_buf, b, v.r, lbytes());
+      launch_u64(c.stream, lat32_of(L.A), v.val, (const double*)nullptr, 0.0, (const double*)s_buf,
+                 (const double*)nullptr, b, v.r);
       MHFP_LAUNCH_CHECK();
     }
   } else {

@@ -66,34 +66,6 @@ struct Lat {
 
 Lat lat_of(const StructOp& A) { return Lat{A.Lx, A.Ly, A.Lz, A.N}; }
 
-// ------------------------------------------------------------------ SpMV
-// y = A x (or r = b - A x) on a lattice level; thread per lattice point.
-template <int BS, int KIND, typename T>
-__device__ __forceinline__ void spmv_body(const Lat& L, const T* __restrict__ val, const T* __restrict__ x,
-                                          const T* __restrict__ b, T* __restrict__ y) {
-  const long long p = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (p >= L.N) return;
-  int i, j, k;
-  L.ijk(p, i, j, k);
-  T acc[BS];
-#pragma unroll
-  for (int r = 0; r < BS; ++r) acc[r] = T(0);
-#pragma unroll
-  for (int o = 0; o < St<KIND>::N; ++o) {
-    int dx, dy, dz;
-    St<KIND>::off(o, dx, dy, dz);
-    if (!L.in(i + dx, j + dy, k + dz)) continue;
-    const long long q = p + dx + (long long)L.Lx * (dy + (long long)L.Ly * dz);
-    const T* v = val + (long long)o * BS * BS * L.N + p;
-#pragma unroll
-    for (int r = 0; r < BS; ++r)
-#pragma unroll
-      for (int s = 0; s < BS; ++s) acc[r] += v[(long long)(r * BS + s) * L.N] * x[BS * q + s];
-  }
-#pragma unroll
-  for (int r = 0; r < BS; ++r) y[BS * p + r] = b ? b[BS * p + r] - acc[r] : acc[r];
-}
-
 // ------------------------------------------------------- lattice helpers
 // 32-bit lattice indexing for the coarse levels (see the coarse-level sweeps
 // below).
@@ -146,13 +118,6 @@ struct Sf<ST_DIAMOND2> {
   __device__ static constexpr int y(int o) { return (dia_box(o) / 5) % 5 - 2; }
   __device__ static constexpr int z(int o) { return dia_box(o) / 25 - 2; }
 };
-
-template <class F>
-void dispatch_kind(int kind, F&& f) {
-  if (kind == ST_BOX1) f(std::integral_constant<int, ST_BOX1>{});
-  else if (kind == ST_DIAMOND2) f(std::integral_constant<int, ST_DIAMOND2>{});
-  else f(std::integral_constant<int, ST_BOX2>{});
-}
 
 // block sizes of lattice levels: 1 (interface pressure), 3 (displacement),
 // 6 (coarse displacement levels with the rigid-body modes; 27-point only)
