@@ -776,7 +776,7 @@ __global__ void __launch_bounds__(256) k_dense_mv(int n, const double* __restric
   if (row < n) {
     const double* a = Ainv + (long long)row * n;
 #pragma unroll 4
-    for (int c = c0 + lane; c < c1; c += 32) s += a[c] * (double)b[c];
+    for (int c = c0 + lane; c < c1; c += 32) s += a[c] * widen(b[c]);
   }
   for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
   if (lane == 0) part[warp] = s;

@@ -46,6 +46,37 @@ inline unsigned grid_for(long long n, int block) {
   return (unsigned)(g < 1 ? 1 : g);
 }
 
+// ------------------------------------------------------------ conversions
+// FP32 <-> FP64 on the integer pipe, bit for bit what the conversion
+// instructions give.  Those run on the FP64 pipe (2 per clock and SM on
+// GB300, as an FMA), which made them the bound of kernels that only convert,
+// scale or accumulate FP32 data in FP64; the few integer operations here
+// issue at 64 per clock.  Values outside the normal FP32 range (zeros,
+// subnormals, infinities, NaN) take the instruction.
+__host__ __device__ __forceinline__ double widen(float f) {
+#ifdef __CUDA_ARCH__
+  const unsigned b = __float_as_uint(f);
+  if (((b >> 23) & 255u) - 1u < 254u)
+    return __hiloint2double((int)((b & 0x80000000u) | (((b & 0x7fffffffu) >> 3) + (896u << 20))), (int)(b << 29));
+#endif
+  return (double)f;
+}
+__host__ __device__ __forceinline__ double widen(double d) { return d; }
+__host__ __device__ __forceinline__ float narrow(double d) {
+#ifdef __CUDA_ARCH__
+  const unsigned hi = (unsigned)__double2hiint(d), lo = (unsigned)__double2loint(d);
+  if (((hi >> 20) & 2047u) - 897u < 254u) {
+    // truncated FP32 bits, then round to nearest even on the 29 bits dropped
+    // (a carry runs into the exponent, up to infinity, as it should)
+    unsigned f = (((hi & 0x7fffffffu) - (896u << 20)) << 3) | (lo >> 29);
+    const unsigned rem = lo & 0x1fffffffu;
+    f += (rem > 0x10000000u || (rem == 0x10000000u && (f & 1u))) ? 1u : 0u;
+    return __uint_as_float(f | (hi & 0x80000000u));
+  }
+#endif
+  return (float)d;
+}
+
 // ------------------------------------------------------------ lanes
 // Several right-hand sides of one handle solved in lockstep ("lanes"): every
 // kernel of the solve runs once for all of them, lane l in blockIdx.z.  A

@@ -6,6 +6,7 @@
 // estimate per iteration.
 #include "common.cuh"
 
+#include <algorithm>
 #include <chrono>
 #include <cmath>
 
@@ -75,24 +76,56 @@ __device__ __forceinline__ void gs_rows(long long n, const double* __restrict__ 
   }
 }
 
-__global__ void __launch_bounds__(RED_THREADS, 4) k_gs_dots(long long n, const double* __restrict__ V, int ncols,
+// The blocks of a reduction meet on a counter: every block publishes its
+// partial sums, and the last one to arrive reduces them all in a fixed order
+// (no block waits) and rearms the counter.  Saves the separate reduction
+// kernels: a launch and 3 us each.
+__device__ __forceinline__ bool last_block(unsigned* counter, unsigned nblocks) {
+  __shared__ bool last;
+  __threadfence();
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    last = atomicAdd(counter, 1u) == nblocks - 1;
+    if (last) *counter = 0u;
+  }
+  __syncthreads();
+  if (last) __threadfence();
+  return last;
+}
+
+// sum of p[0..nb) by one warp in a fixed order; every lane returns it
+__device__ __forceinline__ double warp_sum_of(const double* p, int nb) {
+  double v = 0.0;
+  for (int b = threadIdx.x & 31; b < nb; b += 32) v += __ldcg(p + b);
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  return v;
+}
+
+// hout[c] = V[:, c] . w for the columns c <= j, eight per block row
+// (blockIdx.y), and *nrm2 = w . w when given.  Nothing happens when *skip.
+__global__ void __launch_bounds__(RED_THREADS, 4) k_gs_dots(long long n, const double* __restrict__ V, int j,
                                                              const double* __restrict__ w,
-                                                             double* __restrict__ partials,
-                                                             const int* __restrict__ skip, int with_norm,
-                                                             long long lb) {
+                                                             double* __restrict__ partials, double* __restrict__ hout,
+                                                             double* __restrict__ nrm2,
+                                                             const int* __restrict__ skip,
+                                                             unsigned* __restrict__ counters, long long lb) {
   static_assert(GS_COLS == 8, "warp_sum8 reduces eight columns");
   V = lane_ptr(V, lb);
   w = lane_ptr(w, lb);
   partials = lane_ptr(partials, lb);
+  hout = lane_ptr(hout, lb);
+  nrm2 = lane_ptr(nrm2, lb);
   skip = lane_ptr(skip, lb);
-  if (skip && *skip) return;
+  counters = lane_ptr(counters, lb);
+  const int ncols = j + 1, c0 = blockIdx.y * GS_COLS;
+  if (c0 >= ncols || (skip && *skip)) return;
   __shared__ double sh[RED_THREADS / 32][GS_COLS];
   __shared__ double shn[RED_THREADS / 32];
-  const int c0 = blockIdx.y * GS_COLS;
-  const bool do_norm = with_norm && blockIdx.y == 0;
+  const bool do_norm = nrm2 != nullptr && blockIdx.y == 0;
   double acc[GS_COLS] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0}, nw = 0.0;
+  const int nc = ncols - c0 < GS_COLS ? ncols - c0 : GS_COLS;
   // block-uniform branch on the number of valid columns in this group
-  switch ((ncols - c0 < GS_COLS ? ncols - c0 : GS_COLS) + (do_norm ? 16 : 0)) {
+  switch (nc + (do_norm ? 16 : 0)) {
     case 1: gs_rows<1, false>(n, V, c0, w, acc, nw); break;
     case 2: gs_rows<2, false>(n, V, c0, w, acc, nw); break;
     case 3: gs_rows<3, false>(n, V, c0, w, acc, nw); break;
@@ -119,38 +152,25 @@ __global__ void __launch_bounds__(RED_THREADS, 4) k_gs_dots(long long n, const d
     if (lane == 0) shn[wid] = nw;
   }
   __syncthreads();
-  if (threadIdx.x < GS_COLS && c0 + (int)threadIdx.x < ncols) {
+  const int nb = gridDim.x;
+  if ((int)threadIdx.x < nc) {
     double s = 0.0;
     for (int k = 0; k < RED_THREADS / 32; ++k) s += sh[k][threadIdx.x];
-    partials[(long long)(c0 + threadIdx.x) * gridDim.x + blockIdx.x] = s;
+    partials[(long long)(c0 + threadIdx.x) * nb + blockIdx.x] = s;
   }
   if (do_norm && threadIdx.x == 32) {
     double s = 0.0;
     for (int k = 0; k < RED_THREADS / 32; ++k) s += shn[k];
-    partials[(long long)ncols * gridDim.x + blockIdx.x] = s;
+    partials[(long long)ncols * nb + blockIdx.x] = s;
   }
-}
-
-// same reduction, skipped when *skip != 0
-__global__ void k_reduce_partials_flag(int nb, const double* __restrict__ partials, double* __restrict__ out,
-                                       const int* __restrict__ skip, long long lb);
-
-
-// out[col] (+)= sum_b partials[col * nb + b] in a fixed order
-// the ncols dot products into hout[0..ncols) and, when nrm2 is given, the
-// norm partials (row ncols) into *nrm2; same fixed-order sums as below
-__global__ void k_reduce_dots(int nb, const double* __restrict__ partials, double* __restrict__ hout, int ncols,
-                              double* __restrict__ nrm2, long long lb) {
-  partials = lane_ptr(partials, lb);
-  hout = lane_ptr(hout, lb);
-  nrm2 = lane_ptr(nrm2, lb);
-  __shared__ double sh[RED_THREADS / 32];
-  double v = 0.0;
-  for (int b = threadIdx.x; b < nb; b += blockDim.x) v += partials[(long long)blockIdx.x * nb + b];
-  const double s = block_sum(v, sh);
-  if (threadIdx.x == 0) {
-    if ((int)blockIdx.x < ncols) hout[blockIdx.x] = s;
-    else *nrm2 = s;
+  if (!last_block(counters + blockIdx.y, nb)) return;
+  for (int q = wid; q < nc + (do_norm ? 1 : 0); q += RED_THREADS / 32) {
+    const int c = q < nc ? c0 + q : ncols;  // the norm's partials are row ncols
+    const double s = warp_sum_of(partials + (long long)c * nb, nb);
+    if (lane == 0) {
+      if (q < nc) hout[c] = s;
+      else *nrm2 = s;
+    }
   }
 }
 
@@ -165,32 +185,116 @@ __global__ void k_reduce_partials(int nb, const double* __restrict__ partials, d
   if (threadIdx.x == 0) out[blockIdx.x] = accumulate ? out[blockIdx.x] + s : s;
 }
 
-__global__ void k_reduce_partials_flag(int nb, const double* __restrict__ partials, double* __restrict__ out,
-                                       const int* __restrict__ skip, long long lb) {
-  partials = lane_ptr(partials, lb);
-  out = lane_ptr(out, lb);
-  skip = lane_ptr(skip, lb);
-  if (*skip) return;
-  __shared__ double sh[RED_THREADS / 32];
-  double v = 0.0;
-  for (int b = threadIdx.x; b < nb; b += blockDim.x) v += partials[(long long)blockIdx.x * nb + b];
-  const double s = block_sum(v, sh);
-  if (threadIdx.x == 0) out[blockIdx.x] = s;
+// What the last block of k_gemv_sub does with ||w||^2: the DGKS test after a
+// first pass, or the Hessenberg column and its Givens rotation after the last.
+//
+// DGKS test (Daniel, Gragg, Kaufman & Stewart, 1976): after one classical
+// Gram-Schmidt projection, reorthogonalise only if the norm fell below
+// 1/sqrt(2) of its value before the projection (nrm0 = ||w||^2 before).
+// flag = 1 means "skip the second projection": then h2 is zero and the norm
+// after the first pass is the final one.
+struct GsTail {
+  int givens;               // 0: DGKS test, 1: Givens
+  const double* nrm0;       // DGKS: ||w||^2 before
+  int* flag;                // DGKS: decision
+  double* h2;               // second pass's coefficients (null: none)
+  double* nrm2;             // the final ||w||^2
+  const double* h1;         // Givens: first pass's coefficients
+  double *H, *cs, *sn, *g, *scal;
+  int m;
+  __device__ __forceinline__ GsTail lane(long long lb) const {
+    return {givens, lane_ptr(nrm0, lb), lane_ptr(flag, lb), lane_ptr(h2, lb), lane_ptr(nrm2, lb), lane_ptr(h1, lb),
+            lane_ptr(H, lb), lane_ptr(cs, lb), lane_ptr(sn, lb), lane_ptr(g, lb), lane_ptr(scal, lb), m};
+  }
+};
+
+// One Arnoldi step's Hessenberg column, by one warp: h = h1 + h2 (j+1
+// entries; h2 null after a single Gram-Schmidt pass), the new subdiagonal
+// ||w|| = sqrt(nrm2); apply the previous rotations, make the new one, update
+// g.  scal[0] = |g_{j+1}|, scal[1] = 1/||w|| (0 on breakdown).  The operands
+// are loaded by the whole warp first: the recurrence itself (2 FP64 steps
+// per rotation) then runs from shared memory.
+__device__ __forceinline__ void givens_step(int j, const GsTail& t, double nrm2) {
+  __shared__ double col[64], c_[64], s_[64];
+  const int lane = threadIdx.x & 31;
+  for (int i = lane; i <= j; i += 32) {
+    col[i] = t.h2 ? t.h1[i] + t.h2[i] : t.h1[i];
+    if (i < j) {
+      c_[i] = t.cs[i];
+      s_[i] = t.sn[i];
+    }
+  }
+  const double gj = t.g[j];
+  __syncwarp();
+  if (lane == 0) {
+    const double hn = sqrt(nrm2);
+    double a = col[0];
+    for (int i = 0; i < j; ++i) {
+      const double b = col[i + 1];
+      col[i] = c_[i] * a + s_[i] * b;
+      a = -s_[i] * a + c_[i] * b;
+    }
+    const double den = hypot(a, hn);
+    const double c = den > 0.0 ? a / den : 1.0;
+    const double s = den > 0.0 ? hn / den : 0.0;
+    t.cs[j] = c;
+    t.sn[j] = s;
+    col[j] = den;
+    t.g[j + 1] = -s * gj;
+    t.g[j] = c * gj;
+    t.scal[0] = fabs(s * gj);
+    t.scal[1] = hn > 0.0 ? 1.0 / hn : 0.0;
+  }
+  __syncwarp();
+  double* out = t.H + (long long)j * (t.m + 1);
+  for (int i = lane; i <= j; i += 32) out[i] = col[i];
+  if (lane == 0) out[j + 1] = 0.0;
 }
 
-// w -= V h as one FMA chain per row, two rows per thread for independent
-// chains (ncols + 1 FP64 operations per row, the norm included); partial
-// sums of the updated w . w into partials[block] when partials is given
-__global__ void __launch_bounds__(RED_THREADS, 8) k_gemv_sub(long long n, const double* __restrict__ V, int ncols,
+// rows r, r + stride (NR = 2) or r alone (NR = 1): v -= V h, four columns'
+// loads in flight per row
+template <int NR>
+__device__ __forceinline__ void sub_rows(long long n, const double* __restrict__ V, int ncols, const double* nh,
+                                         long long r, long long stride, double (&v)[NR]) {
+#pragma unroll 1
+  for (int c = 0; c < ncols; c += 4) {
+    double x[4][NR];
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+      if (c + u < ncols)
+#pragma unroll
+        for (int q = 0; q < NR; ++q) x[u][q] = V[(long long)(c + u) * n + r + q * stride];
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+      if (c + u < ncols)
+#pragma unroll
+        for (int q = 0; q < NR; ++q) v[q] = fma(x[u][q], nh[c + u], v[q]);
+  }
+}
+
+// w -= V h over the columns c <= j, one FMA chain per row (ncols + 1 FP64
+// operations per row, the norm included; at 15 M rows the FP64 pipe bounds
+// it), then the tail on the norm of the updated w.  When *skip only the tail
+// runs, on the norm that is already there.
+__global__ void __launch_bounds__(RED_THREADS, 4) k_gemv_sub(long long n, const double* __restrict__ V, int j,
                                                               const double* __restrict__ h, double* __restrict__ w,
                                                               double* __restrict__ partials,
-                                                              const int* __restrict__ skip, long long lb) {
+                                                              const int* __restrict__ skip,
+                                                              unsigned* __restrict__ counter, GsTail t, long long lb) {
   V = lane_ptr(V, lb);
   h = lane_ptr(h, lb);
   w = lane_ptr(w, lb);
   partials = lane_ptr(partials, lb);
   skip = lane_ptr(skip, lb);
-  if (skip && *skip) return;
+  counter = lane_ptr(counter, lb);
+  const int ncols = j + 1;
+  if (skip && *skip) {
+    if (blockIdx.x == 0 && threadIdx.x < 32) {
+      t = t.lane(lb);
+      givens_step(j, t, *t.nrm2);
+    }
+    return;
+  }
   __shared__ double sh[RED_THREADS / 32];
   __shared__ double nh[64];
   for (int c = threadIdx.x; c < ncols; c += blockDim.x) nh[c] = -h[c];
@@ -198,25 +302,36 @@ __global__ void __launch_bounds__(RED_THREADS, 8) k_gemv_sub(long long n, const 
   double acc = 0.0;
   const long long stride = (long long)gridDim.x * blockDim.x;
   for (long long r = (long long)blockIdx.x * blockDim.x + threadIdx.x; r < n; r += 2 * stride) {
-    const long long r1 = r + stride;
-    const bool two = r1 < n;
-    double v0 = w[r], v1 = two ? w[r1] : 0.0;
-#pragma unroll 2
-    for (int c = 0; c < ncols; ++c) {
-      const double* col = V + (long long)c * n;
-      v0 = fma(col[r], nh[c], v0);
-      if (two) v1 = fma(col[r1], nh[c], v1);
-    }
-    w[r] = v0;
-    acc = fma(v0, v0, acc);
-    if (two) {
-      w[r1] = v1;
-      acc = fma(v1, v1, acc);
+    if (r + stride < n) {
+      double v[2] = {w[r], w[r + stride]};
+      sub_rows<2>(n, V, ncols, nh, r, stride, v);
+      w[r] = v[0];
+      w[r + stride] = v[1];
+      acc = fma(v[0], v[0], acc);
+      acc = fma(v[1], v[1], acc);
+    } else {
+      double v[1] = {w[r]};
+      sub_rows<1>(n, V, ncols, nh, r, stride, v);
+      w[r] = v[0];
+      acc = fma(v[0], v[0], acc);
     }
   }
-  if (partials) {
-    const double t = block_sum(acc, sh);
-    if (threadIdx.x == 0) partials[blockIdx.x] = t;
+  const double p = block_sum(acc, sh);
+  if (threadIdx.x == 0) partials[blockIdx.x] = p;
+  if (!last_block(counter, gridDim.x) || threadIdx.x >= 32) return;
+  t = t.lane(lb);
+  const double nrm = warp_sum_of(partials, gridDim.x);
+  if (t.givens) {
+    if (threadIdx.x == 0) *t.nrm2 = nrm;
+    givens_step(j, t, nrm);
+  } else {
+    const bool enough = nrm > 0.5 * t.nrm0[0];
+    if (threadIdx.x == 0) {
+      *t.flag = enough ? 1 : 0;
+      if (enough) *t.nrm2 = nrm;
+    }
+    if (enough)
+      for (int c = threadIdx.x; c < ncols; c += 32) t.h2[c] = 0.0;
   }
 }
 
@@ -232,39 +347,51 @@ __global__ void __launch_bounds__(RED_THREADS) k_norm_partials(long long n, cons
   if (threadIdx.x == 0) partials[blockIdx.x] = t;
 }
 
+// x_r + sum_c Z[r, c] y_c for c < k, four columns' loads in flight.  With an
+// FP32 Z every product is exact in FP64 (the same sums as with the widened
+// columns); widen() keeps the conversions off the FP64 pipe.
+template <typename ZT>
+__device__ __forceinline__ double gemv_row(long long r, long long ld, const ZT* __restrict__ Z, int k,
+                                           const double* __restrict__ y, double s) {
+#pragma unroll 1
+  for (int c = 0; c < k; c += 4) {
+    ZT z[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+      if (c + u < k) z[u] = Z[(long long)(c + u) * ld + r];
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+      if (c + u < k) s += widen(z[u]) * y[c + u];
+  }
+  return s;
+}
+
 // x += Z y
-// x += Z y with an FP32 Z (every product exact in FP64, the same sums as
-// with the widened columns)
-__global__ void k_gemv_add_f(long long n, long long ld, const float* __restrict__ Z, int ncols,
-                             const double* __restrict__ y, double* __restrict__ x) {
+template <typename ZT>
+__global__ void k_gemv_add(long long n, long long ld, const ZT* __restrict__ Z, int ncols,
+                           const double* __restrict__ y, double* __restrict__ x) {
   const long long r = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (r >= n) return;
-  double s = x[r];
-  for (int c = 0; c < ncols; ++c) s += (double)Z[(long long)c * ld + r] * y[c];
-  x[r] = s;
+  if (r < n) x[r] = gemv_row(r, ld, Z, ncols, y, x[r]);
 }
 
-__global__ void k_gemv_add(long long n, const double* __restrict__ Z, int ncols, const double* __restrict__ y,
-                           double* __restrict__ x) {
-  const long long r = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (r >= n) return;
-  double s = x[r];
-  for (int c = 0; c < ncols; ++c) s += Z[(long long)c * n + r] * y[c];
-  x[r] = s;
-}
-
-__global__ void k_scale_dev(long long n, const double* __restrict__ x, const double* __restrict__ s,
-                            double* __restrict__ y, long long lb) {
+// The next basis vector and the preconditioner's input from it: v = x s and
+// t = v mul (FP64, or rounded to FP32 in the mixed form), in one pass.  s is
+// s_dev[0], or s_host when s_dev is null; mul is the shared unscaling D_s^-1.
+template <typename T>
+__global__ void k_next_basis(long long n, const double* __restrict__ x, const double* __restrict__ s_dev,
+                             double s_host, const double* __restrict__ mul, double* __restrict__ v,
+                             T* __restrict__ t, long long lb) {
   x = lane_ptr(x, lb);
-  s = lane_ptr(s, lb);
-  y = lane_ptr(y, lb);
+  s_dev = lane_ptr(s_dev, lb);
+  v = lane_ptr(v, lb);
+  t = lane_ptr(t, lb);
   const long long r = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (r < n) y[r] = x[r] * s[0];
-}
-
-__global__ void k_scale_host(long long n, const double* __restrict__ x, double s, double* __restrict__ y) {
-  const long long r = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (r < n) y[r] = x[r] * s;
+  if (r >= n) return;
+  const double vr = x[r] * (s_dev ? s_dev[0] : s_host);
+  v[r] = vr;
+  const double tr = vr * mul[r];
+  if constexpr (sizeof(T) == 4) t[r] = narrow(tr);
+  else t[r] = tr;
 }
 
 // s is a shared elementwise scaling (not a work vector)
@@ -276,75 +403,38 @@ __global__ void k_ewise(long long n, const double* __restrict__ x, const double*
   if (r < n) y[r] = divide ? x[r] / s[r] : x[r] * s[r];
 }
 
-// DGKS test (Daniel, Gragg, Kaufman & Stewart, 1976): after one classical
-// Gram-Schmidt projection, reorthogonalise only if the norm fell below
-// 1/sqrt(2) of its value before the projection.  nrm[0] = ||w||^2 before,
-// nrm[1] = ||w||^2 after.  flag = 1 means "skip the second projection";
-// when it is skipped h2 is zeroed and the norm after the first pass is
-// carried into nrm[2], which the second pass overwrites otherwise.
-__global__ void k_dgks(int ncols, const double* __restrict__ nrm, int* __restrict__ flag, double* __restrict__ h2,
-                       double* __restrict__ nrm_final, long long lb) {
-  nrm = lane_ptr(nrm, lb);
-  flag = lane_ptr(flag, lb);
-  h2 = lane_ptr(h2, lb);
-  nrm_final = lane_ptr(nrm_final, lb);
-  const int i = threadIdx.x;
-  const bool skip = nrm[1] > 0.5 * nrm[0];
-  if (i == 0) {
-    *flag = skip ? 1 : 0;
-    if (skip) nrm_final[0] = nrm[1];
-  }
-  if (skip)
-    for (int c = i; c < ncols; c += blockDim.x) h2[c] = 0.0;
-}
-
-// One Arnoldi step's Hessenberg column: h = h1 + h2 (j+1 entries; h2 null
-// after a single Gram-Schmidt pass), the new
-// subdiagonal ||w|| = sqrt(nrm2); apply the previous rotations, make the new
-// one, update g.  scal[0] = |g_{j+1}|, scal[1] = 1/||w|| (0 on breakdown).
-__global__ void k_givens(int j, int m, const double* __restrict__ h1, const double* __restrict__ h2,
-                         const double* __restrict__ nrm2, double* __restrict__ H, double* __restrict__ cs,
-                         double* __restrict__ sn, double* __restrict__ g, double* __restrict__ scal, long long lb) {
-  if (threadIdx.x != 0 || blockIdx.x != 0) return;
-  h1 = lane_ptr(h1, lb);
-  h2 = lane_ptr(h2, lb);
-  nrm2 = lane_ptr(nrm2, lb);
-  H = lane_ptr(H, lb);
-  cs = lane_ptr(cs, lb);
-  sn = lane_ptr(sn, lb);
-  g = lane_ptr(g, lb);
-  scal = lane_ptr(scal, lb);
-  double* col = H + (long long)j * (m + 1);
-  for (int i = 0; i <= j; ++i) col[i] = h2 ? h1[i] + h2[i] : h1[i];
-  const double hn = sqrt(nrm2[0]);
-  col[j + 1] = hn;
-  for (int i = 0; i < j; ++i) {
-    const double t = cs[i] * col[i] + sn[i] * col[i + 1];
-    col[i + 1] = -sn[i] * col[i] + cs[i] * col[i + 1];
-    col[i] = t;
-  }
-  const double den = hypot(col[j], col[j + 1]);
-  const double c = den > 0.0 ? col[j] / den : 1.0;
-  const double s = den > 0.0 ? col[j + 1] / den : 0.0;
-  cs[j] = c;
-  sn[j] = s;
-  col[j] = den;
-  col[j + 1] = 0.0;
-  g[j + 1] = -s * g[j];
-  g[j] = c * g[j];
-  scal[0] = fabs(g[j + 1]);
-  scal[1] = hn > 0.0 ? 1.0 / hn : 0.0;
-}
-
-// back substitution R y = g (k x k upper triangle of the rotated H)
-__global__ void k_lsq(int k, int m, const double* __restrict__ H, const double* __restrict__ g, double* __restrict__ y) {
-  if (threadIdx.x != 0 || blockIdx.x != 0) return;
+// back substitution R y = g (k x k upper triangle of the rotated H) by one
+// warp, k <= 64: each lane keeps two entries of the right-hand side, column i
+// is loaded while y_i's predecessor is applied (20-55 us in one thread for
+// k = 15-50 before)
+__device__ __forceinline__ void back_substitute(int k, int m, const double* __restrict__ H,
+                                                const double* __restrict__ g, double* __restrict__ y) {
+  const int lane = threadIdx.x & 31, l2 = lane + 32;
+  double r0 = lane < k ? g[lane] : 0.0, r1 = l2 < k ? g[l2] : 0.0;
+  const double d0 = lane < k ? H[(long long)lane * (m + 1) + lane] : 1.0;
+  const double d1 = l2 < k ? H[(long long)l2 * (m + 1) + l2] : 1.0;
+  const double* col = H + (long long)(k - 1) * (m + 1);
+  double c0 = lane < k - 1 ? col[lane] : 0.0, c1 = l2 < k - 1 ? col[l2] : 0.0;
   for (int i = k - 1; i >= 0; --i) {
-    double s = g[i];
-    for (int c = i + 1; c < k; ++c) s -= H[(long long)c * (m + 1) + i] * y[c];
-    const double d = H[(long long)i * (m + 1) + i];
-    y[i] = d != 0.0 ? s / d : 0.0;
+    double n0 = 0.0, n1 = 0.0;
+    if (i > 0) {
+      col = H + (long long)(i - 1) * (m + 1);
+      n0 = lane < i - 1 ? col[lane] : 0.0;
+      n1 = l2 < i - 1 ? col[l2] : 0.0;
+    }
+    const double rhs = __shfl_sync(0xffffffffu, i < 32 ? r0 : r1, i & 31);
+    const double d = __shfl_sync(0xffffffffu, i < 32 ? d0 : d1, i & 31);
+    const double yi = d != 0.0 ? rhs / d : 0.0;
+    if (lane == 0) y[i] = yi;
+    if (lane < i) r0 = fma(-c0, yi, r0);
+    if (l2 < i) r1 = fma(-c1, yi, r1);
+    c0 = n0;
+    c1 = n1;
   }
+}
+
+__global__ void k_lsq(int k, int m, const double* __restrict__ H, const double* __restrict__ g, double* __restrict__ y) {
+  back_substitute(k, m, H, g, y);
 }
 
 __global__ void k_set_g(int m, double beta, double* __restrict__ g) {
@@ -353,18 +443,23 @@ __global__ void k_set_g(int m, double beta, double* __restrict__ g) {
 }
 
 
-// hout[0..ncols) = V^T w; with nrm2 non-null also ||w||^2 into nrm2[0];
+// blocks of the Gram-Schmidt kernels: no more than the rows fill
+inline unsigned gs_blocks(long long n, int most) { return std::min<unsigned>(grid_for(n, RED_THREADS), (unsigned)most); }
+
+// hout[0..j] = V^T w; with nrm2 non-null also ||w||^2 into nrm2[0];
 // with skip non-null nothing happens when *skip != 0
-void gs_dots(Ctx& c, int ncols, double* hout, double* nrm2, const int* skip) {
-  const int wn = nrm2 ? 1 : 0;
-  const dim3 grid = lgrid(GS_DOT_BLOCKS, (ncols + GS_COLS - 1) / GS_COLS);
-  k_gs_dots<<<grid, RED_THREADS, 0, c.stream>>>(c.n, c.V, ncols, c.w, c.partials, skip, wn, lbytes());
+void gs_dots(Ctx& c, int j, double* hout, double* nrm2, const int* skip) {
+  const dim3 grid = lgrid(gs_blocks(c.n, GS_DOT_BLOCKS), j / GS_COLS + 1);
+  k_gs_dots<<<grid, RED_THREADS, 0, c.stream>>>(c.n, c.V, j, c.w, c.partials, hout, nrm2, skip,
+                                                (unsigned*)(c.dflag + 2), lbytes());
   MHFP_LAUNCH_CHECK();
-  if (skip) {
-    k_reduce_partials_flag<<<lgrid(ncols), RED_THREADS, 0, c.stream>>>(GS_DOT_BLOCKS, c.partials, hout, skip, lbytes());
-  } else {
-    k_reduce_dots<<<lgrid(ncols + wn), RED_THREADS, 0, c.stream>>>(GS_DOT_BLOCKS, c.partials, hout, ncols, nrm2, lbytes());
-  }
+}
+
+// w -= V h, then the tail t (see GsTail)
+void gs_sub(Ctx& c, int j, const double* h, const int* skip, const GsTail& t) {
+  k_gemv_sub<<<lgrid(gs_blocks(c.n, GS_BLOCKS)), RED_THREADS, 0, c.stream>>>(
+      c.n, c.V, j, h, c.w, c.partials + (size_t)c.opt.restart * GS_BLOCKS, skip, (unsigned*)(c.dflag + 1), t,
+      lbytes());
   MHFP_LAUNCH_CHECK();
 }
 
@@ -401,7 +496,8 @@ void ensure_workspace(Ctx& c) {
   c.npart = GS_BLOCKS;
   c.partials = dalloc_n<double>(c, (size_t)(m + 2) * GS_BLOCKS);
   c.scal = dalloc_n<double>(c, 8);
-  c.dflag = dalloc_n<int>(c, 4);
+  c.dflag = dalloc_n<int>(c, 16);  // DGKS flag, then the Gram-Schmidt kernels' block counters
+  MHFP_CUDA(cudaMemsetAsync(c.dflag, 0, 16 * sizeof(int), c.stream));
   if (!c.host_scal) MHFP_CUDA(cudaMallocHost(&c.host_scal, 8 * sizeof(double)));
   c.m_alloc = m;
 }
@@ -432,18 +528,16 @@ void vec_scale(Ctx& c, const double* x, const double* s, bool divide, double* y,
   MHFP_LAUNCH_CHECK();
 }
 
-// mul is a shared elementwise scaling (not a work vector)
-__global__ void k_to_f32(long long n, const double* __restrict__ x, const double* __restrict__ mul,
-                         float* __restrict__ y, long long lb) {
+__global__ void k_to_f32(long long n, const double* __restrict__ x, float* __restrict__ y, long long lb) {
   x = lane_ptr(x, lb);
   y = lane_ptr(y, lb);
   const long long r = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (r < n) y[r] = (float)(mul ? x[r] * mul[r] : x[r]);
+  if (r < n) y[r] = narrow(x[r]);
 }
 
 __global__ void k_to_f64(long long n, const float* __restrict__ x, double* __restrict__ y) {
   const long long r = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (r < n) y[r] = (double)x[r];
+  if (r < n) y[r] = widen(x[r]);
 }
 
 // Back substitution with M (Eq. hybridPrec): pi, then p, then u; or, for the
@@ -471,16 +565,18 @@ void precond_blocks(Ctx& c, const T* t, T* z, T* work_u, T* work_pi, bool transp
   }
 }
 
-// z = M^-1 (v .* mul) (or M^-T) with the FP32 V-cycles and Schur steps; v
-// FP64; the FP32 result in zf_out (default: the handle's FP32 work vector)
-// and, when z is given, widened into z
-void apply_precond_mixed(Ctx& c, const double* v, const double* mul, double* z, bool transpose,
-                         float* zf_out = nullptr) {
+// z = M^-1 v (or M^-T) with the FP32 V-cycles and Schur steps: v FP64, or,
+// when null, already rounded in the handle's FP32 vector c.tf; the FP32
+// result in zf_out (default: the handle's FP32 work vector) and, when z is
+// given, widened into z
+void apply_precond_mixed(Ctx& c, const double* v, double* z, bool transpose, float* zf_out = nullptr) {
   const long long n = c.n;
   float* zo = zf_out ? zf_out : c.zf;
   timing_begin(c, 3);
-  k_to_f32<<<lgrid(grid_for(n, 256)), 256, 0, c.stream>>>(n, v, mul, c.tf, lbytes());
-  MHFP_LAUNCH_CHECK();
+  if (v) {
+    k_to_f32<<<lgrid(grid_for(n, 256)), 256, 0, c.stream>>>(n, v, c.tf, lbytes());
+    MHFP_LAUNCH_CHECK();
+  }
   // level-0 right-hand-side buffers are free at the finest levels
   precond_blocks<float>(c, c.tf, zo, c.hu[0].bf, c.hpi[0].bf, transpose);
   if (z) {
@@ -516,7 +612,7 @@ void apply_precond(Ctx& c, const double* v, double* z, bool transpose) {
     return;
   }
   if (c.opt.precision == 1) {
-    apply_precond_mixed(c, v, nullptr, z, transpose);
+    apply_precond_mixed(c, v, z, transpose);
     return;
   }
   timing_begin(c, 3);
@@ -524,26 +620,35 @@ void apply_precond(Ctx& c, const double* v, double* z, bool transpose) {
   timing_end(c, 3, 0.0);
 }
 
-// Enqueue Arnoldi step j: z_j = M^-1 v_j, w = D_s A z_j, Gram-Schmidt, the
+// basis vector `col` from x: V[:, col] = x s and the preconditioner's input
+// D_s^-1 V[:, col] in c.tf (FP32 form) or c.t
+void enqueue_next_basis(Ctx& c, int col, const double* x, const double* s_dev, double s_host = 0.0) {
+  const long long n = c.n;
+  double* v = c.V + (long long)col * n;
+  const dim3 grid = lgrid(grid_for(n, 256));
+  if (c.opt.precision == 1)
+    k_next_basis<float><<<grid, 256, 0, c.stream>>>(n, x, s_dev, s_host, c.ds_inv, v, c.tf, lbytes());
+  else
+    k_next_basis<double><<<grid, 256, 0, c.stream>>>(n, x, s_dev, s_host, c.ds_inv, v, c.t, lbytes());
+  MHFP_LAUNCH_CHECK();
+}
+
+// Enqueue Arnoldi step j (V[:, j] and the preconditioner's input are there,
+// enqueue_next_basis): z_j = M^-1 v_j, w = D_s A z_j, Gram-Schmidt with the
 // Givens update, v_{j+1}, and the copy of |g_{j+1}| to pinned host memory.
 void enqueue_arnoldi_step(Ctx& c, int j, bool transpose, bool host_copy = true) {
   const int m = c.opt.restart;
   const long long n = c.n;
-  double* vj = c.V + (long long)j * n;
   if (ff_krylov(c)) {
     // z_j stays in FP32 (it is the FP32 preconditioner's output): the
     // float-float operator reads it, and x += Z y widens it
     float* zfj = c.Zf + (long long)j * c.ldz;
-    apply_precond_mixed(c, vj, c.ds_inv, nullptr, transpose, zfj);  // unscale into the FP32 preconditioner
+    apply_precond_mixed(c, nullptr, nullptr, transpose, zfj);
     apply_operator_arnoldi(c, nullptr, zfj, c.w, c.ds, transpose);  // w = D_s A z_j
   } else {
     double* zj = c.Z + (long long)j * n;
-    if (c.opt.precision == 1) {
-      apply_precond_mixed(c, vj, c.ds_inv, zj, transpose);  // unscale into the FP32 preconditioner
-    } else {
-      vec_scale(c, vj, c.ds_inv, false, c.t, n);  // unscale into the preconditioner
-      apply_precond(c, c.t, zj, transpose);
-    }
+    if (c.opt.precision == 1) apply_precond_mixed(c, nullptr, zj, transpose);
+    else apply_precond(c, c.t, zj, transpose);
     apply_operator_arnoldi(c, zj, c.zf, c.w, c.ds, transpose);  // w = D_s A z_j
   }
   timing_begin(c, 2);
@@ -552,31 +657,29 @@ void enqueue_arnoldi_step(Ctx& c, int j, bool transpose, bool host_copy = true) 
   // norm dropped by more than 1/sqrt(2), h2 = V^T w and w -= V h2
   // (reorth = 0: the first pass alone, the second is not even queued)
   const bool reorth = c.opt.reorth != 0;
-  gs_dots(c, j + 1, c.h, c.scal + 4, nullptr);
-  k_gemv_sub<<<lgrid(GS_BLOCKS), RED_THREADS, 0, c.stream>>>(n, c.V, j + 1, c.h, c.w, c.partials + (size_t)m * GS_BLOCKS,
-                                                     nullptr, lbytes());
-  MHFP_LAUNCH_CHECK();
-  // one pass: the new norm goes straight to the slot the Givens step reads
-  k_reduce_partials<<<lgrid(1), RED_THREADS, 0, c.stream>>>(GS_BLOCKS, c.partials + (size_t)m * GS_BLOCKS,
-                                                     reorth ? c.scal + 5 : c.scal + 2, 0, lbytes());
-  MHFP_LAUNCH_CHECK();
+  double* h2 = c.h + (m + 1);
+  GsTail tail{};
+  tail.nrm0 = c.scal + 4;
+  tail.flag = c.dflag;
+  tail.h2 = reorth ? h2 : nullptr;
+  tail.nrm2 = c.scal + 2;
+  tail.h1 = c.h;
+  tail.H = c.H;
+  tail.cs = c.cs;
+  tail.sn = c.sn;
+  tail.g = c.g;
+  tail.scal = c.scal;
+  tail.m = m;
+  tail.givens = reorth ? 0 : 1;
+  gs_dots(c, j, c.h, reorth ? c.scal + 4 : nullptr, nullptr);
+  gs_sub(c, j, c.h, nullptr, tail);
   if (reorth) {
-    k_dgks<<<lgrid(1), 64, 0, c.stream>>>(j + 1, c.scal + 4, c.dflag, c.h + (m + 1), c.scal + 2, lbytes());
-    MHFP_LAUNCH_CHECK();
-    gs_dots(c, j + 1, c.h + (m + 1), nullptr, c.dflag);
-    k_gemv_sub<<<lgrid(GS_BLOCKS), RED_THREADS, 0, c.stream>>>(n, c.V, j + 1, c.h + (m + 1), c.w,
-                                                       c.partials + (size_t)m * GS_BLOCKS, c.dflag, lbytes());
-    MHFP_LAUNCH_CHECK();
-    k_reduce_partials_flag<<<lgrid(1), RED_THREADS, 0, c.stream>>>(GS_BLOCKS, c.partials + (size_t)m * GS_BLOCKS,
-                                                           c.scal + 2, c.dflag, lbytes());
-    MHFP_LAUNCH_CHECK();
+    tail.givens = 1;
+    gs_dots(c, j, h2, nullptr, c.dflag);
+    gs_sub(c, j, h2, c.dflag, tail);
   }
   timing_end(c, 2, 8.0 * n * (2.0 * (j + 1) + 4.0));
-  k_givens<<<lgrid(1), 32, 0, c.stream>>>(j, m, c.h, reorth ? c.h + (m + 1) : nullptr, c.scal + 2, c.H, c.cs, c.sn, c.g,
-                                   c.scal, lbytes());
-  MHFP_LAUNCH_CHECK();
-  k_scale_dev<<<lgrid(grid_for(n, 256)), 256, 0, c.stream>>>(n, c.w, c.scal + 1, c.V + (long long)(j + 1) * n, lbytes());
-  MHFP_LAUNCH_CHECK();
+  if (j + 1 < m) enqueue_next_basis(c, j + 1, c.w, c.scal + 1);  // the last step's successor is never used
   if (host_copy) MHFP_CUDA(cudaMemcpyAsync(c.host_scal, c.scal, sizeof(double), cudaMemcpyDeviceToHost, c.stream));
 }
 
@@ -702,8 +805,7 @@ void fgmres_advance(Ctx& c, FgState& f) {
         finish(c, f, beta / f.bnorm);
         return;
       }
-      k_scale_host<<<grid_for(n, 256), 256, 0, c.stream>>>(n, c.tmp, 1.0 / beta, c.V);
-      MHFP_LAUNCH_CHECK();
+      enqueue_next_basis(c, 0, c.tmp, nullptr, 1.0 / beta);
       k_set_g<<<1, 64, 0, c.stream>>>(m, beta, c.g);
       MHFP_LAUNCH_CHECK();
       f.j = 0;
@@ -729,9 +831,9 @@ void fgmres_advance(Ctx& c, FgState& f) {
         k_lsq<<<1, 32, 0, c.stream>>>(k, m, c.H, c.g, c.yv);
         MHFP_LAUNCH_CHECK();
         if (ff_krylov(c))
-          k_gemv_add_f<<<grid_for(n, 256), 256, 0, c.stream>>>(n, c.ldz, c.Zf, k, c.yv, f.x);
+          k_gemv_add<float><<<grid_for(n, 256), 256, 0, c.stream>>>(n, c.ldz, c.Zf, k, c.yv, f.x);
         else
-          k_gemv_add<<<grid_for(n, 256), 256, 0, c.stream>>>(n, c.Z, k, c.yv, f.x);
+          k_gemv_add<double><<<grid_for(n, 256), 256, 0, c.stream>>>(n, n, c.Z, k, c.yv, f.x);
         MHFP_LAUNCH_CHECK();
         ++f.cycles;
         enqueue_residual(c, f);
@@ -895,18 +997,8 @@ __global__ void k_step_done(DevCtl* __restrict__ ctl, const double* __restrict__
 
 __global__ void k_lsq_dev(const DevCtl* __restrict__ ctl, const double* __restrict__ H, const double* __restrict__ g,
                           double* __restrict__ y, long long lb) {
-  if (threadIdx.x != 0 || blockIdx.x != 0) return;
   ctl = lane_ptr(ctl, lb);
-  H = lane_ptr(H, lb);
-  g = lane_ptr(g, lb);
-  y = lane_ptr(y, lb);
-  const int k = ctl->k, m = ctl->m;
-  for (int i = k - 1; i >= 0; --i) {
-    double s = g[i];
-    for (int c = i + 1; c < k; ++c) s -= H[(long long)c * (m + 1) + i] * y[c];
-    const double d = H[(long long)i * (m + 1) + i];
-    y[i] = d != 0.0 ? s / d : 0.0;
-  }
+  back_substitute(ctl->k, ctl->m, lane_ptr(H, lb), lane_ptr(g, lb), lane_ptr(y, lb));
 }
 
 template <typename ZT>
@@ -914,14 +1006,8 @@ __global__ void k_gemv_add_dev(long long n, long long ld, const ZT* __restrict__
                                const double* __restrict__ y, double* __restrict__ x, long long lb) {
   const long long r = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (r >= n) return;
-  Z = lane_ptr(Z, lb);
-  ctl = lane_ptr(ctl, lb);
-  y = lane_ptr(y, lb);
   x = lane_ptr(x, lb);
-  const int k = ctl->k;
-  double s = x[r];
-  for (int c = 0; c < k; ++c) s += (double)Z[(long long)c * ld + r] * y[c];
-  x[r] = s;
+  x[r] = gemv_row(r, ld, lane_ptr(Z, lb), lane_ptr(ctl, lb)->k, lane_ptr(y, lb), x[r]);
 }
 
 __global__ void k_cycle_end(DevCtl* __restrict__ ctl, long long lb) {
@@ -1061,8 +1147,7 @@ cudaGraphNode_t add_solve(Ctx& c, cudaGraph_t G, cudaGraphNode_t dep, bool trans
   b = add_kernel(W, b, k_cycle_decide, dim3(1), dim3(32), ctl, (const double*)(c.scal + 4), c.scal, c.g, hw,
                  (const cudaGraphConditionalHandle*)d_hif, K, lb);
   b = add_child(W, b, capture_piece(c, [&] {
-    k_scale_dev<<<lgrid(grid_for(n, 256)), 256, 0, c.stream>>>(n, c.tmp, c.scal + 6, c.V, lbytes());
-    MHFP_LAUNCH_CHECK();
+    enqueue_next_basis(c, 0, c.tmp, c.scal + 6);
   }));
   const long long nk_cycle = g_launches - l1;
   long long nk_step = 0;
@@ -1192,7 +1277,7 @@ Ctx* make_lane_ctx(Ctx& base, int K) {
   add(lc->yv, (size_t)m * sizeof(double));
   add(lc->partials, (size_t)(m + 2) * GS_BLOCKS * sizeof(double));
   add(lc->scal, 8 * sizeof(double));
-  add(lc->dflag, 4 * sizeof(int));
+  add(lc->dflag, 16 * sizeof(int));
   if (base.Zf) add(lc->Zf, (size_t)m * (size_t)base.ldz * sizeof(float));  // mixed precision: FP32 Z
   if (base.Z) add(lc->Z, (size_t)m * n * sizeof(double));                  // FP64 throughout
   if (base.tf) add(lc->tf, n * sizeof(float));

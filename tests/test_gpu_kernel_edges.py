@@ -74,3 +74,44 @@ def test_fp64_rows_at_tile_edges(dims):
     assert np.isclose(r, np.linalg.norm(ds * (b - A @ x)), rtol=1e-12)
     assert np.isclose(n0, np.linalg.norm(ds * b), rtol=1e-12)
     s.close()
+
+
+# Gram-Schmidt: the basis columns in groups of eight and chunks of four, rows
+# in blocks of 256, reductions by the last block, both numbers of passes;
+# restart 1, 7, 9 and 63 (column counts 1..63) and vectors of one block up
+@pytest.mark.parametrize("precision", [0, 1])
+@pytest.mark.parametrize("reorth", [0, 1])
+@pytest.mark.parametrize("dims,restart", [((1, 1, 1), 7), ((3, 2, 2), 9), ((6, 5, 4), 63), ((7, 6, 5), 1)])
+def test_arnoldi_vectors_at_edges(dims, restart, reorth, precision):
+    prob = mi.random_small(*dims, seed=5, jitter=0.1)
+    B = oracle.assemble(prob)
+    s = _solver(prob, autotune=0, restart=restart, reorth=reorth, precision=precision, coarse_max=8, cheb_degree=3,
+                maxit=3000)
+    x, st = s.solve(s.build_rhs(), tol=1e-10)
+    ref = oracle.solve_direct(B, oracle.rhs(B))
+    # energy-norm-like check at the residual tolerance (1e-8, as test_gpu_parity's solves)
+    ds = s.scalings()[1].cpu().numpy()
+    err = np.linalg.norm((x.cpu().numpy() - ref) / ds) / np.linalg.norm(ref / ds)
+    assert st["converged"] and err < 1e-7, (st, err)
+    s.close()
+
+
+def test_conversions_match_the_instructions():
+    """The integer-pipe FP32 <-> FP64 conversions (vectors that the mixed form
+    rounds and widens) bit for bit, over every exponent, ties, signed zeros,
+    subnormals, infinities and NaN."""
+    s = _solver(mi.random_small(6, 5, 4, seed=2), autotune=0, precision=1)
+    rng = np.random.default_rng(0)
+    n = s.n
+    v = rng.standard_normal(n) * 2.0 ** rng.integers(-160, 140, n)
+    v[:8] = [0.0, -0.0, np.inf, -np.inf, np.nan, 2.0 ** -149, 3.4028235677973366e38, -2.0 ** -126 * (1 - 2.0 ** -25)]
+    m = rng.integers(0, 1 << 23, n - 8).astype(np.float64) / (1 << 23) + 1.0  # FP32 values plus an exact half ulp
+    v[8:n // 2] = (m + 2.0 ** -24)[: n // 2 - 8] * 2.0 ** rng.integers(-120, 120, n // 2 - 8)
+    x = torch.from_numpy(v).cuda()
+    s.apply_operator_ff(x)  # rounds x; the operator itself is tested elsewhere
+    # apply_precond rounds its input the same way: equal for x and fl32(x)
+    ok = torch.isfinite(x) & (x.abs() < 1e30)
+    x = torch.where(ok, x, torch.zeros_like(x))
+    a, b = s.apply_precond(x), s.apply_precond(x.float().double())
+    assert torch.equal(a, b) and torch.equal(a, a.float().double())
+    s.close()
