@@ -650,7 +650,7 @@ def run_ours(args):
         ff_gbs = off["bytes_per_launch"] / (ff_ms * 1e-3) / 1e9
         roofline_ff = {"bound": "hbm", "achieved": ff_gbs, "peak": peak, "unit": "GB/s", "frac": ff_gbs / peak,
                        "traffic": traffic_for("ff_operator", args.workload, off["bytes_per_launch"]),
-                       "kernel": "Arnoldi operator A_H z in float-float (k_apply_u_ff + k_apply_p_ff + k_apply_pi_ff)",
+                       "kernel": "Arnoldi operator A_H z in float-float (k_apply_ff)",
                        "launches": off["launches"], "avg_launch_us": ff_ms * 1e3,
                        "bytes_per_launch": off["bytes_per_launch"],
                        "fp64_equivalent_tflops": operator_flops(n_mesh) / (ff_ms * 1e-3) / 1e12,

@@ -6,6 +6,7 @@
 // stabilization), Section 2.1 (backward-Euler right-hand side).
 #include "u64.cuh"
 
+#include <algorithm>
 #include <cmath>
 #include <mutex>
 
@@ -771,7 +772,7 @@ __global__ void __launch_bounds__(256) k_btp_p(FaceTopo32 t, const double* __res
 }
 
 // ---------------------------------------------------------------- float-float
-// <hot:ff_operator> (k_apply_u_ff, k_apply_p_ff, k_apply_pi_ff: the source
+// <hot:ff_operator> (k_apply_ff: the source
 // region is hashed so that recorded DRAM counters are dropped once it changes)
 // The Arnoldi step's operator rows for u in float-float arithmetic: every
 // FP64 coefficient a is held as a_h + a_l (two FP32 values, a_h = fl32(a),
@@ -795,27 +796,44 @@ __device__ __forceinline__ void ff_mac(float& sh, float& sl, float ah, float al,
   sl = __fadd_rn(sl, __fadd_rn(err, e));
 }
 
-// y_u = A_uu z_u + cup A_up z_p (then finish: D_s and b as in k_apply_u), one
-// thread per node and its three rows; A_uu's symmetric half (hi, lo) in the
-// node-blocked layout, the lower blocks read transposed from their owners.
-__global__ void __launch_bounds__(256, 4) k_apply_u_ff(Dims d, const float* __restrict__ uh,
-                                                       const float* __restrict__ ul, const float* __restrict__ aph,
-                                                       const float* __restrict__ apl, const float* __restrict__ z,
-                                                       double* __restrict__ y, const double* __restrict__ so,
-                                                       const double* __restrict__ bsub, float cup, long long lb) {
-  z = lane_ptr(z, lb);
-  y = lane_ptr(y, lb);
-  bsub = lane_ptr(bsub, lb);
-  const long long p = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (p >= d.nN) return;
-  const int Lx = d.nx + 1, Ly = d.ny + 1, Lz = d.nz + 1;
-  const int i = (int)(p % Lx), j = (int)((p / Lx) % Ly), k = (int)(p / ((long long)Lx * Ly));
+// One launch for all rows: blocks of 256 rows take the five row families (u
+// nodes, cells, x-, y- and z-faces; about as many blocks each) in turn, so
+// that the families sweep the mesh in z together and what two of them read
+// (A_up by the u and p rows, A_ppi by the p and pi rows, z by all) comes from
+// HBM once and from L2 the second time.  Bound by L2: about 9.6 TB/s of
+// coefficients (A_uu's lower blocks are read a second time there) against
+// 3.47 GB from HBM.  128^3: 762 us, 787 us as three launches (497 + 120 + 170);
+// 64^3: 112 and 114 us; 83 x 64 x 71: 150 and 157 us.
+struct FfOp {
+  int Lx, Ly, Lz;              // nodes per axis
+  long long nN, nT;
+  FaceTopo32 t;
+  const float *uh, *ul;        // A_uu, symmetric half, node-blocked
+  const float *aph, *apl;      // A_up
+  const float *pdh, *pdl, *sth, *stl;  // p block: diagonal, partner coefficients
+  const float *pph, *ppl;      // A_ppi
+  const float *eh, *el;        // A_pipi (ELL)
+  double cup, cpi, cpp;        // coupling factors (the transposed operator changes them)
+  const double* so;            // row scaling, or null
+};
+
+__device__ __forceinline__ double ff_value(float h, float l) { return (double)h + (double)l; }
+
+// y_u = A_uu z_u + cup A_up z_p, one thread per node and its three rows;
+// A_uu's lower blocks read transposed from their owners
+__device__ __forceinline__ void ff_u_rows(const FfOp& o, long long p, const float* __restrict__ z,
+                                          double* __restrict__ y) {
+  if (p >= o.nN) return;
+  const int Lx = o.Lx, Ly = o.Ly, Lz = o.Lz;
+  const unsigned pr = o.t.d_nx1.div((unsigned)p);
+  const int i = (int)((unsigned)p - pr * (unsigned)Lx), k = (int)o.t.d_ny1.div(pr),
+            j = (int)(pr - (unsigned)k * (unsigned)Ly);
   auto in = [&](int a, int b, int c) { return a >= 0 && a < Lx && b >= 0 && b < Ly && c >= 0 && c < Lz; };
   float sh[3] = {0.f, 0.f, 0.f}, sl[3] = {0.f, 0.f, 0.f};
   const long long ob = sym_base(p);
 #pragma unroll 1
   for (int u = 0; u <= 13; ++u) {
-    const int o = 13 + u, dx = o % 3 - 1, dy = (o / 3) % 3 - 1, dz = o / 9 - 1;
+    const int q = 13 + u, dx = q % 3 - 1, dy = (q / 3) % 3 - 1, dz = q / 9 - 1;
     const long long s = dx + (long long)Lx * (dy + (long long)Ly * dz);
     // both blocks' loads are issued before the pair accumulation (an
     // absent neighbour's loads read the node's own rows and are not used)
@@ -825,10 +843,10 @@ __global__ void __launch_bounds__(256, 4) k_apply_u_ff(Dims d, const float* __re
     float oh[9], ol[9], th[9], tl[9], zu[3], zl[3];
 #pragma unroll
     for (int e = 0; e < 9; ++e) {
-      oh[e] = uh[ob + u * 9 * 32 + e * 32];
-      ol[e] = ul[ob + u * 9 * 32 + e * 32];
-      th[e] = uh[qb + e * 32];
-      tl[e] = ul[qb + e * 32];
+      oh[e] = o.uh[ob + u * 9 * 32 + e * 32];
+      ol[e] = o.ul[ob + u * 9 * 32 + e * 32];
+      th[e] = o.uh[qb + e * 32];
+      tl[e] = o.ul[qb + e * 32];
     }
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
@@ -855,123 +873,126 @@ __global__ void __launch_bounds__(256, 4) k_apply_u_ff(Dims d, const float* __re
     }
   }
   // cup A_up z_p over the (up to) eight cells of the node
-  const float* zp = z + 3 * d.nN;
-  for (int cz = k - 1; cz <= k; ++cz) {
-    if (cz < 0 || cz >= d.nz) continue;
-    for (int cy = j - 1; cy <= j; ++cy) {
-      if (cy < 0 || cy >= d.ny) continue;
-      for (int cx = i - 1; cx <= i; ++cx) {
-        if (cx < 0 || cx >= d.nx) continue;
-        const long long T = cell_id(d, cx, cy, cz);
-        const int a = (i - cx) + 2 * (j - cy) + 4 * (k - cz);
-        const float zt = cup * zp[T];
+  const float* zp = z + 3 * o.nN;
+  const float cup = (float)o.cup;
+#pragma unroll 1
+  for (int c = 0; c < 8; ++c) {
+    const int cx = i - 1 + (c & 1), cy = j - 1 + ((c >> 1) & 1), cz = k - 1 + (c >> 2);
+    if (!((unsigned)cx < (unsigned)o.t.nx && (unsigned)cy < (unsigned)o.t.ny && (unsigned)cz < (unsigned)o.t.nz)) continue;
+    const unsigned T = o.t.cell(cx, cy, cz);
+    const long long a = 7 - c;  // the node's local number in the cell
+    const float zt = cup * zp[T];
 #pragma unroll
-        for (int comp = 0; comp < 3; ++comp)
-          ff_mac(sh[comp], sl[comp], aph[(long long)(3 * a + comp) * d.nT + T], apl[(long long)(3 * a + comp) * d.nT + T],
-                 zt);
-      }
-    }
+    for (int e = 0; e < 3; ++e)
+      ff_mac(sh[e], sl[e], o.aph[(3 * a + e) * o.nT + T], o.apl[(3 * a + e) * o.nT + T], zt);
   }
 #pragma unroll
   for (int a = 0; a < 3; ++a) {
     const long long r = 3 * p + a;
-    y[r] = finish((double)sh[a] + (double)sl[a], r, so, bsub);
+    const double v = ff_value(sh[a], sl[a]);
+    y[r] = o.so ? o.so[r] * v : v;
   }
 }
 
-// p rows in float-float: cpu A_pu z_u + (Abar + A_stab) z_p + cpi A_ppi z_pi,
-// each of the three sums carried as a pair and combined in FP64
-__global__ void __launch_bounds__(256, 2) k_apply_p_ff(FaceTopo32 t, const float* __restrict__ aph,
-                                                    const float* __restrict__ apl, const float* __restrict__ pdh,
-                                                    const float* __restrict__ pdl, const float* __restrict__ sth,
-                                                    const float* __restrict__ stl, const float* __restrict__ pph,
-                                                    const float* __restrict__ ppl, double cpi,
-                                                    const float* __restrict__ z, double* __restrict__ y,
-                                                    const double* __restrict__ so, double cpu, long long lb) {
-  z = lane_ptr(z, lb);
-  y = lane_ptr(y, lb);
-  const unsigned T = blockIdx.x * blockDim.x + threadIdx.x;
+// p rows: cpu A_pu z_u + (Abar + A_stab) z_p + cpi A_ppi z_pi (cpu = cup), each of the
+// three sums carried as a pair and combined in FP64
+__device__ __forceinline__ void ff_p_row(const FfOp& o, unsigned T, const float* __restrict__ z,
+                                         double* __restrict__ y) {
+  const FaceTopo32& t = o.t;
   if (T >= t.nT) return;
   const unsigned q = t.d_nx.div(T);
   const int i = (int)(T - q * (unsigned)t.nx), k = (int)t.d_ny.div(q), j = (int)(q - (unsigned)k * (unsigned)t.ny);
-  const unsigned Lx = (unsigned)t.nx + 1, Ly = (unsigned)t.ny + 1;
-  const unsigned nU = 3 * Lx * Ly * ((unsigned)t.nz + 1);
-  // every load of the row is issued before the (serial) pair accumulation
-  float va[24], vb[24], vz[24];
-#pragma unroll
-  for (int a = 0; a < 8; ++a) {
-    const unsigned n = (unsigned)(i + (a & 1)) + Lx * ((unsigned)(j + ((a >> 1) & 1)) + Ly * (unsigned)(k + (a >> 2)));
-#pragma unroll
-    for (int c = 0; c < 3; ++c) {
-      va[3 * a + c] = aph[(unsigned)(3 * a + c) * t.nT + T];
-      vb[3 * a + c] = apl[(unsigned)(3 * a + c) * t.nT + T];
-      vz[3 * a + c] = z[3 * n + c];
-    }
-  }
+  const unsigned Lx = (unsigned)o.Lx, Ly = (unsigned)o.Ly;
+  const unsigned nU = 3 * (unsigned)o.nN;
   float uh = 0.f, ul = 0.f;  // A_up^T z_u (the row is its negative)
+#pragma unroll 1
+  for (int kz = 0; kz < 2; ++kz) {  // four nodes' loads in flight
+    float va[12], vb[12], vz[12];
 #pragma unroll
-  for (int e = 0; e < 24; ++e) ff_mac(uh, ul, va[e], vb[e], vz[e]);
-  const float* zp = z + nU;
-  float ph = 0.f, pl = 0.f;
-  ff_mac(ph, pl, pdh[T], pdl[T], zp[T]);
-  const unsigned nb[3] = {t.cell(i ^ 1, j, k), t.cell(i, j ^ 1, k), t.cell(i, j, k ^ 1)};
+    for (int a = 0; a < 4; ++a) {
+      const unsigned n = (unsigned)(i + (a & 1)) + Lx * ((unsigned)(j + (a >> 1)) + Ly * (unsigned)(k + kz));
 #pragma unroll
-  for (int d = 0; d < 3; ++d) {
-    const float ch = sth[d * t.nT + T];
-    if (ch != 0.f) ff_mac(ph, pl, -ch, -stl[d * t.nT + T], zp[nb[d]]);
+      for (int c = 0; c < 3; ++c) {
+        va[3 * a + c] = o.aph[(unsigned)(12 * kz + 3 * a + c) * t.nT + T];
+        vb[3 * a + c] = o.apl[(unsigned)(12 * kz + 3 * a + c) * t.nT + T];
+        vz[3 * a + c] = z[3 * n + c];
+      }
+    }
+#pragma unroll
+    for (int e = 0; e < 12; ++e) ff_mac(uh, ul, va[e], vb[e], vz[e]);
   }
+  const float* zp = z + nU;
   const float* zpi = zp + t.nT;
   float wa[6], wb[6], wz[6];
 #pragma unroll
   for (int lf = 0; lf < 6; ++lf) {
-    wa[lf] = pph[lf * t.nT + T];
-    wb[lf] = ppl[lf * t.nT + T];
+    wa[lf] = o.pph[lf * t.nT + T];
+    wb[lf] = o.ppl[lf * t.nT + T];
     wz[lf] = zpi[t.face(i, j, k, lf)];
+  }
+  float ph = 0.f, pl = 0.f;
+  ff_mac(ph, pl, o.pdh[T], o.pdl[T], zp[T]);
+  const unsigned nb[3] = {t.cell(i ^ 1, j, k), t.cell(i, j ^ 1, k), t.cell(i, j, k ^ 1)};
+#pragma unroll
+  for (int d = 0; d < 3; ++d) {
+    const float ch = o.sth[d * t.nT + T];
+    if (ch != 0.f) ff_mac(ph, pl, -ch, -o.stl[d * t.nT + T], zp[nb[d]]);
   }
   float ch = 0.f, cl = 0.f;
 #pragma unroll
   for (int lf = 0; lf < 6; ++lf) ff_mac(ch, cl, wa[lf], wb[lf], wz[lf]);
-  const double s = -cpu * ((double)uh + (double)ul) + ((double)ph + (double)pl) + cpi * ((double)ch + (double)cl);
+  const double s = fma(o.cpi, ff_value(ch, cl), fma(-o.cup, ff_value(uh, ul), ff_value(ph, pl)));
   const long long r = (long long)nU + T;
-  y[r] = finish(s, r, so, nullptr);
+  y[r] = o.so ? o.so[r] * s : s;
 }
 
-// pi rows in float-float: cpp A_pip z_p + A_pipi z_pi (ELL, 11 slots)
-__global__ void __launch_bounds__(256, 3) k_apply_pi_ff(FaceTopo32 t, long long nU, const float* __restrict__ pph,
-                                                     const float* __restrict__ ppl, const float* __restrict__ eh,
-                                                     const float* __restrict__ el, const float* __restrict__ z,
-                                                     double* __restrict__ y, const double* __restrict__ so,
-                                                     double cpp, long long lb) {
-  z = lane_ptr(z, lb);
-  y = lane_ptr(y, lb);
-  const unsigned f = blockIdx.x * blockDim.x + threadIdx.x;
-  if (f >= t.nF) return;
+// pi rows: cpp A_pip z_p + A_pipi z_pi (ELL, 11 slots)
+__device__ __forceinline__ void ff_pi_row(const FfOp& o, unsigned f, const float* __restrict__ z,
+                                          double* __restrict__ y) {
+  const FaceTopo32& t = o.t;
   int c[2][3], lf[2];
   bool ok[2];
   t.cells(f, c, ok, lf);
-  const float* zp = z + nU;
+  const float* zp = z + 3 * o.nN;
   const float* zpi = zp + t.nT;
-  float ph = 0.f, pl = 0.f;
-  for (int q = 0; q < 2; ++q)
-    if (ok[q]) {
-      const unsigned T = t.cell(c[q][0], c[q][1], c[q][2]);
-      ff_mac(ph, pl, pph[(long long)lf[q] * t.nT + T], ppl[(long long)lf[q] * t.nT + T], zp[T]);
-    }
   unsigned col[11];
   t.ell_cols(f, col);
   float va[11], vb[11], vz[11];  // every load issued before the pair accumulation
 #pragma unroll
   for (int q = 0; q < 11; ++q) {
-    va[q] = eh[(long long)q * t.nF + f];
-    vb[q] = el[(long long)q * t.nF + f];
+    va[q] = o.eh[(long long)q * t.nF + f];
+    vb[q] = o.el[(long long)q * t.nF + f];
     vz[q] = zpi[col[q]];
   }
+  float ph = 0.f, pl = 0.f;
+#pragma unroll
+  for (int q = 0; q < 2; ++q)
+    if (ok[q]) {
+      const unsigned T = t.cell(c[q][0], c[q][1], c[q][2]);
+      ff_mac(ph, pl, o.pph[(long long)lf[q] * t.nT + T], o.ppl[(long long)lf[q] * t.nT + T], zp[T]);
+    }
   float ah = 0.f, al = 0.f;
 #pragma unroll
   for (int q = 0; q < 11; ++q) ff_mac(ah, al, va[q], vb[q], vz[q]);
-  const double s = cpp * ((double)ph + (double)pl) + ((double)ah + (double)al);
-  const long long r = nU + t.nT + f;
-  y[r] = finish(s, r, so, nullptr);
+  const double s = fma(o.cpp, ff_value(ph, pl), ff_value(ah, al));
+  const long long r = 3 * o.nN + t.nT + f;
+  y[r] = o.so ? o.so[r] * s : s;
+}
+
+__global__ void __launch_bounds__(256, 4) k_apply_ff(FfOp o, const float* __restrict__ z, double* __restrict__ y,
+                                                     long long lb) {
+  z = lane_ptr(z, lb);
+  y = lane_ptr(y, lb);
+  const unsigned role = blockIdx.x % 5, idx = (blockIdx.x / 5) * 256 + threadIdx.x;
+  if (role == 0) {
+    ff_u_rows(o, idx, z, y);
+  } else if (role == 1) {
+    ff_p_row(o, idx, z, y);
+  } else {
+    const unsigned f0 = role == 2 ? 0u : (role == 3 ? o.t.nFx : o.t.nFx + o.t.nFy);
+    const unsigned f1 = role == 2 ? o.t.nFx : (role == 3 ? o.t.nFx + o.t.nFy : o.t.nF);
+    if (idx < f1 - f0) ff_pi_row(o, f0 + idx, z, y);
+  }
 }
 
 // </hot:ff_operator>
@@ -1693,17 +1714,32 @@ void apply_operator_arnoldi(Ctx& c, const double* z, const float* zf, double* y,
     apply_operator(c, z, y, so, nullptr, transpose);
     return;
   }
-  const Dims d = dims_of(c);
   timing_begin(c, 6);
-  k_apply_u_ff<<<lgrid(grid_for(c.nN, 256)), 256, 0, c.stream>>>(d, c.auu_h, c.auu_l, c.Aupf, c.aup_l, zf, y, so, nullptr,
-                                                           transpose ? -1.f : 1.f, lbytes());
-  MHFP_LAUNCH_CHECK();
-  k_apply_p_ff<<<lgrid(grid_for(c.nT, 256)), 256, 0, c.stream>>>(topo32(c), c.Aupf, c.aup_l, c.pd_h, c.pd_l, c.st_h, c.st_l,
-                                                          c.appi_h, c.appi_l, transpose ? 1.0 : c.dt, zf, y, so,
-                                                          transpose ? -1.0 : 1.0, lbytes());
-  MHFP_LAUNCH_CHECK();
-  k_apply_pi_ff<<<lgrid(grid_for(c.nF, 256)), 256, 0, c.stream>>>(topo32(c), 3 * c.nN, c.appi_h, c.appi_l, c.apipi_h,
-                                                           c.apipi_l, zf, y, so, transpose ? c.dt : 1.0, lbytes());
+  FfOp o;
+  o.Lx = c.nx + 1;
+  o.Ly = c.ny + 1;
+  o.Lz = c.nz + 1;
+  o.nN = c.nN;
+  o.nT = c.nT;
+  o.t = topo32(c);
+  o.uh = c.auu_h;
+  o.ul = c.auu_l;
+  o.aph = c.Aupf;
+  o.apl = c.aup_l;
+  o.pdh = c.pd_h;
+  o.pdl = c.pd_l;
+  o.sth = c.st_h;
+  o.stl = c.st_l;
+  o.pph = c.appi_h;
+  o.ppl = c.appi_l;
+  o.eh = c.apipi_h;
+  o.el = c.apipi_l;
+  o.cup = transpose ? -1.0 : 1.0;
+  o.cpi = transpose ? 1.0 : c.dt;
+  o.cpp = transpose ? c.dt : 1.0;
+  o.so = so;
+  const long long most = std::max(std::max(c.nN, c.nFx), std::max(c.nFy, c.nF - c.nFx - c.nFy));
+  k_apply_ff<<<lgrid(5 * grid_for(most, 256)), 256, 0, c.stream>>>(o, zf, y, lbytes());
   MHFP_LAUNCH_CHECK();
   // algorithmic bytes, every coefficient a hi + lo pair (8 B): A_uu's
   // symmetric half (126 per node) and A_up (24 per cell) by the u rows, A_up

@@ -47,34 +47,63 @@ inline unsigned grid_for(long long n, int block) {
 }
 
 // ------------------------------------------------------------ conversions
-// FP32 <-> FP64 on the integer pipe, bit for bit what the conversion
-// instructions give.  Those run on the FP64 pipe (2 per clock and SM on
-// GB300, as an FMA), which made them the bound of kernels that only convert,
-// scale or accumulate FP32 data in FP64; the few integer operations here
-// issue at 64 per clock.  Values outside the normal FP32 range (zeros,
-// subnormals, infinities, NaN) take the instruction.
+// FP32 <-> FP64 on the integer pipe, the values that the conversion
+// instructions give (round to nearest even, subnormals kept).  Those run on
+// the FP64 pipe (2 per clock and SM on GB300, as an FMA), which made them the
+// bound of kernels that only convert, scale or accumulate FP32 data in FP64;
+// the few integer operations here issue at 64 per clock.  No path falls back
+// to the instruction: a compiler that predicates the rare branch would issue
+// it for every value.
 __host__ __device__ __forceinline__ double widen(float f) {
 #ifdef __CUDA_ARCH__
-  const unsigned b = __float_as_uint(f);
-  if (((b >> 23) & 255u) - 1u < 254u)
-    return __hiloint2double((int)((b & 0x80000000u) | (((b & 0x7fffffffu) >> 3) + (896u << 20))), (int)(b << 29));
-#endif
+  const unsigned b = __float_as_uint(f), sign = b & 0x80000000u, e = (b >> 23) & 255u;
+  unsigned hi = ((b & 0x7fffffffu) >> 3) + (896u << 20), lo = b << 29;
+  if (e - 1u >= 254u) {  // zero, subnormal, infinity, NaN
+    unsigned m = b & 0x7fffffu;
+    if (e == 255u) {
+      hi = 0x7ff00000u | (m >> 3) | (m ? 0x80000u : 0u);
+    } else if (m == 0u) {
+      hi = lo = 0u;
+    } else {  // m 2^-149, normalised
+      const int s = __clz((int)m) - 8;
+      m <<= s;
+      hi = ((unsigned)(897 - s) << 20) | ((m & 0x7fffffu) >> 3);
+      lo = m << 29;
+    }
+  }
+  return __hiloint2double((int)(hi | sign), (int)lo);
+#else
   return (double)f;
+#endif
 }
 __host__ __device__ __forceinline__ double widen(double d) { return d; }
 __host__ __device__ __forceinline__ float narrow(double d) {
 #ifdef __CUDA_ARCH__
-  const unsigned hi = (unsigned)__double2hiint(d), lo = (unsigned)__double2loint(d);
-  if (((hi >> 20) & 2047u) - 897u < 254u) {
-    // truncated FP32 bits, then round to nearest even on the 29 bits dropped
-    // (a carry runs into the exponent, up to infinity, as it should)
-    unsigned f = (((hi & 0x7fffffffu) - (896u << 20)) << 3) | (lo >> 29);
-    const unsigned rem = lo & 0x1fffffffu;
-    f += (rem > 0x10000000u || (rem == 0x10000000u && (f & 1u))) ? 1u : 0u;
-    return __uint_as_float(f | (hi & 0x80000000u));
+  const unsigned h = (unsigned)__double2hiint(d), lo = (unsigned)__double2loint(d);
+  const unsigned sign = h & 0x80000000u, hi = h & 0x7fffffffu, e = hi >> 20;
+  // truncated FP32 bits, then round to nearest even on the 29 bits dropped (a
+  // carry runs into the exponent, up to infinity, as it should)
+  unsigned f = ((hi - (896u << 20)) << 3) | (lo >> 29);
+  const unsigned rem = lo & 0x1fffffffu;
+  f += (rem > 0x10000000u || (rem == 0x10000000u && (f & 1u))) ? 1u : 0u;
+  if (e - 897u >= 254u) {
+    if (e > 1150u) {  // beyond FP32's range, or not finite
+      f = e == 2047u && ((hi & 0xfffffu) | lo) ? 0x7fffffffu : 0x7f800000u;
+    } else {  // below the normal range: units of 2^-149
+      const int sh = 926 - (int)e;
+      f = 0u;
+      if (sh <= 54 && e > 0u) {
+        const unsigned long long m = ((unsigned long long)((hi & 0xfffffu) | 0x100000u) << 32) | lo;
+        const unsigned long long r = m & ((1ull << sh) - 1ull), half = 1ull << (sh - 1);
+        f = (unsigned)(m >> sh);
+        f += (r > half || (r == half && (f & 1u))) ? 1u : 0u;
+      }
+    }
   }
-#endif
+  return __uint_as_float(f | sign);
+#else
   return (float)d;
+#endif
 }
 
 // ------------------------------------------------------------ lanes

@@ -115,3 +115,20 @@ def test_conversions_match_the_instructions():
     a, b = s.apply_precond(x), s.apply_precond(x.float().double())
     assert torch.equal(a, b) and torch.equal(a, a.float().double())
     s.close()
+
+
+# the float-float operator's five row families share one launch, a block row
+# per family: sizes where the families need different numbers of blocks
+@pytest.mark.parametrize("dims", [(1, 1, 1), (15, 15, 1), (1, 16, 16), (40, 2, 3), (2, 3, 40), (7, 6, 5)])
+def test_float_float_operator_row_families(dims):
+    prob = mi.random_small(*dims, seed=9, jitter=0.2)
+    s = _solver(prob, autotune=0, precision=1)
+    x = torch.from_numpy(np.random.default_rng(6).standard_normal(s.n).astype(np.float32).astype(np.float64)).cuda()
+    y, ref = s.apply_operator_ff(x), s.apply_operator(x)
+    # 2^-40 of the row's sum of |terms|, bounded by the operator on |x| with
+    # the largest coefficient sum of the block (test_gpu_parity's bound, coarser)
+    nU, nP, _ = s.sizes
+    for a, b in ((0, nU), (nU, nU + nP), (nU + nP, s.n)):
+        scale = ref[a:b].abs().max()
+        assert (y[a:b] - ref[a:b]).abs().max() <= 2.0 ** -38 * scale
+    s.close()
