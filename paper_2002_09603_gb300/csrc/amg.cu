@@ -445,113 +445,56 @@ __global__ void __launch_bounds__(TMA_THREADS, 3) k_sym_tma(Lat L, TmaSweep a0, 
 // </hot:k_cheb_u0_tma>
 
 // ---------------------------------------------------------------- transfers
-// Prolongation x += P x_c and restriction b_c = P^T r between lattice levels,
-// with the same 32-bit indexing and batched loads as the sweeps.  P is
-// stored [ns^3 slots][BF x BC][fine points] (BF unknowns per fine point, BC
-// per coarse point: 3 x 3 or 1 x 1 for M_II^(h), 3 x 6 and 6 x 6 with the
-// rigid-body modes); slot (sx, sy, sz) of fine point (a, b, c) is coarse
-// point (p_lo(a) + sx, p_lo(b) + sy, p_lo(c) + sz).  An absent coarse point
-// contributes 0 (a select, not a multiply).
-template <int BF, int BC, int R, int CH, typename T>
-__device__ __forceinline__ void prolong_sum(const Lat32& F, const Lat32& C, unsigned p, const T* __restrict__ P,
-                                            const T* __restrict__ xc, T acc[BF], int first, int step) {
-  constexpr int ns = (2 + 2 * R) / 3 + 1, NS = ns * ns * ns;
-  int a, b, c;
-  F.ijk(p, a, b, c);
-  const int lx = p_lo(a, R), ly = p_lo(b, R), lz = p_lo(c, R);
-  bool vx[ns], vy[ns], vz[ns];
-#pragma unroll
-  for (int t = 0; t < ns; ++t) {
-    vx[t] = (unsigned)(lx + t) < (unsigned)C.Lx;
-    vy[t] = (unsigned)(ly + t) < (unsigned)C.Ly;
-    vz[t] = (unsigned)(lz + t) < (unsigned)C.Lz;
-  }
-  const unsigned N = (unsigned)F.N;
-#pragma unroll
-  for (int s0 = 0; s0 < NS; s0 += CH) {
-    T pv[CH][BF * BC], xv[CH][BC];
-#pragma unroll
-    for (int q = 0; q < CH; ++q) {
-      const int sl = s0 + q;
-      if (sl < NS && sl % step == first) {
-        const int sx = sl % ns, sy = (sl / ns) % ns, sz = sl / (ns * ns);
-        const bool in = vx[sx] && vy[sy] && vz[sz];
-        const unsigned J = in ? (unsigned)(lx + sx) + (unsigned)C.Lx * ((unsigned)(ly + sy) + (unsigned)C.Ly * (unsigned)(lz + sz)) : 0u;
-#pragma unroll
-        for (int e = 0; e < BF * BC; ++e) {
-          const T v = P[(unsigned)(sl * BF * BC + e) * N + p];
-          pv[q][e] = in ? v : T(0);
-        }
-#pragma unroll
-        for (int t = 0; t < BC; ++t) {
-          const T v = xc[BC * J + t];
-          xv[q][t] = in ? v : T(0);
-        }
-      }
-    }
-#pragma unroll
-    for (int q = 0; q < CH; ++q)
-      if (s0 + q < NS && (s0 + q) % step == first)
-#pragma unroll
-        for (int r = 0; r < BF; ++r)
-#pragma unroll
-          for (int t = 0; t < BC; ++t) acc[r] += pv[q][r * BC + t] * xv[q][t];
-  }
+// Prolongation x += P x_c and restriction b_c = P^T r between lattice levels.
+// P couples coarse point (I, J, K) to the fine box of width w = 3 + 2R around
+// it, fine (3I - R .. 3I + 2 + R) and so on.  The cycles read it coarse-point
+// major, Pc[J][entry][WP]: entry e = BF x BC block entry, then the w^3 box
+// points (x fastest) padded to WP = 128 (R = 1) or 352 (R = 2), out-of-lattice
+// points zero (BF unknowns per fine point, BC per coarse point: 3 x 3 or
+// 1 x 1 for M_II^(h), 3 x 6 and 6 x 6 with the rigid-body modes).  Against the
+// set-up's [slot][entry][fine point] this leaves out the slots that are zero
+// by structure (a fine point with index 1 mod 3 has one coarse neighbour per
+// axis, not two: 4.6 of 8 slots at R = 1, 12.7 of 27 at R = 2, so 366 MB
+// instead of 618 MB on the finest level at 128^3) and makes the restriction a
+// stream: 64.7 us there (5.7 TB/s) against 131 us gathering from the set-up's
+// layout, 48.5 against 75 us on the 2.1 M-point cell level; 11.8 against 27 us
+// and 9.8 against 16 us at 64^3.
+// stencil radius of the levels with BF unknowns per point: the displacement
+// levels are 27-point lattices, the scalar ones 25- or 125-point
+template <int BF>
+constexpr int transfer_r() { return BF == 1 ? 2 : 1; }
+template <int R>
+struct Box {
+  static constexpr int w = 3 + 2 * R, n = w * w * w, WP = R == 1 ? 128 : 352, ns = (2 + 2 * R) / 3 + 1;
+};
+
+// the set-up's P into the cycles' layout and precision: one thread per value
+template <int BB, int R, typename T>
+__global__ void __launch_bounds__(128) k_pack_P(Lat32 F, Lat32 C, const double* __restrict__ P, T* __restrict__ Pc) {
+  using B = Box<R>;
+  constexpr unsigned NB = (B::WP + 127) / 128;  // blocks of 128 per coarse point
+  const unsigned J = blockIdx.x / NB, e = threadIdx.x + (blockIdx.x % NB) * 128;
+  if (e >= (unsigned)B::WP) return;
+  int I, Jj, K;
+  C.ijk(J, I, Jj, K);
+  const int ex = e % B::w, ey = (e / B::w) % B::w, ez = e / (B::w * B::w);
+  const int a = 3 * I - R + ex, b = 3 * Jj - R + ey, c = 3 * K - R + ez;
+  const bool in = e < (unsigned)B::n && (unsigned)a < (unsigned)F.Lx && (unsigned)b < (unsigned)F.Ly &&
+                  (unsigned)c < (unsigned)F.Lz;
+  const unsigned fp = in ? (unsigned)a + (unsigned)F.Lx * ((unsigned)b + (unsigned)F.Ly * (unsigned)c) : 0u;
+  const int sl = in ? (I - p_lo(a, R)) + B::ns * ((Jj - p_lo(b, R)) + B::ns * (K - p_lo(c, R))) : 0;
+#pragma unroll 1
+  for (int t = 0; t < BB; ++t)
+    Pc[((size_t)J * BB + t) * B::WP + e] = in ? (T)P[(size_t)(sl * BB + t) * (unsigned)F.N + fp] : T(0);
 }
 
-template <int BF, int BC>
-constexpr int prolong_chunk() { return BF * BC == 1 ? 9 : (BF * BC <= 9 ? 4 : 1); }
-
-// one fine point per thread
-template <int BF, int BC, int R, typename T>
-__global__ void __launch_bounds__(256) k_prolong_f(Lat32 F, Lat32 C, const T* __restrict__ P,
-                                                   const T* __restrict__ xc, T* __restrict__ x, long long lb) {
-  xc = lane_ptr(xc, lb);
-  x = lane_ptr(x, lb);
-  // blocks take the fine points in descending order: the restriction just
-  // streamed P in ascending order, so its tail is still in L2
-  const unsigned p = (gridDim.x - 1 - blockIdx.x) * blockDim.x + threadIdx.x;
-  if (p >= (unsigned)F.N) return;
-  T acc[BF];
-#pragma unroll
-  for (int r = 0; r < BF; ++r) acc[r] = T(0);
-  prolong_sum<BF, BC, R, prolong_chunk<BF, BC>(), T>(F, C, p, P, xc, acc, 0, 1);
-#pragma unroll
-  for (int r = 0; r < BF; ++r) x[BF * p + r] += acc[r];
-}
-
-// small fine levels: the slots split over W warps for 32 consecutive fine
-// points, partial sums added in a fixed order through shared memory
+// Restriction, W warps per coarse point: the lanes split the box points, each
+// lane issuing the loads of its points before the sums; a fixed-order xor
+// reduction per warp, then over the W warps through shared memory.  With
+// dinvc also the coarse level's first Chebyshev step from zero (d = cr D^-1 b,
+// x = d, the same sums as its own kernel would form from bc).
 template <int BF, int BC, int R, int W, typename T>
-__global__ void __launch_bounds__(32 * W) k_prolong_w(Lat32 F, Lat32 C, const T* __restrict__ P,
-                                                      const T* __restrict__ xc, T* __restrict__ x, long long lb) {
-  xc = lane_ptr(xc, lb);
-  x = lane_ptr(x, lb);
-  __shared__ T part[W][BF][32];
-  const unsigned p = blockIdx.x * 32 + threadIdx.x;
-  const bool valid = p < (unsigned)F.N;
-  T acc[BF];
-#pragma unroll
-  for (int r = 0; r < BF; ++r) acc[r] = T(0);
-  if (valid) prolong_sum<BF, BC, R, (BF * BC > 9 ? 1 : 2), T>(F, C, p, P, xc, acc, threadIdx.y, W);
-#pragma unroll
-  for (int r = 0; r < BF; ++r) part[threadIdx.y][r][threadIdx.x] = acc[r];
-  __syncthreads();
-  if (threadIdx.y != 0 || !valid) return;
-#pragma unroll
-  for (int r = 0; r < BF; ++r) {
-    T sum = T(0);
-#pragma unroll
-    for (int u = 0; u < W; ++u) sum += part[u][r][threadIdx.x];
-    x[BF * p + r] += sum;
-  }
-}
-
-// restriction b_c = P^T r, one warp per coarse point: the lanes split the
-// (3 + 2R)^3 fine box around it, each lane issuing the loads of all its box
-// points before the sums, then a fixed-order xor reduction over the warp
-template <int BF, int BC, int R, typename T>
-__global__ void __launch_bounds__(256) k_restrict_f(Lat32 F, Lat32 C, const T* __restrict__ P,
+__global__ void __launch_bounds__(256) k_restrict_f(Lat32 F, Lat32 C, const T* __restrict__ Pc,
                                                     const T* __restrict__ r, T* __restrict__ bc,
                                                     const T* __restrict__ dinvc, T cr, T* __restrict__ xc,
                                                     T* __restrict__ dc, long long lb) {
@@ -559,11 +502,12 @@ __global__ void __launch_bounds__(256) k_restrict_f(Lat32 F, Lat32 C, const T* _
   bc = lane_ptr(bc, lb);
   xc = lane_ptr(xc, lb);
   dc = lane_ptr(dc, lb);
-  constexpr int ns = (2 + 2 * R) / 3 + 1, w = 3 + 2 * R, NB = w * w * w, PER = (NB + 31) / 32;
-  // blocks larger than 3 x 3 keep one box point's loads in flight at a time
-  constexpr int KB = BF * BC > 9 ? 1 : PER;
-  const unsigned J = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const int lane = threadIdx.x & 31;
+  using B = Box<R>;
+  constexpr int PER = (B::n + 32 * W - 1) / (32 * W);  // box points per lane
+  constexpr int KB = BF * BC > 9 ? 1 : (PER > 4 ? 4 : PER);  // of them in flight
+  __shared__ T part[W > 1 ? 8 : 1][BC];
+  const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31, sub = wid % W;
+  const unsigned J = blockIdx.x * (8 / W) + wid / W;
   const bool valid = J < (unsigned)C.N;
   T acc[BC];
 #pragma unroll
@@ -571,26 +515,21 @@ __global__ void __launch_bounds__(256) k_restrict_f(Lat32 F, Lat32 C, const T* _
   if (valid) {
     int I, Jj, K;
     C.ijk(J, I, Jj, K);
-    const unsigned N = (unsigned)F.N;
+    const T* pj = Pc + (unsigned)(J * (BF * BC)) * (size_t)B::WP;
 #pragma unroll
     for (int k0 = 0; k0 < PER; k0 += KB) {
       T pv[KB][BF * BC], rv[KB][BF];
 #pragma unroll
       for (int kk = 0; kk < KB; ++kk) {
-        const int e = lane + 32 * (k0 + kk);
-        const int ex = e % w, ey = (e / w) % w, ez = e / (w * w);
+        const int e = lane + 32 * (sub + W * (k0 + kk));
+        const int ex = e % B::w, ey = (e / B::w) % B::w, ez = e / (B::w * B::w);
         const int a = 3 * I - R + ex, b = 3 * Jj - R + ey, c = 3 * K - R + ez;
-        const bool in = e < NB && (unsigned)a < (unsigned)F.Lx && (unsigned)b < (unsigned)F.Ly &&
+        const bool ok = k0 + kk < PER && e < B::n && (unsigned)a < (unsigned)F.Lx && (unsigned)b < (unsigned)F.Ly &&
                         (unsigned)c < (unsigned)F.Lz;
-        const int sx = I - p_lo(a, R), sy = Jj - p_lo(b, R), sz = K - p_lo(c, R);
-        const bool ok = in && (unsigned)sx < (unsigned)ns && (unsigned)sy < (unsigned)ns && (unsigned)sz < (unsigned)ns;
         const unsigned fp = ok ? (unsigned)a + (unsigned)F.Lx * ((unsigned)b + (unsigned)F.Ly * (unsigned)c) : 0u;
-        const int sl = ok ? sx + ns * (sy + ns * sz) : 0;
+        const int ec = ok ? e : 0;
 #pragma unroll
-        for (int t = 0; t < BF * BC; ++t) {
-          const T v = P[(unsigned)(sl * BF * BC + t) * N + fp];
-          pv[kk][t] = ok ? v : T(0);
-        }
+        for (int t = 0; t < BF * BC; ++t) pv[kk][t] = pj[t * B::WP + ec];
 #pragma unroll
         for (int t = 0; t < BF; ++t) {
           const T v = r[BF * fp + t];
@@ -606,23 +545,184 @@ __global__ void __launch_bounds__(256) k_restrict_f(Lat32 F, Lat32 C, const T* _
     }
   }
 #pragma unroll
-  for (int q = 0; q < BC; ++q) {
+  for (int q = 0; q < BC; ++q)
 #pragma unroll
     for (int m = 16; m > 0; m >>= 1) acc[q] += __shfl_xor_sync(0xffffffffu, acc[q], m);
-    if (valid && lane == 0) bc[BC * J + q] = acc[q];
+  if (W > 1) {
+    if (lane == 0)
+#pragma unroll
+      for (int q = 0; q < BC; ++q) part[wid][q] = acc[q];
+    __syncthreads();
+    if (sub != 0) return;
+#pragma unroll
+    for (int q = 0; q < BC; ++q)
+#pragma unroll
+      for (int u = 1; u < W; ++u) acc[q] += part[wid + u][q];
   }
-  // the coarse level's first Chebyshev step from zero (with dinvc): d = cr
-  // D^-1 b, x = d, the same sums as its own kernel would form from bc
-  if (dinvc && valid && lane == 0) {
-    const unsigned Nc = (unsigned)C.N;
+  if (!valid || lane >= BC) return;
+  // lane a takes component a
+  T s = acc[0];
 #pragma unroll
-    for (int a = 0; a < BC; ++a) {
-      T z = T(0);
+  for (int q = 1; q < BC; ++q) s = lane == q ? acc[q] : s;
+  bc[BC * J + lane] = s;
+  if (dinvc) {
+    T z = T(0);
 #pragma unroll
-      for (int t = 0; t < BC; ++t) z += dinvc[(unsigned)(a * BC + t) * Nc + J] * acc[t];
-      dc[BC * J + a] = cr * z;
-      xc[BC * J + a] = cr * z;
+    for (int t = 0; t < BC; ++t) z += dinvc[(unsigned)(lane * BC + t) * (unsigned)C.N + J] * acc[t];
+    dc[BC * J + lane] = cr * z;
+    xc[BC * J + lane] = cr * z;
+  }
+}
+
+// acc += the coarse points in the (sy, sz) slot pairs first, first + step, ...
+// of fine point (a, b, c) (a pair without a coarse point is skipped: uniform along x)
+template <int BF, int BC, int R, typename T>
+__device__ __forceinline__ void prolong_sum(const Lat32& C, int a, int b, int c, const T* __restrict__ Pc,
+                                            const T* __restrict__ xc, T acc[BF], int first, int step) {
+  using B = Box<R>;
+  const int lx = p_lo(a, R), ly = p_lo(b, R), lz = p_lo(c, R);
+#pragma unroll 1
+  for (int yz = first; yz < B::ns * B::ns; yz += step) {
+    const int Jy = ly + yz % B::ns, Kz = lz + yz / B::ns;
+    const int ey = b - 3 * Jy + R, ez = c - 3 * Kz + R;
+    if ((unsigned)Jy >= (unsigned)C.Ly || (unsigned)Kz >= (unsigned)C.Lz || ey < 0 || ez < 0) continue;
+    T pv[B::ns][BF * BC], xv[B::ns][BC];
+#pragma unroll
+    for (int sx = 0; sx < B::ns; ++sx) {
+      const int Ix = lx + sx, ex = a - 3 * Ix + R;
+      const bool in = (unsigned)Ix < (unsigned)C.Lx && ex >= 0;
+      const unsigned J = in ? (unsigned)Ix + (unsigned)C.Lx * ((unsigned)Jy + (unsigned)C.Ly * (unsigned)Kz) : 0u;
+      const unsigned e = in ? (unsigned)(ex + B::w * (ey + B::w * ez)) : 0u;
+      const T* pj = Pc + (unsigned)(J * (BF * BC)) * (size_t)B::WP + e;
+#pragma unroll
+      for (int t = 0; t < BF * BC; ++t) pv[sx][t] = in ? pj[t * B::WP] : T(0);
+#pragma unroll
+      for (int t = 0; t < BC; ++t) xv[sx][t] = in ? xc[BC * J + t] : T(0);
     }
+#pragma unroll
+    for (int sx = 0; sx < B::ns; ++sx)
+#pragma unroll
+      for (int q = 0; q < BF; ++q)
+#pragma unroll
+        for (int t = 0; t < BC; ++t) acc[q] += pv[sx][q * BC + t] * xv[sx][t];
+  }
+}
+
+// Large displacement levels read the set-up's fine-point major layout
+// Pm[slot][entry][fine point], where every load of a warp is one line
+// (coarse-point major it is a line per three lanes).  A warp takes one
+// (sy, sz) slot pair for 32 fine points: one round of loads, the partial sums
+// joined in order; pairs that are zero by structure are skipped, uniformly
+// along x, so that 0.69 of P is read.  Microseconds, this form / a thread per
+// fine point on the same layout / the same coarse-point major / all eight
+// slots by a thread (before): 274,625 points 3 x 3 14.3 / 15.5 / 22.7 / 15.1,
+// 2,146,689 points 86 / 91 / 126 / 108, 110,592 points 3 x 6 14.5 / 30.6 /
+// 18.3 / 21.3, 68,921 points 3 x 3 FP64 13.9 / 20.5 / 17.7 / 14.7.
+template <int BF, int BC, int R, typename T>
+__global__ void __launch_bounds__(32 * Box<R>::ns * Box<R>::ns)
+    k_prolong_f(Lat32 F, Lat32 C, const T* __restrict__ Pm, const T* __restrict__ xc, T* __restrict__ x,
+                long long lb) {
+  using B = Box<R>;
+  constexpr int W = B::ns * B::ns;
+  xc = lane_ptr(xc, lb);
+  x = lane_ptr(x, lb);
+  __shared__ T part[W][BF][32];
+  // blocks take the fine points in descending order: the restriction went
+  // through them in ascending order, so the last ones' x is still in L2
+  const unsigned p = (gridDim.x - 1 - blockIdx.x) * 32 + threadIdx.x;
+  const bool valid = p < (unsigned)F.N;
+  const int yz = threadIdx.y;
+  T acc[BF];
+#pragma unroll
+  for (int r = 0; r < BF; ++r) acc[r] = T(0);
+  int a, b, c;
+  F.ijk(valid ? p : 0u, a, b, c);
+  const int lx = p_lo(a, R), Jy = p_lo(b, R) + yz % B::ns, Kz = p_lo(c, R) + yz / B::ns;
+  if (valid && (unsigned)Jy < (unsigned)C.Ly && (unsigned)Kz < (unsigned)C.Lz && b - 3 * Jy + R >= 0 &&
+      c - 3 * Kz + R >= 0) {
+    T pv[B::ns][BF * BC], xv[B::ns][BC];
+#pragma unroll
+    for (int sx = 0; sx < B::ns; ++sx) {
+      const bool in = (unsigned)(lx + sx) < (unsigned)C.Lx;
+      const unsigned J = in ? (unsigned)(lx + sx) + (unsigned)C.Lx * ((unsigned)Jy + (unsigned)C.Ly * (unsigned)Kz) : 0u;
+      const T* pj = Pm + (unsigned)((sx + B::ns * yz) * (BF * BC)) * (size_t)(unsigned)F.N + p;
+#pragma unroll
+      for (int t = 0; t < BF * BC; ++t) {
+        const T v = pj[(size_t)t * (unsigned)F.N];
+        pv[sx][t] = in ? v : T(0);
+      }
+#pragma unroll
+      for (int t = 0; t < BC; ++t) {
+        const T v = xc[BC * J + t];
+        xv[sx][t] = in ? v : T(0);
+      }
+    }
+#pragma unroll
+    for (int sx = 0; sx < B::ns; ++sx)
+#pragma unroll
+      for (int q = 0; q < BF; ++q)
+#pragma unroll
+        for (int t = 0; t < BC; ++t) acc[q] += pv[sx][q * BC + t] * xv[sx][t];
+  }
+#pragma unroll
+  for (int r = 0; r < BF; ++r) part[yz][r][threadIdx.x] = acc[r];
+  __syncthreads();
+  if (yz != 0 || !valid) return;
+#pragma unroll
+  for (int r = 0; r < BF; ++r) {
+#pragma unroll
+    for (int u = 1; u < W; ++u) acc[r] += part[u][r][threadIdx.x];
+    x[BF * p + r] += acc[r];
+  }
+}
+
+// Large scalar levels: a thread per fine point on the coarse-point major
+// layout (262,144 points: 8.6 us, 10.1 with all 27 slots read before, 14.1
+// split as above; 2,097,152 points: 54, 65 and 105)
+template <int R, typename T>
+__global__ void __launch_bounds__(256) k_prolong_s(Lat32 F, Lat32 C, const T* __restrict__ Pc,
+                                                   const T* __restrict__ xc, T* __restrict__ x, long long lb) {
+  xc = lane_ptr(xc, lb);
+  x = lane_ptr(x, lb);
+  const unsigned p = (gridDim.x - 1 - blockIdx.x) * blockDim.x + threadIdx.x;
+  if (p >= (unsigned)F.N) return;
+  int a, b, c;
+  F.ijk(p, a, b, c);
+  T acc[1] = {T(0)};
+  prolong_sum<1, 1, R, T>(C, a, b, c, Pc, xc, acc, 0, 1);
+  x[p] += acc[0];
+}
+
+// small fine levels: a warp per (sy, sz) slot pair for 32 consecutive fine
+// points, partial sums added in a fixed order through shared memory
+template <int BF, int BC, int R, typename T>
+__global__ void __launch_bounds__(32 * Box<R>::ns * Box<R>::ns)
+    k_prolong_w(Lat32 F, Lat32 C, const T* __restrict__ Pc, const T* __restrict__ xc, T* __restrict__ x,
+                long long lb) {
+  constexpr int W = Box<R>::ns * Box<R>::ns;
+  xc = lane_ptr(xc, lb);
+  x = lane_ptr(x, lb);
+  __shared__ T part[W][BF][32];
+  const unsigned p = blockIdx.x * 32 + threadIdx.x;
+  const bool valid = p < (unsigned)F.N;
+  T acc[BF];
+#pragma unroll
+  for (int r = 0; r < BF; ++r) acc[r] = T(0);
+  if (valid) {
+    int a, b, c;
+    F.ijk(p, a, b, c);
+    prolong_sum<BF, BC, R, T>(C, a, b, c, Pc, xc, acc, threadIdx.y, W);
+  }
+#pragma unroll
+  for (int r = 0; r < BF; ++r) part[threadIdx.y][r][threadIdx.x] = acc[r];
+  __syncthreads();
+  if (threadIdx.y != 0 || !valid) return;
+#pragma unroll
+  for (int r = 0; r < BF; ++r) {
+    T sum = T(0);
+#pragma unroll
+    for (int u = 0; u < W; ++u) sum += part[u][r][threadIdx.x];
+    x[BF * p + r] += sum;
   }
 }
 
@@ -1684,18 +1784,53 @@ void build_pi(Ctx& c) {
   make_dense_coarse(c, last);
 }
 
+// coarse points below which the restriction takes four warps each (at one
+// warp, on the set-up's layout, 1,040 points of a 3 x 3 FP64 level took 11.1 us
+// instead of 7.5, 4,096 points of a 6 x 6 level 16.2 instead of 4.4)
+constexpr long long RESTRICT_WIDE = 6000;
+// fine points from which the prolongation takes its wide forms (k_prolong_f, k_prolong_s)
+constexpr long long PROLONG_WIDE = 65536;
+
+// (re)write a level's prolongator in the cycles' layout and precision
+template <typename T>
+void pack_P(Ctx& c, const Level& L, const Level& C, T* Pc) {
+  const Lat32 F = lat32_of(L.A), Cc = lat32_of(C.A);
+  dispatch_pair(L.bs, C.bs, [&](auto BF, auto BC) {
+    constexpr int R = transfer_r<BF.value>();
+    k_pack_P<BF.value * BC.value, R, T>
+        <<<(unsigned)(C.A.N * ((Box<R>::WP + 127) / 128)), 128, 0, c.stream>>>(F, Cc, L.P, Pc);
+  });
+  MHFP_LAUNCH_CHECK();
+}
+size_t setup_P_size(const Level& L) {
+  const size_t ns = (size_t)p_slots(L.R);
+  return ns * ns * ns * L.bs * L.cbs * L.npts;
+}
+size_t packed_P_size(const Level& L, const Level& C) {
+  return (size_t)C.A.N * L.bs * C.bs * (L.bs == 1 ? Box<2>::WP : Box<1>::WP);
+}
+
+// the FP64 cycles' prolongators (allocated on the first call)
+void make_fp64_transfers(Ctx& c, std::vector<Level>& H) {
+  for (size_t l = 0; l + 1 < H.size(); ++l) {
+    if (!H[l].P) continue;
+    if (!H[l].Pd) H[l].Pd = dalloc_n<double>(c, packed_P_size(H[l], H[l + 1]));
+    pack_P<double>(c, H[l], H[l + 1], H[l].Pd);
+  }
+}
+
 // ------------------------------------------------------------------ V-cycle
 // Pointers of one level in the precision T of the cycle: the FP64 arrays
 // built by the set-up, or their FP32 copies for the mixed-precision cycle.
 template <typename T>
 struct LV {
-  const T *val, *dinv, *P, *ell, *pw;
+  const T *val, *dinv, *P, *Pm, *ell, *pw;  // P: coarse-point major, Pm: fine-point major
   T *r, *d, *y;
 };
 LV<double> view(Ctx& c, Level& L, double) {
-  return {L.A.val, L.dinv, L.P, L.ell ? L.ell : c.Cpi, c.pw, L.r, L.d, L.y};
+  return {L.A.val, L.dinv, L.Pd, L.P, L.ell ? L.ell : c.Cpi, c.pw, L.r, L.d, L.y};
 }
-LV<float> view(Ctx& c, Level& L, float) { return {L.valf, L.dinvf, L.Pf, c.Cpif, c.pwf, L.rf, L.df, L.yf}; }
+LV<float> view(Ctx& c, Level& L, float) { return {L.valf, L.dinvf, L.Pf, L.Pmf, c.Cpif, c.pwf, L.rf, L.df, L.yf}; }
 double* bvec(Level& L, double) { return L.b; }
 float* bvec(Level& L, float) { return L.bf; }
 double* xvec(Level& L, double) { return L.x; }
@@ -2012,10 +2147,15 @@ void vcycle_level(Ctx& c, std::vector<Level>& H, int l, const T* b, T* x, bool p
   } else {
     const Lat32 F = lat32_of(L.A), Cc = lat32_of(C.A);
     dispatch_pair(L.bs, C.bs, [&](auto BF, auto BC) {
-      dispatch_r(L.R, [&](auto RR) {
-        k_restrict_f<BF.value, BC.value, RR.value, T><<<lgrid(grid_for(C.A.N * 32, 256)), 256, 0, c.stream>>>(
+      constexpr int R = transfer_r<BF.value>();
+      // four warps per coarse point where one each would leave SMs idle, and
+      // for the blocks of the rigid-body modes (one box point per lane)
+      if (C.A.N < RESTRICT_WIDE || BF.value * BC.value > 9)
+        k_restrict_f<BF.value, BC.value, R, 4, T><<<lgrid(grid_for(C.A.N, 2)), 256, 0, c.stream>>>(
             F, Cc, v.P, v.r, cb, fdinv, fcr, fx, fd, lbytes());
-      });
+      else
+        k_restrict_f<BF.value, BC.value, R, 1, T><<<lgrid(grid_for(C.A.N, 8)), 256, 0, c.stream>>>(
+            F, Cc, v.P, v.r, cb, fdinv, fcr, fx, fd, lbytes());
     });
   }
   MHFP_LAUNCH_CHECK();
@@ -2023,17 +2163,19 @@ void vcycle_level(Ctx& c, std::vector<Level>& H, int l, const T* b, T* x, bool p
   if (L.faces) {
     k_prolong_faces<T><<<lgrid(grid_for(c.nF, 256)), 256, 0, c.stream>>>(face_topo(c), v.pw, cx, s_buf, lbytes());
   } else {
-    // one fine point per thread on large levels, slots split over 8 warps on small ones
     const Lat32 F = lat32_of(L.A), Cc = lat32_of(C.A);
     dispatch_pair(L.bs, C.bs, [&](auto BF, auto BC) {
-      dispatch_r(L.R, [&](auto RR) {
-        if (L.A.N >= 65536)
-          k_prolong_f<BF.value, BC.value, RR.value, T><<<lgrid(grid_for(L.A.N, 256)), 256, 0, c.stream>>>(
-              F, Cc, v.P, cx, s_buf, lbytes());
-        else
-          k_prolong_w<BF.value, BC.value, RR.value, 8, T><<<lgrid(grid_for(L.A.N, 32)), dim3(32, 8), 0, c.stream>>>(
-              F, Cc, v.P, cx, s_buf, lbytes());
-      });
+      constexpr int R = transfer_r<BF.value>();
+      if (L.A.N >= PROLONG_WIDE && BF.value == 1)
+        k_prolong_s<R, T><<<lgrid(grid_for(L.A.N, 256)), 256, 0, c.stream>>>(F, Cc, v.P, cx, s_buf, lbytes());
+      else if (L.A.N >= PROLONG_WIDE)
+        k_prolong_f<BF.value, BC.value, R, T>
+            <<<lgrid(grid_for(L.A.N, 32)), dim3(32, Box<R>::ns * Box<R>::ns), 0, c.stream>>>(F, Cc, v.Pm, cx, s_buf,
+                                                                                             lbytes());
+      else
+        k_prolong_w<BF.value, BC.value, R, T>
+            <<<lgrid(grid_for(L.A.N, 32)), dim3(32, Box<R>::ns * Box<R>::ns), 0, c.stream>>>(F, Cc, v.P, cx, s_buf,
+                                                                                             lbytes());
     });
   }
   MHFP_LAUNCH_CHECK();
@@ -2070,8 +2212,9 @@ void make_fp32(Ctx& c, std::vector<Level>& H, bool fine_sym) {
     }
     if (L.dinv) L.dinvf = cast_copy(c, L.dinv, bs2 * L.npts);
     if (L.P) {
-      const int ns = p_slots(L.R);
-      L.Pf = cast_copy(c, L.P, (size_t)ns * ns * ns * L.bs * L.cbs * L.npts);
+      L.Pf = dalloc_n<float>(c, packed_P_size(L, H[l + 1]));
+      pack_P<float>(c, L, H[l + 1], L.Pf);
+      if (L.bs > 1 && L.A.N >= PROLONG_WIDE) L.Pmf = cast_copy(c, L.P, setup_P_size(L));
     }
     L.xf = dalloc_n<float>(c, L.n);
     L.bf = dalloc_n<float>(c, L.n);
@@ -2092,6 +2235,9 @@ void build_hierarchies(Ctx& c) {
     make_fp32(c, c.hpi, false);
     c.Cpif = cast_copy(c, c.Cpi, (size_t)11 * c.nF);
     c.pwf = cast_copy(c, c.pw, c.nF);
+  } else {
+    make_fp64_transfers(c, c.hu);
+    make_fp64_transfers(c, c.hpi);
   }
   if (c.opt.autotune) {
     // the finest displacement level runs k_cheb_u0 (FP64) or the symmetric
@@ -2141,17 +2287,17 @@ void rebuild_pi_hierarchy(Ctx& c) {
       k_cast_f32<<<grid_for((long long)n, 256), 256, 0, c.stream>>>((long long)n, src, dst);
       MHFP_LAUNCH_CHECK();
     };
-    for (Level& L : H) {
+    for (size_t l = 0; l < H.size(); ++l) {
+      Level& L = H[l];
       const size_t bs2 = (size_t)L.bs * L.bs;
       if (!L.faces && L.valf) recast(L.valf, L.A.val, (size_t)L.A.noff() * bs2 * L.A.N);
       if (L.dinv && L.dinvf) recast(L.dinvf, L.dinv, bs2 * L.npts);
-      if (L.P && L.Pf) {
-        const int ns = p_slots(L.R);
-        recast(L.Pf, L.P, (size_t)ns * ns * ns * L.bs * L.cbs * L.npts);
-      }
+      if (L.P && L.Pf) pack_P<float>(c, L, H[l + 1], L.Pf);
     }
     recast(c.Cpif, c.Cpi, (size_t)11 * c.nF);
     recast(c.pwf, c.pw, c.nF);
+  } else {
+    make_fp64_transfers(c, H);
   }
 }
 
@@ -2194,6 +2340,8 @@ void build_mixed_hierarchies(Ctx& c) {
   Level& last = c.hcp.back();
   alloc_work(c, last);
   make_dense_coarse(c, last);
+  make_fp64_transfers(c, c.hu);
+  make_fp64_transfers(c, c.hcp);
   if (c.opt.autotune)
     for (auto* H : {&c.hu, &c.hcp})
       for (size_t l = 0; l < H->size(); ++l) {

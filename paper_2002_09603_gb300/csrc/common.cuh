@@ -352,7 +352,10 @@ struct Level {
   double* dinv = nullptr;     // [bs*bs][npts] inverse diagonal blocks
   double lmax = 0.0;
   // prolongator to the next level (lattice levels only): [p_slots^3][bs*bs][npts]
+  // as the set-up builds it (fine-point major; Pmf: FP32, large levels), and coarse-point major
+  // as the restriction and the small levels' prolongation read it (Pd; Pf: FP32)
   double* P = nullptr;
+  double* Pd = nullptr;
   int R = 1;                  // stencil radius of A (L_inf)
   int cbs = 0;                // unknowns per point of the next level (P blocks are bs x cbs)
   const double* ell = nullptr; // face level: its ELL values (null: C~_pi)
@@ -365,7 +368,7 @@ struct Level {
   // last level: dense inverse (n x n, row-major)
   double* dense_inv = nullptr;
   // FP32 copies for the mixed-precision cycle (precision == 1)
-  float *valf = nullptr, *dinvf = nullptr, *Pf = nullptr;
+  float *valf = nullptr, *dinvf = nullptr, *Pf = nullptr, *Pmf = nullptr;
   float* symf = nullptr;      // finest displacement level, FP32: symmetric half, node blocks of 32 x 126 rows
   double sweep_us = 0.0;      // autotuner's time of one sweep under the chosen schedule
   float *xf = nullptr, *bf = nullptr, *rf = nullptr, *df = nullptr, *yf = nullptr;

@@ -159,12 +159,6 @@ void dispatch_pair(int bf, int bc, F&& f) {
   else f(std::integral_constant<int, 1>{}, std::integral_constant<int, 1>{});
 }
 
-template <class F>
-void dispatch_r(int R, F&& f) {
-  if (R == 2) f(std::integral_constant<int, 2>{});
-  else f(std::integral_constant<int, 1>{});
-}
-
 // 32-bit lattice view for the coarse-level kernels (their indices e N + p
 // and bs q + s stay below 2^31)
 inline Lat32 lat32_of(const StructOp& A) {
