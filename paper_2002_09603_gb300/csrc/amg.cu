@@ -949,27 +949,54 @@ __global__ void k_dinv_ell(long long n, const double* __restrict__ val, double* 
   if (f < n) dinv[f] = 1.0 / val[f];
 }
 
-// y = D^-1 x (block), x and y of length BS*N
+// One power-iteration step after r = A v: w = (D^-1 r) / *rho_v and, by the
+// last block, *rho_w = ||w||, with *rho_v the norm of v: the iterates are
+// never scaled by a pass of their own and the host reads only the last norm.
+// Without dinv only *rho_w = ||r|| (the start vector's norm).
+constexpr int POWER_BLOCKS = 304;
 template <int BS>
-__global__ void k_apply_dinv(long long N, const double* __restrict__ dinv, const double* __restrict__ x,
-                             double* __restrict__ y) {
-  const long long p = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (p >= N) return;
-  for (int a = 0; a < BS; ++a) {
-    double s = 0.0;
-    for (int t = 0; t < BS; ++t) s += dinv[(long long)(a * BS + t) * N + p] * x[BS * p + t];
-    y[BS * p + a] = s;
+__global__ void __launch_bounds__(256) k_power_step(long long N, const double* __restrict__ dinv,
+                                                    const double* __restrict__ r, double* __restrict__ w,
+                                                    const double* __restrict__ rho_v, double* __restrict__ rho_w,
+                                                    double* __restrict__ partials, unsigned* __restrict__ counter) {
+  __shared__ double sh[8];
+  const double inv = dinv ? 1.0 / *rho_v : 0.0;
+  double acc = 0.0;
+  for (long long p = (long long)blockIdx.x * 256 + threadIdx.x; p < N; p += (long long)gridDim.x * 256) {
+    double x[BS];
+#pragma unroll
+    for (int t = 0; t < BS; ++t) x[t] = r[BS * p + t];
+    if (!dinv) {
+#pragma unroll
+      for (int t = 0; t < BS; ++t) acc = fma(x[t], x[t], acc);
+      continue;
+    }
+#pragma unroll
+    for (int a = 0; a < BS; ++a) {
+      double s = 0.0;
+#pragma unroll
+      for (int t = 0; t < BS; ++t) s += dinv[(long long)(a * BS + t) * N + p] * x[t];
+      s *= inv;
+      w[BS * p + a] = s;
+      acc = fma(s, s, acc);
+    }
   }
+  for (int o = 16; o > 0; o >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, o);
+  if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = acc;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    double s = 0.0;
+    for (int k = 0; k < 8; ++k) s += sh[k];
+    partials[blockIdx.x] = s;
+  }
+  if (!last_block(counter, gridDim.x) || threadIdx.x >= 32) return;
+  const double n2 = warp_sum_of(partials, (int)gridDim.x);
+  if (threadIdx.x == 0) *rho_w = sqrt(n2);
 }
 
 __global__ void k_power_start(long long n, double* __restrict__ v) {
   const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (i < n) v[i] = 1.0 + (double)((7919LL * i) % 97) / 97.0;
-}
-
-__global__ void k_scale_by(long long n, double s, double* __restrict__ v) {
-  const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < n) v[i] *= s;
 }
 
 // Smoothed prolongator: P[a, J] = [a in J] diag(active_a) - omega D_a^-1 sum_{b in J, b ~ a} A_ab diag(active_b)
@@ -1013,6 +1040,11 @@ __global__ void k_build_P(Lat F, Lat Cc, const double* __restrict__ val, const d
       for (int r = 0; r < BS; ++r) out[r * BS + r] += active[BS * p + r] ? 1.0 : 0.0;
   }
   for (int q = 0; q < BS * BS; ++q) P[((long long)s * BS * BS + q) * F.N + p] = out[q];
+}
+
+__global__ void k_active_fine(long long nU, const unsigned char* __restrict__ fix, unsigned char* __restrict__ act) {
+  const long long r = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  if (r < nU) act[r] = ((fix[r / 3] >> (r % 3)) & 1) ? 0 : 1;
 }
 
 template <int BS>
@@ -1348,6 +1380,9 @@ void level_spmv(Ctx& c, Level& L, const double* x, const double* b, double* y) {
   if (L.faces) {
     k_spmv_ell<double><<<lgrid(grid_for(L.n, 256)), 256, 0, c.stream>>>(face_topo(c), L.ell ? L.ell : c.Cpi, x, b, y,
                                                                          lbytes());
+  } else if (L.bs == 3) {
+    launch_u64(c.stream, lat32_of(L.A), (const double*)L.A.val, (const double*)nullptr, 0.0, x,
+               (const double*)nullptr, b, y);
   } else {
     launch_spmv<double>(c, L.A, L.bs, L.A.val, x, b, y, default_schedule(L.A.N, L.bs));
   }
@@ -1362,29 +1397,35 @@ void alloc_work(Ctx& c, Level& L) {
   L.y = dalloc_n<double>(c, L.n);
 }
 
-// rho(D^-1 A) by power iteration from the fixed start vector
+// rho(D^-1 A) by power iteration from the fixed start vector: two launches
+// per iteration and one read at the end (five launches and a read before)
 double spectral_radius(Ctx& c, Level& L) {
   const long long n = L.n;
   double* v = L.x;
   double* w = L.y;
-  k_power_start<<<grid_for(n, 256), 256, 0, c.stream>>>(n, v);
-  MHFP_LAUNCH_CHECK();
-  double nv = device_norm2(c, v, n);
-  k_scale_by<<<grid_for(n, 256), 256, 0, c.stream>>>(n, 1.0 / nv, v);
-  MHFP_LAUNCH_CHECK();
-  double rho = 0.0;
-  for (int it = 0; it < c.opt.power_iters; ++it) {
-    level_spmv(c, L, v, nullptr, L.r);
+  ensure_workspace(c);
+  // the partial sums, the block counter and the norms of the last two
+  // iterates (scal[4], scal[5], in turn) are the Krylov workspace's
+  unsigned* counter = (unsigned*)(c.dflag + 1);
+  auto step = [&](const double* dinv, const double* r, double* out, int it) {
     dispatch_bs(L.bs, [&](auto BS) {
-      k_apply_dinv<BS.value><<<grid_for(L.npts, 256), 256, 0, c.stream>>>(L.npts, L.dinv, L.r, w);
+      k_power_step<BS.value><<<std::min<unsigned>(grid_for(L.npts, 256), POWER_BLOCKS), 256, 0, c.stream>>>(
+          L.npts, dinv, r, out, c.scal + 4 + (it + 1) % 2, c.scal + 4 + it % 2, c.partials, counter);
     });
     MHFP_LAUNCH_CHECK();
-    rho = device_norm2(c, w, n);
-    k_scale_by<<<grid_for(n, 256), 256, 0, c.stream>>>(n, 1.0 / rho, w);
-    MHFP_LAUNCH_CHECK();
+  };
+  k_power_start<<<grid_for(n, 256), 256, 0, c.stream>>>(n, v);
+  MHFP_LAUNCH_CHECK();
+  step(nullptr, v, nullptr, 0);
+  for (int it = 0; it < c.opt.power_iters; ++it) {
+    level_spmv(c, L, v, nullptr, L.r);
+    step(L.dinv, L.r, w, it + 1);
     std::swap(v, w);
   }
-  return rho;
+  double h = 0.0;
+  MHFP_CUDA(cudaMemcpyAsync(&h, c.scal + 4 + c.opt.power_iters % 2, sizeof(double), cudaMemcpyDeviceToHost, c.stream));
+  MHFP_CUDA(cudaStreamSynchronize(c.stream));
+  return h;
 }
 
 // Gauss-Jordan inverse with partial pivoting (host, FP64), row-major
@@ -1422,112 +1463,97 @@ __global__ void k_gj_extract(int n, const double* __restrict__ M, double* __rest
   inv[t] = M[r * 2 * n + n + cidx];
 }
 
-__global__ void k_gj_init(int n, const double* __restrict__ A, double* __restrict__ M) {
+// Galerkin scratch of the set-up: one buffer for every level of a handle's
+// hierarchies (the first level of the first one needs the most), given back
+// by release_setup_scratch once they are built
+void release_setup_scratch(Ctx& c) {
+  if (!c.setup_Q) return;
+  MHFP_CUDA(cudaStreamSynchronize(c.stream));  // its last kernel may still run
+  dfree(c, c.setup_Q);
+  c.setup_Q = nullptr;
+  c.setup_Q_elems = 0;
+}
+double* setup_scratch(Ctx& c, size_t elems) {
+  if (c.setup_Q_elems < elems) {
+    release_setup_scratch(c);
+    c.setup_Q = (double*)dalloc_own(c, elems * sizeof(double));
+    c.setup_Q_elems = elems;
+  }
+  return c.setup_Q;
+}
+// the coarsest level's matrix as the left half of the elimination's [A | I]
+__global__ void k_gj_init(int n, double* __restrict__ M) {
   const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= (long long)n * 2 * n) return;
   const long long r = t / (2 * n), cidx = t % (2 * n);
-  M[t] = cidx < n ? A[r * n + cidx] : (cidx - n == r ? 1.0 : 0.0);
+  M[t] = cidx - n == r ? 1.0 : 0.0;
+}
+// a row's stencil offsets have distinct columns: plain stores
+__global__ void k_gj_lattice(Lat L, int kind, int no, int bs, const double* __restrict__ val, double* __restrict__ M) {
+  const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  if (t >= L.N * no) return;
+  const int o = (int)(t / L.N);
+  const long long p = t - (long long)o * L.N;
+  int i, j, k, dx, dy, dz;
+  L.ijk(p, i, j, k);
+  stencil_offset(kind, o, dx, dy, dz);
+  if (!L.in(i + dx, j + dy, k + dz)) return;
+  const long long q = L.id(i + dx, j + dy, k + dz), w = 2 * bs * L.N;
+  for (int r = 0; r < bs; ++r)
+    for (int s = 0; s < bs; ++s) M[(bs * p + r) * w + bs * q + s] = val[((long long)o * bs * bs + r * bs + s) * L.N + p];
+}
+// face rows (absent cells' slots name the row's own face with value 0)
+__global__ void k_gj_faces(int n, const int* __restrict__ col, const double* __restrict__ val, double* __restrict__ M) {
+  const int f = blockIdx.x * blockDim.x + threadIdx.x;
+  if (f >= n) return;
+  for (int q = 0; q < 11; ++q) M[(long long)f * 2 * n + col[(long long)q * n + f]] += val[(long long)q * n + f];
 }
 
-// A (host, n x n row-major) -> its inverse in device memory `inv`.  With
-// keep, the elimination workspace is the handle's persistent one (allocated
-// once, for permeability updates); otherwise it is allocated and freed here.
-void invert_dense_gpu(Ctx& c, const std::vector<double>& A, int n, double* inv, bool keep = false) {
-  double *dA = nullptr, *M = nullptr, *prow = nullptr, *fcol = nullptr;
-  int* err = nullptr;
-  auto release = [&] {
-    if (keep) return;
-    cudaFree(dA);
-    cudaFree(M);
-    cudaFree(prow);
-    cudaFree(fcol);
-    cudaFree(err);
-  };
-  cudaError_t e = cudaSuccess;
-  if (keep) {
-    if (c.gj_n < n) {
-      c.gj_A = dalloc_n<double>(c, (size_t)n * n);
-      c.gj_M = dalloc_n<double>(c, (size_t)n * 2 * n);
-      c.gj_prow = dalloc_n<double>(c, (size_t)2 * n);
-      c.gj_fcol = dalloc_n<double>(c, (size_t)n);
-      if (!c.gj_err) c.gj_err = dalloc_n<int>(c, 1);
-      c.gj_n = n;
-    }
-    dA = c.gj_A;
-    M = c.gj_M;
-    prow = c.gj_prow;
-    fcol = c.gj_fcol;
-    err = c.gj_err;
-  } else {
-    e = cudaMalloc(&dA, (size_t)n * n * sizeof(double));
-    if (e == cudaSuccess) e = cudaMalloc(&M, (size_t)n * 2 * n * sizeof(double));
-    if (e == cudaSuccess) e = cudaMalloc(&prow, (size_t)2 * n * sizeof(double));
-    if (e == cudaSuccess) e = cudaMalloc(&fcol, (size_t)n * sizeof(double));
-    if (e == cudaSuccess) e = cudaMalloc(&err, sizeof(int));
-  }
-  if (e != cudaSuccess) {
-    release();
-    throw Error{MHFP_ERR_OOM, "device allocation failed (dense coarsest level)"};
-  }
-  try {
-    MHFP_CUDA(cudaMemcpyAsync(dA, A.data(), (size_t)n * n * sizeof(double), cudaMemcpyHostToDevice, c.stream));
-    MHFP_CUDA(cudaMemsetAsync(err, 0, sizeof(int), c.stream));
-    k_gj_init<<<grid_for((long long)n * 2 * n, 256), 256, 0, c.stream>>>(n, dA, M);
-    MHFP_LAUNCH_CHECK();
-    for (int col = 0; col < n; ++col) {
-      k_gj_pivot<<<grid_for(2 * n, 256), 256, 0, c.stream>>>(n, col, M, prow, fcol, err);
-      MHFP_LAUNCH_CHECK();
-      k_gj_update<<<dim3(grid_for(2 * n - col, 256), n), 256, 0, c.stream>>>(n, col, M, prow, fcol);
-      MHFP_LAUNCH_CHECK();
-    }
-    k_gj_extract<<<grid_for((long long)n * n, 256), 256, 0, c.stream>>>(n, M, inv);
-    MHFP_LAUNCH_CHECK();
-    int h_err = 0;
-    MHFP_CUDA(cudaMemcpyAsync(&h_err, err, sizeof(int), cudaMemcpyDeviceToHost, c.stream));
-    MHFP_CUDA(cudaStreamSynchronize(c.stream));
-    if (h_err) throw Error{MHFP_ERR_ARG, "singular or indefinite coarsest multigrid level"};
-  } catch (...) {
-    cudaStreamSynchronize(c.stream);
-    release();
-    throw;
-  }
-  release();
-}
-
+// The dense inverse of the coarsest level into L.dense_inv.  On a rebuild
+// (permeability update) the elimination workspace is the handle's persistent
+// one (allocated once); otherwise it is the set-up's scratch.
 void make_dense_coarse(Ctx& c, Level& L) {
   const int n = (int)L.n;
-  std::vector<double> A((size_t)n * n, 0.0);
-  if (L.faces) {
-    std::vector<int> col(11 * (size_t)n);
-    std::vector<double> val(11 * (size_t)n);
-    MHFP_CUDA(cudaMemcpyAsync(col.data(), c.ell_col, col.size() * sizeof(int), cudaMemcpyDeviceToHost, c.stream));
-    MHFP_CUDA(cudaMemcpyAsync(val.data(), c.Cpi, val.size() * sizeof(double), cudaMemcpyDeviceToHost, c.stream));
-    MHFP_CUDA(cudaStreamSynchronize(c.stream));
-    for (int f = 0; f < n; ++f)
-      for (int q = 0; q < 11; ++q) A[(size_t)f * n + col[(size_t)q * n + f]] += val[(size_t)q * n + f];
-  } else {
-    const StructOp& S = L.A;
-    const int bs = S.bs, no = S.noff();
-    std::vector<double> val((size_t)no * bs * bs * S.N);
-    MHFP_CUDA(cudaMemcpyAsync(val.data(), S.val, val.size() * sizeof(double), cudaMemcpyDeviceToHost, c.stream));
-    MHFP_CUDA(cudaStreamSynchronize(c.stream));
-    for (long long p = 0; p < S.N; ++p) {
-      const int i = (int)(p % S.Lx), j = (int)((p / S.Lx) % S.Ly), k = (int)(p / ((long long)S.Lx * S.Ly));
-      for (int o = 0; o < no; ++o) {
-        int dx, dy, dz;
-        stencil_offset(S.kind, o, dx, dy, dz);
-        const int a = i + dx, b = j + dy, cc = k + dz;
-        if (a < 0 || a >= S.Lx || b < 0 || b >= S.Ly || cc < 0 || cc >= S.Lz) continue;
-        const long long q = a + (long long)S.Lx * (b + (long long)S.Ly * cc);
-        for (int r = 0; r < bs; ++r)
-          for (int t = 0; t < bs; ++t)
-            A[(size_t)(bs * p + r) * n + bs * q + t] += val[((size_t)o * bs * bs + r * bs + t) * S.N + p];
-      }
-    }
-  }
   const bool rebuild = L.dense_inv != nullptr;
   if (!rebuild) L.dense_inv = dalloc_n<double>(c, (size_t)n * n);
-  invert_dense_gpu(c, A, n, L.dense_inv, rebuild);
+  double *M, *prow, *fcol;
+  int* err;
+  const size_t elems = (size_t)n * 2 * n + 3 * (size_t)n + 1;
+  double* ws;
+  if (rebuild) {
+    if (c.gj_n < n) {
+      c.gj_M = dalloc_n<double>(c, elems);
+      c.gj_n = n;
+    }
+    ws = c.gj_M;
+  } else {
+    ws = setup_scratch(c, elems);
+  }
+  M = ws;
+  prow = M + (size_t)n * 2 * n;
+  fcol = prow + 2 * (size_t)n;
+  err = (int*)(fcol + n);
+  MHFP_CUDA(cudaMemsetAsync(err, 0, sizeof(int), c.stream));
+  k_gj_init<<<grid_for((long long)n * 2 * n, 256), 256, 0, c.stream>>>(n, M);
+  MHFP_LAUNCH_CHECK();
+  if (L.faces)
+    k_gj_faces<<<grid_for(n, 128), 128, 0, c.stream>>>(n, c.ell_col, c.Cpi, M);
+  else
+    k_gj_lattice<<<grid_for(L.A.N * L.A.noff(), 128), 128, 0, c.stream>>>(lat_of(L.A), L.A.kind, L.A.noff(), L.A.bs,
+                                                                          L.A.val, M);
+  MHFP_LAUNCH_CHECK();
+  for (int col = 0; col < n; ++col) {
+    k_gj_pivot<<<grid_for(2 * n, 256), 256, 0, c.stream>>>(n, col, M, prow, fcol, err);
+    MHFP_LAUNCH_CHECK();
+    k_gj_update<<<dim3(grid_for(2 * n - col, 256), n), 256, 0, c.stream>>>(n, col, M, prow, fcol);
+    MHFP_LAUNCH_CHECK();
+  }
+  k_gj_extract<<<grid_for((long long)n * n, 256), 256, 0, c.stream>>>(n, M, L.dense_inv);
+  MHFP_LAUNCH_CHECK();
+  int h_err = 0;
+  MHFP_CUDA(cudaMemcpyAsync(&h_err, err, sizeof(int), cudaMemcpyDeviceToHost, c.stream));
+  MHFP_CUDA(cudaStreamSynchronize(c.stream));
+  if (h_err) throw Error{MHFP_ERR_ARG, "singular or indefinite coarsest multigrid level"};
 }
 
 void finish_level(Ctx& c, Level& L) {
@@ -1587,10 +1613,10 @@ Level coarsen(Ctx& c, Level& L, Level* into = nullptr) {
     }
     Q = c.upd_Q;
   } else {
-    MHFP_CUDA(cudaMalloc(&Q, q_elems * sizeof(double)));
+    Q = setup_scratch(c, q_elems);
   }
   const double omega = 4.0 / (3.0 * L.lmax);
-  try {
+  {
     dispatch_bs13(L.bs, [&](auto BS) {
       dispatch_kind_bs<BS.value>(A.kind, [&](auto K) {
         k_build_P<BS.value, K.value><<<grid_for(F.N * ns * ns * ns, 256), 256, 0, c.stream>>>(F, Cc, A.val, L.dinv,
@@ -1612,12 +1638,7 @@ Level coarsen(Ctx& c, Level& L, Level* into = nullptr) {
                                                                                              Cl.active, Cl.A.val);
       MHFP_LAUNCH_CHECK();
     });
-    MHFP_CUDA(cudaStreamSynchronize(c.stream));
-  } catch (...) {
-    if (!into) cudaFree(Q);
-    throw;
   }
-  if (!into) MHFP_CUDA(cudaFree(Q));
   return Cl;
 }
 
@@ -1630,15 +1651,8 @@ void build_u_level0(Ctx& c) {
   L0.n = c.nU;
   L0.R = 1;
   L0.active = dalloc_n<unsigned char>(c, c.nU);
-  {
-    std::vector<unsigned char> fix(c.nN), act(c.nU);
-    MHFP_CUDA(cudaMemcpyAsync(fix.data(), c.node_fix, c.nN, cudaMemcpyDeviceToHost, c.stream));
-    MHFP_CUDA(cudaStreamSynchronize(c.stream));
-    for (long long n = 0; n < c.nN; ++n)
-      for (int q = 0; q < 3; ++q) act[3 * n + q] = ((fix[n] >> q) & 1) ? 0 : 1;
-    MHFP_CUDA(cudaMemcpyAsync(L0.active, act.data(), c.nU, cudaMemcpyHostToDevice, c.stream));
-    MHFP_CUDA(cudaStreamSynchronize(c.stream));
-  }
+  k_active_fine<<<grid_for(c.nU, 256), 256, 0, c.stream>>>(c.nU, c.node_fix, L0.active);
+  MHFP_LAUNCH_CHECK();
   c.hu.push_back(L0);
 }
 
@@ -1703,9 +1717,8 @@ void build_u_rbm(Ctx& c) {
     Cl.A.val = dalloc_n<double>(c, (size_t)27 * RBM_K * RBM_K * Cc.N);
     MHFP_CUDA(cudaMemsetAsync(Pt, 0, (size_t)pb * F.N * sizeof(double), c.stream));
     const double omega = 4.0 / (3.0 * L.lmax);
-    double* Q = nullptr;
-    MHFP_CUDA(cudaMalloc(&Q, (size_t)nq * nq * nq * pb * F.N * sizeof(double)));
-    try {
+    double* Q = setup_scratch(c, (size_t)nq * nq * nq * pb * F.N);
+    {
       const unsigned warps = grid_for(Cc.N * 32, 128);
       auto galerkin = [&](auto BF) {
         constexpr int bf = decltype(BF)::value;
@@ -1729,12 +1742,7 @@ void build_u_rbm(Ctx& c) {
         MHFP_LAUNCH_CHECK();
         galerkin(std::integral_constant<int, RBM_K>{});
       }
-      MHFP_CUDA(cudaStreamSynchronize(c.stream));
-    } catch (...) {
-      cudaFree(Q);
-      throw;
     }
-    MHFP_CUDA(cudaFree(Q));
     Nprev = Nc;
     c.hu.push_back(Cl);
   }
@@ -1935,9 +1943,11 @@ void launch_resid_sym(Ctx& c, const Level& L, const float* x, const float* b, fl
 // `reps` calls captured once into a CUDA graph on a private stream, the
 // graph replayed once to warm up and three times under events, the fastest
 // replay kept.  Timing graph replays leaves out host launch overhead, as in
-// the solve, which runs as graphs.
+// the solve, which runs as graphs.  A candidate that is twice as slow as
+// `best` in its warm-up, or 1.15 times in its first timed replay, is not
+// replayed again.
 template <class F>
-float graph_time_us(Ctx& c, int reps, F&& body) {
+float graph_time_us(Ctx& c, int reps, float best_us, F&& body) {
   cudaStream_t user = c.stream, st = nullptr;
   MHFP_CUDA(cudaStreamCreateWithFlags(&st, cudaStreamNonBlocking));
   MHFP_CUDA(cudaStreamSynchronize(user));
@@ -1974,6 +1984,11 @@ float graph_time_us(Ctx& c, int reps, F&& body) {
     float ms = 0.f;
     if (e == cudaSuccess) e = cudaEventElapsedTime(&ms, e0, e1);
     if (e == cudaSuccess && it > 0 && ms < best) best = ms;
+    const float us = ms * 1e3f / reps;
+    if (e == cudaSuccess && (it == 0 ? us > 2.f * best_us : us > 1.15f * best_us)) {
+      best = std::min(best, ms);
+      break;
+    }
   }
   if (e0) cudaEventDestroy(e0);
   if (e1) cudaEventDestroy(e1);
@@ -1982,6 +1997,11 @@ float graph_time_us(Ctx& c, int reps, F&& body) {
   MHFP_CUDA(e);
   return best * 1e3f / reps;
 }
+
+// sweeps per timed replay: about 40 us of them at 3 TB/s, 2 to 5 (ten
+// sweeps, replayed four times whatever the candidate, took 32 of the 122 ms of
+// a 96^3 set-up and 14 of 34 ms at 45 x 52 x 39)
+int tune_reps(double bytes) { return (int)std::min(5.0, std::max(2.0, 40.0 / (bytes / 3e6))); }
 
 // Set-up autotuner for the finest displacement level in FP32: time the two
 // occupancy variants of the symmetric sweep and keep the faster in L.tpp.
@@ -1993,7 +2013,7 @@ void autotune_fine_sym(Ctx& c, Level& L) {
   int best_minb = 0;
   for (int minb : {8, 7, 6, 5, 4}) {
     L.tpp = minb;
-    const float us = graph_time_us(c, 5, [&] { launch_cheb_sym(c, L, L.bf, L.xf, L.yf, L.df, 0.5f, 0.5f); });
+    const float us = graph_time_us(c, tune_reps(4.0 * 126 * L.A.N), best, [&] { launch_cheb_sym(c, L, L.bf, L.xf, L.yf, L.df, 0.5f, 0.5f); });
     if (us < best) {
       best = us;
       best_minb = minb;
@@ -2018,7 +2038,7 @@ void autotune_level(Ctx& c, Level& L) {
   float best = 1e30f;
   int best_tpp = default_schedule(L.A.N, L.bs);
   for (int tpp : {1, 4, 8, 16}) {
-    const float us = graph_time_us(c, 10, [&] {
+    const float us = graph_time_us(c, tune_reps((double)sizeof(T) * L.A.noff() * L.bs * L.bs * L.A.N), best, [&] {
       launch_cheb<T>(c, L, v, b, x, v.y, T(0.5), T(0.5), tpp);
       MHFP_LAUNCH_CHECK();
     });
@@ -2230,6 +2250,7 @@ void build_hierarchies(Ctx& c) {
   if (c.opt.near_kernel == 1) build_u_rbm(c);
   else build_u(c);
   build_pi(c);
+  release_setup_scratch(c);
   if (c.opt.precision == 1) {
     make_fp32(c, c.hu, true);
     make_fp32(c, c.hpi, false);
@@ -2340,6 +2361,7 @@ void build_mixed_hierarchies(Ctx& c) {
   Level& last = c.hcp.back();
   alloc_work(c, last);
   make_dense_coarse(c, last);
+  release_setup_scratch(c);
   make_fp64_transfers(c, c.hu);
   make_fp64_transfers(c, c.hcp);
   if (c.opt.autotune)

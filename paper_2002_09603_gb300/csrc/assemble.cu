@@ -1351,7 +1351,7 @@ FaceTopo32 topo32(const Ctx& c) { return FaceTopo32::make(c.nx, c.ny, c.nz, c.nT
 void assemble_all(Ctx& c) {
   const Dims d = dims_of(c);
   MHFP_CUDA(cudaMemsetAsync(c.d_flag, 0, sizeof(int), c.stream));
-  double* Ke = dalloc_n<double>(c, (size_t)576 * c.nT);
+  double* Ke = (double*)dalloc_own(c, (size_t)576 * c.nT * sizeof(double));
   c.Aup = dalloc_n<double>(c, (size_t)24 * c.nT);
   c.vol = dalloc_n<double>(c, c.nT);
   MHFP_CUDA(cudaFuncSetAttribute(k_q1, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Q1_SMEM));
@@ -1383,9 +1383,7 @@ void assemble_all(Ctx& c) {
   MHFP_CUDA(cudaMemcpyAsync(&hflag, c.d_flag, sizeof(int), cudaMemcpyDeviceToHost, c.stream));
   MHFP_CUDA(cudaStreamSynchronize(c.stream));
   // the element stiffness is consumed by the gather; release it now
-  for (auto it = c.allocs.begin(); it != c.allocs.end(); ++it)
-    if (*it == (void*)Ke) { c.allocs.erase(it); break; }
-  MHFP_CUDA(cudaFree(Ke));
+  dfree(c, Ke);
   if (hflag & 1) throw Error{MHFP_ERR_MESH, "inverted or degenerate element (det J <= 0 at a Gauss point)"};
   if (hflag & 2) throw Error{MHFP_ERR_MESH, "RT0 element mass matrix is not positive definite"};
 }
@@ -1482,7 +1480,7 @@ void update_logk_blocks(Ctx& c, const double* logk) {
 // D_s = diag(A_uu, C~_p, A_qq)^(-1/2).
 void build_mixed_blocks(Ctx& c) {
   const Dims d = dims_of(c);
-  double* Aww = dalloc_n<double>(c, (size_t)36 * c.nT);
+  double* Aww = (double*)dalloc_own(c, (size_t)36 * c.nT * sizeof(double));
   MHFP_CUDA(cudaMemsetAsync(c.d_flag, 0, sizeof(int), c.stream));
   k_rt0<<<grid_for(c.nT, 128), 128, 0, c.stream>>>(d, c.coords, c.mu, c.kappa, c.Seps, c.vol, c.dt, c.W, c.W1, c.sW,
                                                    c.Abar, c.d_flag, Aww);
@@ -1511,9 +1509,7 @@ void build_mixed_blocks(Ctx& c) {
   MHFP_CUDA(cudaMemcpyAsync(&hflag, c.d_flag, sizeof(int), cudaMemcpyDeviceToHost, c.stream));
   MHFP_CUDA(cudaStreamSynchronize(c.stream));
   // the cell mass matrices are consumed by the face rows; release them now
-  for (auto it = c.allocs.begin(); it != c.allocs.end(); ++it)
-    if (*it == (void*)Aww) { c.allocs.erase(it); break; }
-  MHFP_CUDA(cudaFree(Aww));
+  dfree(c, Aww);
   if (hflag & 2) throw Error{MHFP_ERR_MESH, "RT0 element mass matrix is not positive definite"};
 }
 

@@ -106,6 +106,32 @@ __host__ __device__ __forceinline__ float narrow(double d) {
 #endif
 }
 
+// ------------------------------------------------------------ reductions
+// The blocks of a reduction meet on a counter: every block publishes its
+// partial sums, and the last one to arrive reduces them all in a fixed order
+// (no block waits) and rearms the counter.  Saves the separate reduction
+// kernels: a launch and 3 us each.
+__device__ __forceinline__ bool last_block(unsigned* counter, unsigned nblocks) {
+  __shared__ bool last;
+  __threadfence();
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    last = atomicAdd(counter, 1u) == nblocks - 1;
+    if (last) *counter = 0u;
+  }
+  __syncthreads();
+  if (last) __threadfence();
+  return last;
+}
+
+// sum of p[0..nb) by one warp in a fixed order; every lane returns it
+__device__ __forceinline__ double warp_sum_of(const double* p, int nb) {
+  double v = 0.0;
+  for (int b = threadIdx.x & 31; b < nb; b += 32) v += __ldcg(p + b);
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  return v;
+}
+
 // ------------------------------------------------------------ lanes
 // Several right-hand sides of one handle solved in lockstep ("lanes"): every
 // kernel of the solve runs once for all of them, lane l in blockIdx.z.  A
@@ -456,8 +482,7 @@ struct Ctx {
   // (permeability updates): Galerkin Q and the Gauss-Jordan workspace
   double* upd_Q = nullptr;
   size_t upd_Q_elems = 0;
-  double *gj_A = nullptr, *gj_M = nullptr, *gj_prow = nullptr, *gj_fcol = nullptr;
-  int* gj_err = nullptr;
+  double* gj_M = nullptr;
   int gj_n = 0;
   cudaGraphConditionalHandle* d_hif[2] = {nullptr, nullptr};  // IF handles of the solve graphs
 
@@ -497,6 +522,10 @@ struct Ctx {
   Timing timing;
   bool suppress_events = false;  // capture without timing events (conditional bodies)
   std::vector<void*> allocs;
+  char* arena = nullptr;         // small buffers are carved from chunks of the handle's own
+  size_t arena_left = 0;
+  double* setup_Q = nullptr;     // Galerkin scratch, held while a hierarchy is built
+  size_t setup_Q_elems = 0;
   // CUDA graphs of the Arnoldi steps: [transpose][j]
   cudaStream_t cap_stream = nullptr;
   std::vector<IterGraph> graphs[2];
@@ -537,6 +566,8 @@ struct FgState {
 
 // allocation helpers (tracked, freed at destroy)
 void* dalloc(Ctx& c, size_t bytes);
+void* dalloc_own(Ctx& c, size_t bytes);  // a cudaMalloc of its own, for buffers that dfree gives back early
+void dfree(Ctx& c, void* p);
 template <class T>
 T* dalloc_n(Ctx& c, size_t n) { return (T*)dalloc(c, n * sizeof(T)); }
 void dfree_all(Ctx& c);

@@ -76,31 +76,6 @@ __device__ __forceinline__ void gs_rows(long long n, const double* __restrict__ 
   }
 }
 
-// The blocks of a reduction meet on a counter: every block publishes its
-// partial sums, and the last one to arrive reduces them all in a fixed order
-// (no block waits) and rearms the counter.  Saves the separate reduction
-// kernels: a launch and 3 us each.
-__device__ __forceinline__ bool last_block(unsigned* counter, unsigned nblocks) {
-  __shared__ bool last;
-  __threadfence();
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    last = atomicAdd(counter, 1u) == nblocks - 1;
-    if (last) *counter = 0u;
-  }
-  __syncthreads();
-  if (last) __threadfence();
-  return last;
-}
-
-// sum of p[0..nb) by one warp in a fixed order; every lane returns it
-__device__ __forceinline__ double warp_sum_of(const double* p, int nb) {
-  double v = 0.0;
-  for (int b = threadIdx.x & 31; b < nb; b += 32) v += __ldcg(p + b);
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  return v;
-}
-
 // hout[c] = V[:, c] . w for the columns c <= j, eight per block row
 // (blockIdx.y), and *nrm2 = w . w when given.  Nothing happens when *skip.
 __global__ void __launch_bounds__(RED_THREADS, 4) k_gs_dots(long long n, const double* __restrict__ V, int j,
@@ -1247,6 +1222,8 @@ Ctx* make_lane_ctx(Ctx& base, int K) {
   ensure_solve_state(base);
   Ctx* lc = new Ctx(base);
   lc->allocs.clear();
+  lc->arena = nullptr;
+  lc->arena_left = 0;
   lc->timing = Timing{};
   lc->suppress_events = false;
   lc->cap_stream = nullptr;
