@@ -1104,14 +1104,110 @@ __global__ void k_build_Q(Lat F, Lat Cc, const double* __restrict__ val, const d
   for (int q = 0; q < BF * BC; ++q) Q[((long long)s * BF * BC + q) * F.N + p] = out[q];
 }
 
-// A_c[J, J+oc] = sum_{a in box(J)} P[a, J]^T Q[a, J+oc]   (BC x BC blocks)
+// The same for 3 x 3 blocks on the 27-point lattice, bound by the FP64 pipe
+// (125 block products, 3,375 FMA per fine point: 5.1 ms at 96^3).  In the
+// kernel above a warp's lanes have all three residues of the fine x index, so
+// nine (offset, slot) pairs per axis are issued for five that are not zero.
+// Here a warp takes 32 fine points of one residue RHO (a = 3 m + RHO), whose
+// products are known at compile time: x slots of the neighbours 3 n: {n - 1, n},
+// 3 n + 1: {n}, 3 n + 2: {n, n + 1}.  A block has the nine warps (residue,
+// Jy slot) of a line's 96 points, so that the three residues share lines in
+// L1; a lane keeps up to three x slots of 3 x 3 sums.  Slots that are zero by
+// structure are not written (k_rap does not read them).  96^3, finest level:
+// 17.3 ms before, 6.9 ms.
+template <int RHO>
+__device__ __forceinline__ void q3_line(const Lat32& F, unsigned p, int a, int dy, int dz, int py, int pz,
+                                        const double* __restrict__ val, const double* __restrict__ P,
+                                        double (&acc)[3][9]) {
+  const size_t N = (unsigned)F.N;
+  const int o0 = 3 * (dy + 1) + 9 * (dz + 1);
+#pragma unroll
+  for (int dx = -1; dx <= 1; ++dx) {
+    const bool in = (unsigned)(a + dx) < (unsigned)F.Lx;
+    double A[9];
+#pragma unroll
+    for (int e = 0; e < 9; ++e) A[e] = val[(size_t)((o0 + dx + 1) * 9 + e) * N + p];
+    // the neighbour (the point itself where there is none: its block is zero)
+    const unsigned q = p + (unsigned)((in ? dx : 0) + F.Lx * dy + F.LxLy * dz);
+    constexpr int QLO = RHO == 2 ? 0 : -1;  // q_lo(a) - m
+    const int sig = (RHO + dx + 3) % 3, nm = (RHO + dx + 3) / 3 - 1;  // a + dx = 3 (m + nm) + sig
+#pragma unroll
+    for (int sx = 0; sx < 2; ++sx) {
+      if (sig == 1 && sx == 1) continue;
+      const int jx = nm + sx - (sig == 0 ? 1 : 0) - QLO;  // Q slot of coarse m + nm + sx (- 1)
+      const double* pv = P + (size_t)((sx + 2 * (py + 2 * pz)) * 9) * N + q;
+      double b[9];
+#pragma unroll
+      for (int e = 0; e < 9; ++e) b[e] = pv[(size_t)e * N];
+#pragma unroll
+      for (int r = 0; r < 3; ++r)
+#pragma unroll
+        for (int t = 0; t < 3; ++t)
+#pragma unroll
+          for (int u = 0; u < 3; ++u) acc[jx][3 * r + t] = fma(A[3 * r + u], b[3 * u + t], acc[jx][3 * r + t]);
+    }
+  }
+}
+
+template <int RHO>
+__device__ __forceinline__ void q3_point(const Lat32& F, const Lat32& C, int a, int b, int c, int sy,
+                                         const double* __restrict__ val, const double* __restrict__ P,
+                                         double* __restrict__ Q) {
+  const size_t N = (unsigned)F.N;
+  const int Jy = q_lo(b, 1) + sy;
+  if ((unsigned)Jy >= (unsigned)C.Ly || b - 3 * Jy + 2 < 0) return;
+  const unsigned p = (unsigned)(a + F.Lx * b) + (unsigned)F.LxLy * (unsigned)c;
+#pragma unroll 1
+  for (int sz = 0; sz < 3; ++sz) {
+    const int Jz = q_lo(c, 1) + sz;
+    if ((unsigned)Jz >= (unsigned)C.Lz || c - 3 * Jz + 2 < 0) continue;
+    double acc[3][9];
+#pragma unroll
+    for (int j = 0; j < 3; ++j)
+#pragma unroll
+      for (int e = 0; e < 9; ++e) acc[j][e] = 0.0;
+#pragma unroll 1
+    for (int dz = -1; dz <= 1; ++dz) {
+      const int nc = c + dz, pz = Jz - p_lo(nc, 1);
+      if ((unsigned)nc >= (unsigned)F.Lz || (unsigned)(nc - 3 * Jz + 1) >= 5u) continue;
+#pragma unroll 1
+      for (int dy = -1; dy <= 1; ++dy) {
+        const int nb = b + dy, py = Jy - p_lo(nb, 1);
+        if ((unsigned)nb >= (unsigned)F.Ly || (unsigned)(nb - 3 * Jy + 1) >= 5u) continue;
+        q3_line<RHO>(F, p, a, dy, dz, py, pz, val, P, acc);
+      }
+    }
+#pragma unroll
+    for (int j = 0; j < (RHO == 1 ? 3 : 2); ++j)
+#pragma unroll
+      for (int e = 0; e < 9; ++e) Q[(size_t)((j + 3 * (sy + 3 * sz)) * 9 + e) * N + p] = acc[j][e];
+  }
+}
+
+__global__ void __launch_bounds__(288, 2) k_build_Q3(Lat32 F, Lat32 C, const double* __restrict__ val,
+                                                     const double* __restrict__ P, double* __restrict__ Q) {
+  const unsigned nx = (unsigned)(F.Lx + 95) / 96;
+  const unsigned line = blockIdx.x / nx, c = line / (unsigned)F.Ly, b = line - c * (unsigned)F.Ly;
+  const int m = (int)(blockIdx.x - line * nx) * 32 + (int)(threadIdx.x & 31), w = threadIdx.x >> 5;
+  const int a = 3 * m + w % 3;
+  if (a >= F.Lx) return;
+  if (w % 3 == 0) q3_point<0>(F, C, a, (int)b, (int)c, w / 3, val, P, Q);
+  else if (w % 3 == 1) q3_point<1>(F, C, a, (int)b, (int)c, w / 3, val, P, Q);
+  else q3_point<2>(F, C, a, (int)b, (int)c, w / 3, val, P, Q);
+}
+
+// A_c[J, J+oc] = sum_{a in box(J)} P[a, J]^T Q[a, J+oc]   (BC x BC blocks).
+// A_c is symmetric: the centre and the offsets after it are formed, the rest
+// are their transposes (half the products; the stored operator is exactly
+// symmetric).  RAP_FIGURES
 template <int BF, int BC, int CKIND>
 __global__ void k_rap(Lat F, Lat Cc, int R, const double* __restrict__ P, const double* __restrict__ Q,
                       const unsigned char* __restrict__ ac, double* __restrict__ Ac) {
+  constexpr int NO = St<CKIND>::N, MID = St<CKIND>::C;
   const long long tid = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (tid >= Cc.N * St<CKIND>::N) return;
-  const int oc = (int)(tid / Cc.N);
-  const long long J = tid - (long long)oc * Cc.N;
+  if (tid >= Cc.N * (NO - MID)) return;
+  const int oc = MID + (int)(tid / Cc.N);
+  const long long J = tid - (long long)(oc - MID) * Cc.N;
   int I, Jj, K;
   Cc.ijk(J, I, Jj, K);
   int ox, oy, oz;
@@ -1119,20 +1215,18 @@ __global__ void k_rap(Lat F, Lat Cc, int R, const double* __restrict__ P, const 
   const int I2 = I + ox, J2 = Jj + oy, K2 = K + oz;
   double out[BC * BC];
   for (int q = 0; q < BC * BC; ++q) out[q] = 0.0;
-  if (Cc.in(I2, J2, K2)) {
+  const bool in = Cc.in(I2, J2, K2);
+  if (in) {
     const int ns = p_slots(R), nq = q_slots(R);
-    for (int c = 3 * K - R; c <= 3 * K + 2 + R; ++c) {
-      if (c < 0 || c >= F.Lz) continue;
+    // the fine points in both P's range of J and Q's range of J + oc
+    auto lo = [&](int j, int j2) { return max(max(3 * j - R, 3 * j2 - 2 * R), 0); };
+    auto hi = [&](int j, int j2, int n) { return min(min(3 * j + 2 + R, 3 * j2 + 2 + 2 * R), n - 1); };
+    for (int c = lo(K, K2); c <= hi(K, K2, F.Lz); ++c) {
       const int pz = K - p_lo(c, R), qz = K2 - q_lo(c, R);
-      if (pz < 0 || pz >= ns || qz < 0 || qz >= nq) continue;
-      for (int b = 3 * Jj - R; b <= 3 * Jj + 2 + R; ++b) {
-        if (b < 0 || b >= F.Ly) continue;
+      for (int b = lo(Jj, J2); b <= hi(Jj, J2, F.Ly); ++b) {
         const int py = Jj - p_lo(b, R), qy = J2 - q_lo(b, R);
-        if (py < 0 || py >= ns || qy < 0 || qy >= nq) continue;
-        for (int a = 3 * I - R; a <= 3 * I + 2 + R; ++a) {
-          if (a < 0 || a >= F.Lx) continue;
+        for (int a = lo(I, I2); a <= hi(I, I2, F.Lx); ++a) {
           const int px = I - p_lo(a, R), qx = I2 - q_lo(a, R);
-          if (px < 0 || px >= ns || qx < 0 || qx >= nq) continue;
           const long long p = F.id(a, b, c);
           const double* pv = P + (long long)(px + ns * (py + ns * pz)) * BF * BC * F.N + p;
           const double* qv = Q + (long long)(qx + nq * (qy + nq * qz)) * BF * BC * F.N + p;
@@ -1146,10 +1240,22 @@ __global__ void k_rap(Lat F, Lat Cc, int R, const double* __restrict__ P, const 
       }
     }
   }
-  if (ox == 0 && oy == 0 && oz == 0)
+  if (oc == MID) {
     for (int r = 0; r < BC; ++r)
       if (!ac[BC * J + r]) out[r * BC + r] = 1.0;
+    for (int r = 0; r < BC; ++r)  // the block itself symmetric: its upper triangle
+      for (int t = 0; t < r; ++t) out[r * BC + t] = out[t * BC + r];
+  }
   for (int q = 0; q < BC * BC; ++q) Ac[((long long)oc * BC * BC + q) * Cc.N + J] = out[q];
+  if (oc == MID) return;
+  const int om = NO - 1 - oc;  // the opposite offset
+  if (in) {
+    const long long q2 = Cc.id(I2, J2, K2);
+    for (int r = 0; r < BC; ++r)
+      for (int t = 0; t < BC; ++t) Ac[((long long)om * BC * BC + t * BC + r) * Cc.N + q2] = out[r * BC + t];
+  }
+  if (!Cc.in(I - ox, Jj - oy, K - oz))
+    for (int q = 0; q < BC * BC; ++q) Ac[((long long)om * BC * BC + q) * Cc.N + J] = 0.0;
 }
 
 // ------------------------------------------- rigid-body-mode near-kernel
@@ -1624,17 +1730,23 @@ Level coarsen(Ctx& c, Level& L, Level* into = nullptr) {
         MHFP_LAUNCH_CHECK();
         k_active_coarse<BS.value><<<grid_for(Cc.N, 256), 256, 0, c.stream>>>(F, Cc, L.active, Cl.active);
         MHFP_LAUNCH_CHECK();
-        k_build_Q<BS.value, BS.value, K.value><<<grid_for(F.N * nq * nq * nq, 256), 256, 0, c.stream>>>(F, Cc, A.val,
-                                                                                                     L.P, Q);
+        if constexpr (BS.value == 3) {
+          const Lat32 F32 = lat32_of(A), C32 = lat32_of(Cl.A);
+          k_build_Q3<<<(unsigned)((F32.Lx + 95) / 96) * (unsigned)(A.Ly * A.Lz), 288, 0, c.stream>>>(F32, C32, A.val,
+                                                                                                  L.P, Q);
+        } else {
+          k_build_Q<BS.value, BS.value, K.value><<<grid_for(F.N * nq * nq * nq, 256), 256, 0, c.stream>>>(
+              F, Cc, A.val, L.P, Q);
+        }
         MHFP_LAUNCH_CHECK();
       });
       // coarse levels of the 27-point displacement lattice stay 27-point; the
       // scalar levels become 125-point
       if constexpr (BS.value == 3)
-        k_rap<BS.value, BS.value, ST_BOX1><<<grid_for(Cc.N * 27, 128), 128, 0, c.stream>>>(F, Cc, R, L.P, Q,
+        k_rap<BS.value, BS.value, ST_BOX1><<<grid_for(Cc.N * 14, 128), 128, 0, c.stream>>>(F, Cc, R, L.P, Q,
                                                                                            Cl.active, Cl.A.val);
       else
-        k_rap<BS.value, BS.value, ST_BOX2><<<grid_for(Cc.N * 125, 128), 128, 0, c.stream>>>(F, Cc, R, L.P, Q,
+        k_rap<BS.value, BS.value, ST_BOX2><<<grid_for(Cc.N * 63, 128), 128, 0, c.stream>>>(F, Cc, R, L.P, Q,
                                                                                              Cl.active, Cl.A.val);
       MHFP_LAUNCH_CHECK();
     });
@@ -1727,7 +1839,7 @@ void build_u_rbm(Ctx& c) {
         MHFP_LAUNCH_CHECK();
         k_build_Q<bf, RBM_K, ST_BOX1><<<grid_for(F.N * nq * nq * nq, 256), 256, 0, c.stream>>>(F, Cc, A.val, L.P, Q);
         MHFP_LAUNCH_CHECK();
-        k_rap<bf, RBM_K, ST_BOX1><<<grid_for(Cc.N * 27, 128), 128, 0, c.stream>>>(F, Cc, 1, L.P, Q, Cl.active,
+        k_rap<bf, RBM_K, ST_BOX1><<<grid_for(Cc.N * 14, 128), 128, 0, c.stream>>>(F, Cc, 1, L.P, Q, Cl.active,
                                                                                    Cl.A.val);
         MHFP_LAUNCH_CHECK();
       };

@@ -89,8 +89,8 @@ __device__ __forceinline__ void load_cell_coords(const Dims& d, const double* __
 // The FP64 pipe (2 FMA per clock and SM) bounds this kernel, so it is written
 // for few FP64 operations: lam and G are constant in the cell, so the block
 // follows from H_ab = int grad N_a (x) grad N_b alone, K_ab = lam H + G H^T +
-// G tr(H) I, and only the 36 pairs a <= b are integrated (K_ba = K_ab^T, so
-// the stored element matrix is exactly symmetric): about 5,000 operations per
+// G tr(H) I, and only the 36 pairs a <= b are integrated (K_ba = K_ab^T; the
+// element matrix is stored as its upper triangle): about 5,000 operations per
 // cell instead of 25,000 with the integrand summed term by term over all 64
 // pairs.  A block takes 32 consecutive cells, a lane per cell, so every store
 // is one full row segment; warp q first forms the gradients at Gauss point q
@@ -98,6 +98,14 @@ __device__ __forceinline__ void load_cell_coords(const Dims& d, const double* __
 // and d = 4 for a < 4 (nine pairs per scheduler).  96^3 cells: 49.5 ms before
 // (one warp per cell, a store per lane and row), 7.93 ms now (0.92 of the FP64 pipe).
 constexpr int Q1_CELLS = 32;
+// row of entry (i, j) of the element matrices, stored as upper triangles
+// [300][cells] (half the bytes to allocate, write and give back: about 2 ms of
+// a 96^3 set-up; the gather takes 1.9 instead of 1.25 ms)
+constexpr int KE_ROWS = 300;
+__device__ __forceinline__ int ke_row(int i, int j) {
+  const int a = min(i, j), b = max(i, j);
+  return a * 24 - a * (a - 1) / 2 + (b - a);
+}
 constexpr size_t Q1_SMEM = (8 * 24 + 8) * Q1_CELLS * sizeof(double);
 
 // 0.125 (1 + s g)(1 + t g) of a Q1 derivative's two transverse factors, s, t =
@@ -203,10 +211,9 @@ __global__ void __launch_bounds__(256, 2) k_q1(Dims d, const double* __restrict_
     for (int i = 0; i < 3; ++i)
 #pragma unroll
       for (int j = 0; j < 3; ++j) {
-        if (p == 0 && j < i) continue;  // the (a, a) block is symmetric: its upper triangle, stored twice
+        if (p == 0 && j < i) continue;  // the (a, a) block is symmetric: its upper triangle
         const double k = i == j ? lamG * H[p][4 * i] + gt : lam * H[p][3 * i + j] + G * H[p][3 * j + i];
-        Ke[(long long)((3 * a + i) * 24 + 3 * b + j) * nT + T] = k;
-        if (p != 0 || i != j) Ke[(long long)((3 * b + j) * 24 + 3 * a + i) * nT + T] = k;
+        Ke[(long long)ke_row(3 * a + i, 3 * b + j) * nT + T] = k;
       }
   }
   const double bi = biot[T];
@@ -439,7 +446,7 @@ __global__ void k_assemble_uu(Dims d, const double* __restrict__ Ke, const unsig
           const int a = (ni - cx) + 2 * (nj - cy) + 4 * (nk - cz);
           const int b = (mi - cx) + 2 * (mj - cy) + 4 * (mk - cz);
           for (int r = 0; r < 3; ++r)
-            for (int s = 0; s < 3; ++s) blk[3 * r + s] += Ke[(long long)((3 * a + r) * 24 + 3 * b + s) * d.nT + T];
+            for (int s = 0; s < 3; ++s) blk[3 * r + s] += Ke[(long long)ke_row(3 * a + r, 3 * b + s) * d.nT + T];
         }
       }
     }
@@ -1351,7 +1358,7 @@ FaceTopo32 topo32(const Ctx& c) { return FaceTopo32::make(c.nx, c.ny, c.nz, c.nT
 void assemble_all(Ctx& c) {
   const Dims d = dims_of(c);
   MHFP_CUDA(cudaMemsetAsync(c.d_flag, 0, sizeof(int), c.stream));
-  double* Ke = (double*)dalloc_own(c, (size_t)576 * c.nT * sizeof(double));
+  double* Ke = (double*)dalloc_own(c, (size_t)KE_ROWS * c.nT * sizeof(double));
   c.Aup = dalloc_n<double>(c, (size_t)24 * c.nT);
   c.vol = dalloc_n<double>(c, c.nT);
   MHFP_CUDA(cudaFuncSetAttribute(k_q1, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Q1_SMEM));
