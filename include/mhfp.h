@@ -97,8 +97,9 @@ typedef struct {
                         /* 0: kernels are launched one by one                  */
   int autotune;         /* 1 (default): time the launch schedules of each      */
                         /* coarse level's smoother at set-up (one point per    */
-                        /* thread, or the stencil offsets split over 4, 8 or   */
-                        /* 16 warps) and the two occupancy variants of the     */
+                        /* thread, the stencil offsets split over 4, 8 or 16   */
+                        /* warps, or a warp or eight lanes per point on row-   */
+                        /* major values) and the two occupancy variants of the */
                         /* finest FP32 displacement sweep, and keep the        */
                         /* fastest (schedule only: the same products, summed   */
                         /* in a schedule-dependent fixed order)                */
@@ -160,7 +161,8 @@ typedef struct {
   double lmax[8];       /* 1.1 * rho(D^-1 A) per level (0 on the last level)   */
   int schedule[8];      /* launch schedule of the level's sweeps: 1 = one point */
                         /* per thread, 4/8/16 = offsets split over that many    */
-                        /* warps; finest FP32 displacement level: fine_blocks  */
+                        /* warps, 32/64 = a warp / eight lanes per point on     */
+                        /* row-major values (small levels); finest FP32 displacement level: fine_blocks  */
                         /* (4, 6 or 8); 0 = not a lattice sweep                */
   double sweep_us[8];   /* set-up autotuner's time of one sweep under that     */
                         /* schedule, microseconds (0 when not timed)           */

@@ -1478,19 +1478,20 @@ FaceTopo32 face_topo(const Ctx& c) {
 
 // y = b - A x (y = A x when b is null) on a lattice level with schedule sched
 template <typename T>
-void launch_spmv(Ctx& c, const StructOp& A, int bs, const T* val, const T* x, const T* b, T* y, int sched) {
-  sweep_spmv<T>(c.stream, A, bs, val, x, b, y, sched);
+void launch_spmv(Ctx& c, const StructOp& A, int bs, const T* val, const T* rows, const T* x, const T* b, T* y,
+                 int sched) {
+  sweep_spmv<T>(c.stream, A, bs, val, rows, x, b, y, sched);
 }
 
 void level_spmv(Ctx& c, Level& L, const double* x, const double* b, double* y) {
   if (L.faces) {
     k_spmv_ell<double><<<lgrid(grid_for(L.n, 256)), 256, 0, c.stream>>>(face_topo(c), L.ell ? L.ell : c.Cpi, x, b, y,
                                                                          lbytes());
-  } else if (L.bs == 3) {
+  } else if (L.bs == 3 && !L.rowd) {
     launch_u64(c.stream, lat32_of(L.A), (const double*)L.A.val, (const double*)nullptr, 0.0, x,
                (const double*)nullptr, b, y);
   } else {
-    launch_spmv<double>(c, L.A, L.bs, L.A.val, x, b, y, default_schedule(L.A.N, L.bs));
+    launch_spmv<double>(c, L.A, L.bs, L.A.val, L.rowd, x, b, y, default_schedule(L.A, L.rowd != nullptr));
   }
   MHFP_LAUNCH_CHECK();
 }
@@ -1675,6 +1676,11 @@ void finish_level(Ctx& c, Level& L) {
     });
   }
   MHFP_LAUNCH_CHECK();
+  if (!L.faces && row_level(L.A)) {
+    if (!L.rowd) L.rowd = dalloc_n<double>(c, sweep_row_elems<double>(L.A, L.bs));
+    sweep_pack_rows<double>(c.stream, L.A, L.bs, L.A.val, L.rowd);
+    MHFP_LAUNCH_CHECK();
+  }
   L.lmax = 1.1 * spectral_radius(c, L);
 }
 
@@ -1944,13 +1950,13 @@ void make_fp64_transfers(Ctx& c, std::vector<Level>& H) {
 // built by the set-up, or their FP32 copies for the mixed-precision cycle.
 template <typename T>
 struct LV {
-  const T *val, *dinv, *P, *Pm, *ell, *pw;  // P: coarse-point major, Pm: fine-point major
+  const T *val, *rows, *dinv, *P, *Pm, *ell, *pw;  // P: coarse-point major, Pm: fine-point major
   T *r, *d, *y;
 };
 LV<double> view(Ctx& c, Level& L, double) {
-  return {L.A.val, L.dinv, L.Pd, L.P, L.ell ? L.ell : c.Cpi, c.pw, L.r, L.d, L.y};
+  return {L.A.val, L.rowd, L.dinv, L.Pd, L.P, L.ell ? L.ell : c.Cpi, c.pw, L.r, L.d, L.y};
 }
-LV<float> view(Ctx& c, Level& L, float) { return {L.valf, L.dinvf, L.Pf, L.Pmf, c.Cpif, c.pwf, L.rf, L.df, L.yf}; }
+LV<float> view(Ctx& c, Level& L, float) { return {L.valf, L.rowf, L.dinvf, L.Pf, L.Pmf, c.Cpif, c.pwf, L.rf, L.df, L.yf}; }
 double* bvec(Level& L, double) { return L.b; }
 float* bvec(Level& L, float) { return L.bf; }
 double* xvec(Level& L, double) { return L.x; }
@@ -1962,7 +1968,7 @@ void level_spmv_t(Ctx& c, Level& L, const T* x, const T* b, T* y) {
   if (L.faces) {
     k_spmv_ell<T><<<lgrid(grid_for(L.n, 256)), 256, 0, c.stream>>>(face_topo(c), v.ell, x, b, y, lbytes());
   } else {
-    launch_spmv<T>(c, L.A, L.bs, v.val, x, b, y, L.tpp ? L.tpp : default_schedule(L.A.N, L.bs));
+    launch_spmv<T>(c, L.A, L.bs, v.val, v.rows, x, b, y, L.tpp ? L.tpp : default_schedule(L.A, v.rows != nullptr));
   }
   MHFP_LAUNCH_CHECK();
 }
@@ -1975,7 +1981,7 @@ void launch_cheb(Ctx& c, Level& L, const LV<T>& v, const T* b, const T* xin, T* 
     sweep_cheb_zero<T>(c.stream, L.A.N, L.bs, v.dinv, b, out, v.d, cr);
     return;
   }
-  sweep_cheb<T>(c.stream, L.A, L.bs, v.val, v.dinv, b, xin, out, v.d, cd, cr, sched);
+  sweep_cheb<T>(c.stream, L.A, L.bs, v.val, v.rows, v.dinv, b, xin, out, v.d, cd, cr, sched);
 }
 
 // The symmetric FP32 sweep and residual of the finest displacement level
@@ -2148,8 +2154,10 @@ void autotune_level(Ctx& c, Level& L) {
   MHFP_CUDA(cudaMemsetAsync(x, 0, L.n * sizeof(T), c.stream));
   MHFP_CUDA(cudaMemsetAsync(v.d, 0, L.n * sizeof(T), c.stream));
   float best = 1e30f;
-  int best_tpp = default_schedule(L.A.N, L.bs);
-  for (int tpp : {1, 4, 8, 16}) {
+  int best_tpp = default_schedule(L.A, v.rows != nullptr);
+  // likely winners first: a candidate that has lost is dropped early
+  const std::vector<int> cand = v.rows ? std::vector<int>{32, 64, 8, 4, 16} : std::vector<int>{1, 4, 8, 16};
+  for (int tpp : cand) {
     const float us = graph_time_us(c, tune_reps((double)sizeof(T) * L.A.noff() * L.bs * L.bs * L.A.N), best, [&] {
       launch_cheb<T>(c, L, v, b, x, v.y, T(0.5), T(0.5), tpp);
       MHFP_LAUNCH_CHECK();
@@ -2221,7 +2229,7 @@ void smooth(Ctx& c, std::vector<Level>& H, int l, const T* b, const T* x0, T* ds
               lat, v.val, v.dinv, b, xin, out, v.d, cd, cr, lbytes());
       }
     } else {
-      launch_cheb<T>(c, L, v, b, xin, out, (T)cd, (T)cr, L.tpp ? L.tpp : default_schedule(L.A.N, L.bs));
+      launch_cheb<T>(c, L, v, b, xin, out, (T)cd, (T)cr, L.tpp ? L.tpp : default_schedule(L.A, v.rows != nullptr));
     }
     MHFP_LAUNCH_CHECK();
     // algorithmic bytes of a Chebyshev sweep: the matrix values (27 blocks
@@ -2341,6 +2349,11 @@ void make_fp32(Ctx& c, std::vector<Level>& H, bool fine_sym) {
       MHFP_LAUNCH_CHECK();
     } else if (!L.faces) {
       L.valf = cast_copy(c, L.A.val, (size_t)L.A.noff() * bs2 * L.A.N);
+      if (L.rowd) {
+        L.rowf = dalloc_n<float>(c, sweep_row_elems<float>(L.A, L.bs));
+        sweep_pack_rows<float>(c.stream, L.A, L.bs, L.valf, L.rowf);
+        MHFP_LAUNCH_CHECK();
+      }
     }
     if (L.dinv) L.dinvf = cast_copy(c, L.dinv, bs2 * L.npts);
     if (L.P) {
@@ -2424,6 +2437,10 @@ void rebuild_pi_hierarchy(Ctx& c) {
       Level& L = H[l];
       const size_t bs2 = (size_t)L.bs * L.bs;
       if (!L.faces && L.valf) recast(L.valf, L.A.val, (size_t)L.A.noff() * bs2 * L.A.N);
+      if (L.rowf) {
+        sweep_pack_rows<float>(c.stream, L.A, L.bs, L.valf, L.rowf);
+        MHFP_LAUNCH_CHECK();
+      }
       if (L.dinv && L.dinvf) recast(L.dinvf, L.dinv, bs2 * L.npts);
       if (L.P && L.Pf) pack_P<float>(c, L, H[l + 1], L.Pf);
     }
@@ -2500,7 +2517,7 @@ void chebyshev_from_zero(Ctx& c, std::vector<Level>& H, const double* b, double*
 int level_schedule(Ctx& c, std::vector<Level>& H, int l) {
   const Level& L = H[l];
   if (&H == &c.hu && l == 0) return L.symf ? sym_minb(L) : 0;  // FP64: the full-storage k_cheb_u0
-  return L.tpp ? L.tpp : default_schedule(L.A.N, L.bs);
+  return L.tpp ? L.tpp : default_schedule(L.A, (c.opt.precision == 1 ? (void*)L.rowf : (void*)L.rowd) != nullptr);
 }
 
 // timed as class 4 (displacement) or 5 (interface pressure)

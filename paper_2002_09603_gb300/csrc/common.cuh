@@ -387,7 +387,7 @@ struct Level {
   const double* ell = nullptr; // face level: its ELL values (null: C~_pi)
   int tpp = 0;                // launch schedule chosen by the autotuner (0: default rule):
                               // 1 = one point per thread, 4/8/16 = warps splitting the
-                              // offsets; finest FP32 displacement level: blocks per SM (6, 8)
+                              // offsets, 32/64 = a warp / eight lanes per point; finest FP32 displacement level: blocks per SM (6, 8)
   unsigned char* active = nullptr;  // [n] free dofs
   // work vectors of length n
   double *x = nullptr, *b = nullptr, *r = nullptr, *d = nullptr, *y = nullptr;
@@ -396,6 +396,8 @@ struct Level {
   // FP32 copies for the mixed-precision cycle (precision == 1)
   float *valf = nullptr, *dinvf = nullptr, *Pf = nullptr, *Pmf = nullptr;
   float* symf = nullptr;      // finest displacement level, FP32: symmetric half, node blocks of 32 x 126 rows
+  double* rowd = nullptr;     // row-major copies of the values (small box levels), FP64 and FP32
+  float* rowf = nullptr;
   double sweep_us = 0.0;      // autotuner's time of one sweep under the chosen schedule
   float *xf = nullptr, *bf = nullptr, *rf = nullptr, *df = nullptr, *yf = nullptr;
 };

@@ -176,10 +176,29 @@ inline Lat32 lat32_of(const StructOp& A) {
 }
 
 // Launch schedule of a level's sweeps and residuals: 1 = one point per
-// thread, W = 4, 8, 16 = warp-split offsets over W warps.  The set-up
-// autotuner times all four; without it, scalar levels of 64K points and up
-// take one point per thread and the others eight warps.
-inline int default_schedule(long long npts, int bs) { return (bs == 1 && npts >= 65536) ? 1 : 8; }
+// thread, W = 4, 8, 16 = warp-split offsets over W warps, 32 and 64 = a warp,
+// or eight lanes, per point on row-major values, which box levels have up to
+// the size where a split schedule is as fast (row_level).  The set-up
+// autotuner times all that apply.  Without it: row-major levels take a warp
+// per point up to 2,048 points and eight lanes above (27-point 3 x 3 levels
+// eight warps), other scalar levels of 64K points and up one point per thread
+// and the rest eight warps.  Microseconds of a Chebyshev step, best split /
+// warp per point / eight lanes:
+//   125-point FP32:  1,000 5.1 / 2.0 / 2.4; 10,648 5.8 / 4.5 / 3.6; 32,768 6.4 / 10 / 7.1
+//   125-point FP64:  1,000 11.6 / 2.7 / 3.5; 10,648 15.3 / 11.6 / 6.0; 32,768 19 / 32 / 14
+//   3 x 3 FP32:      1,000 2.9 / 2.0 / 4.0;  3,375 3.1 / 2.7 / 4.2;   10,648 4.2 / 5.2 / 5.4
+//   3 x 3 FP64:      343 5.8 / 3.2 / 5.2;    3,375 6.2 / 9.2 / 6.2
+//   6 x 6 FP32:      216 6.0 / 3.0 / 7.6;    4,096 8.4 / 4.7 / 8.4;   10,648 9.3 / 8.3 / 9.7
+//   6 x 6 FP64:      216 14.9 / 5.3 / 9.2;   4,096 15.9 / 22 / 13.4
+inline bool row_level(const StructOp& A) {
+  if (A.kind == ST_DIAMOND2) return false;
+  return A.N <= (A.bs == 1 ? 32768 : (A.bs == 3 ? 4096 : 16384));
+}
+inline int row_lanes(int sched) { return sched == 32 ? 32 : (sched == 64 ? 8 : 0); }
+inline int default_schedule(const StructOp& A, bool rows) {
+  if (rows) return A.N <= 2048 ? 32 : (A.bs == 3 ? 8 : 64);
+  return (A.bs == 1 && A.N >= 65536) ? 1 : 8;
+}
 
 template <class F>
 void dispatch_sched(int sched, F&& f) {
@@ -197,11 +216,16 @@ void dispatch_sched(int sched, F&& f) {
 // Chebyshev step from x = 0 (no stencil work).  They queue one kernel on
 // `stream` and do not check or count it: the caller does.
 template <typename T>
-void sweep_spmv(cudaStream_t stream, const StructOp& A, int bs, const T* val, const T* x, const T* b, T* y,
-                int sched);
+void sweep_spmv(cudaStream_t stream, const StructOp& A, int bs, const T* val, const T* rows, const T* x, const T* b,
+                T* y, int sched);
 template <typename T>
-void sweep_cheb(cudaStream_t stream, const StructOp& A, int bs, const T* val, const T* dinv, const T* b,
+void sweep_cheb(cudaStream_t stream, const StructOp& A, int bs, const T* val, const T* rows, const T* dinv, const T* b,
                 const T* xin, T* out, T* d, T cd, T cr, int sched);
+// row-major copy of a level's values (schedules 32 and 64; null: none)
+template <typename T>
+size_t sweep_row_elems(const StructOp& A, int bs);
+template <typename T>
+void sweep_pack_rows(cudaStream_t stream, const StructOp& A, int bs, const T* val, T* rows);
 template <typename T>
 void sweep_cheb_zero(cudaStream_t stream, long long npts, int bs, const T* dinv, const T* b, T* out, T* d, T cr);
 

@@ -204,12 +204,161 @@ __global__ void __launch_bounds__(32 * W) k_cheb_w(Lat32 L, const T* __restrict_
   cheb_update<T, BS>(p, (unsigned)L.N, r, dinv, xin, xout, d, cd, cr);
 }
 
+// Row-major levels: LPP lanes per point on values Ar[point][row a][PP], the
+// NO x BS (offset, component) pairs of a row padded to PP = a multiple of 32
+// (zeros).  On levels of up to some ten thousand points the split kernels
+// above are bound by the latency of their serial chunks; here every load of a
+// row is issued at once and consecutive lanes read consecutive values, and the
+// sums meet in a fixed-order xor reduction (sizes and times: default_schedule).
+template <int BS, int KIND>
+constexpr int row_pairs() { return Sf<KIND>::N * BS; }
+template <int BS, int KIND>
+constexpr int row_pad() { return (row_pairs<BS, KIND>() + 31) / 32 * 32; }
+
+template <int BS, int KIND>
+__device__ __forceinline__ void pair_of(int e, int& dx, int& dy, int& dz, int& s) {
+  static_assert(KIND != ST_DIAMOND2, "row-major levels are 27- or 125-point boxes");
+  constexpr int w = KIND == ST_BOX1 ? 3 : 5, R = w / 2;
+  const int o = e / BS;
+  s = e - o * BS;
+  dx = o % w - R;
+  dy = (o / w) % w - R;
+  dz = o / (w * w) - R;
+}
+
+// r = A x at point p (the same in each of the point's LPP lanes)
+template <int BS, int KIND, int LPP, typename T>
+__device__ __forceinline__ void row_product(const Lat32& L, unsigned p, const T* __restrict__ Ar,
+                                            const T* __restrict__ x, T r[BS]) {
+  constexpr int PP = row_pad<BS, KIND>(), NP = row_pairs<BS, KIND>(), PER = PP / LPP;
+  constexpr int CH = PER <= 8 ? PER : (PER % 8 == 0 ? 8 : 6);  // pairs in flight per lane
+  static_assert(PP % LPP == 0 && PER % CH == 0, "chunks cover the padded row exactly");
+  const int l = threadIdx.x % LPP;
+  int i, j, k;
+  L.ijk(p, i, j, k);
+#pragma unroll
+  for (int a = 0; a < BS; ++a) r[a] = T(0);
+  const T* row = Ar + (size_t)p * (BS * PP) + l;
+#pragma unroll
+  for (int c0 = 0; c0 < PER; c0 += CH) {
+    T av[CH][BS], xv[CH];
+#pragma unroll
+    for (int c = 0; c < CH; ++c) {
+      const int e = l + LPP * (c0 + c);
+      int dx, dy, dz, s;
+      pair_of<BS, KIND>(e, dx, dy, dz, s);
+      const bool in = e < NP && (unsigned)(i + dx) < (unsigned)L.Lx && (unsigned)(j + dy) < (unsigned)L.Ly &&
+                      (unsigned)(k + dz) < (unsigned)L.Lz;
+      const unsigned q = in ? p + (unsigned)(dx + L.Lx * dy + L.LxLy * dz) : p;
+      const T v = x[BS * q + (in ? s : 0)];
+      xv[c] = in ? v : T(0);
+#pragma unroll
+      for (int a = 0; a < BS; ++a) av[c][a] = row[a * PP + LPP * (c0 + c)];
+    }
+#pragma unroll
+    for (int c = 0; c < CH; ++c)
+#pragma unroll
+      for (int a = 0; a < BS; ++a) r[a] += av[c][a] * xv[c];
+  }
+#pragma unroll
+  for (int a = 0; a < BS; ++a)
+#pragma unroll
+    for (int m = LPP / 2; m > 0; m >>= 1) r[a] += __shfl_xor_sync(0xffffffffu, r[a], m);
+}
+
+template <int BS, typename T>
+__device__ __forceinline__ T pick(const T v[BS], int a) {
+  T s = v[0];
+#pragma unroll
+  for (int q = 1; q < BS; ++q) s = a == q ? v[q] : s;
+  return s;
+}
+
+template <int BS, int KIND, int LPP, typename T>
+__global__ void __launch_bounds__(128) k_spmv_r(Lat32 L, const T* __restrict__ Ar, const T* __restrict__ x,
+                                                const T* __restrict__ b, T* __restrict__ y, long long lb) {
+  x = lane_ptr(x, lb);
+  b = lane_ptr(b, lb);
+  y = lane_ptr(y, lb);
+  const unsigned p0 = (blockIdx.x * 128 + threadIdx.x) / LPP;
+  const unsigned p = p0 < (unsigned)L.N ? p0 : (unsigned)L.N - 1;  // the whole warp takes part in the reduction
+  const int a = threadIdx.x % LPP;
+  T r[BS];
+  row_product<BS, KIND, LPP, T>(L, p, Ar, x, r);
+  if (p0 >= (unsigned)L.N || a >= BS) return;
+  const T v = pick<BS, T>(r, a);
+  y[BS * p + a] = b ? b[BS * p + a] - v : v;
+}
+
+template <int BS, int KIND, int LPP, typename T>
+__global__ void __launch_bounds__(128) k_cheb_r(Lat32 L, const T* __restrict__ Ar, const T* __restrict__ dinv,
+                                                const T* __restrict__ b, const T* __restrict__ xin,
+                                                T* __restrict__ xout, T* __restrict__ d, T cd, T cr, long long lb) {
+  b = lane_ptr(b, lb);
+  xin = lane_ptr(xin, lb);
+  xout = lane_ptr(xout, lb);
+  d = lane_ptr(d, lb);
+  const unsigned p0 = (blockIdx.x * 128 + threadIdx.x) / LPP;
+  const unsigned p = p0 < (unsigned)L.N ? p0 : (unsigned)L.N - 1;
+  const int a = threadIdx.x % LPP;
+  // lane a's row of D^-1 and its vector entries, in flight with the stencil's
+  T di[BS], bv[BS], dv = T(0), xv = T(0);
+  const int ac = a < BS ? a : 0;
+#pragma unroll
+  for (int t = 0; t < BS; ++t) {
+    di[t] = dinv[(ac * BS + t) * (unsigned)L.N + p];
+    bv[t] = b[BS * p + t];
+  }
+  if (cd != T(0)) dv = d[BS * p + ac];
+  xv = xin[BS * p + ac];
+  T r[BS];
+  row_product<BS, KIND, LPP, T>(L, p, Ar, xin, r);
+  if (p0 >= (unsigned)L.N || a >= BS) return;
+  T z = T(0);
+#pragma unroll
+  for (int t = 0; t < BS; ++t) z += di[t] * (bv[t] - r[t]);
+  const T dn = (cd != T(0)) ? cd * dv + cr * z : cr * z;
+  d[BS * p + a] = dn;
+  xout[BS * p + a] = xv + dn;
+}
+
+// offset-major values into the row-major layout: a thread per value
+template <int BS, int KIND, typename T>
+__global__ void __launch_bounds__(256) k_pack_rows(long long N, const T* __restrict__ val, T* __restrict__ Ar) {
+  constexpr int PP = row_pad<BS, KIND>(), NP = row_pairs<BS, KIND>();
+  const long long t = (long long)blockIdx.x * 256 + threadIdx.x;
+  if (t >= N * BS * PP) return;
+  const int e = (int)(t % PP), a = (int)((t / PP) % BS);
+  const long long p = t / (BS * PP);
+  const int o = e / BS, s = e - o * BS;
+  Ar[t] = e < NP ? val[(long long)(o * BS * BS + a * BS + s) * N + p] : T(0);
+}
+
 }  // namespace
 
+// the row-major kernels' block sizes and kinds
+template <class F>
+void dispatch_rows(int bs, int kind, int lpp, F&& f) {
+  auto with = [&](auto BS, auto K) {
+    if (lpp == 8) f(BS, K, std::integral_constant<int, 8>{});
+    else f(BS, K, std::integral_constant<int, 32>{});
+  };
+  if (bs == 3) with(std::integral_constant<int, 3>{}, std::integral_constant<int, ST_BOX1>{});
+  else if (bs == 6) with(std::integral_constant<int, 6>{}, std::integral_constant<int, ST_BOX1>{});
+  else with(std::integral_constant<int, 1>{}, std::integral_constant<int, ST_BOX2>{});
+}
+
 template <typename T>
-void sweep_spmv(cudaStream_t stream, const StructOp& A, int bs, const T* val, const T* x, const T* b, T* y,
-                int sched) {
+void sweep_spmv(cudaStream_t stream, const StructOp& A, int bs, const T* val, const T* rows, const T* x, const T* b,
+                T* y, int sched) {
   const Lat32 L = lat32_of(A);
+  if (const int lpp = rows ? row_lanes(sched) : 0) {
+    dispatch_rows(bs, A.kind, lpp, [&](auto BS, auto K, auto LPP) {
+      k_spmv_r<BS.value, K.value, LPP.value, T><<<lgrid(grid_for(A.N * LPP.value, 128)), 128, 0, stream>>>(
+          L, rows, x, b, y, lbytes());
+    });
+    return;
+  }
   dispatch_bs(bs, [&](auto BS) {
     dispatch_kind_bs<BS.value>(A.kind, [&](auto K) {
       dispatch_sched(sched, [&](auto S) {
@@ -224,9 +373,16 @@ void sweep_spmv(cudaStream_t stream, const StructOp& A, int bs, const T* val, co
 }
 
 template <typename T>
-void sweep_cheb(cudaStream_t stream, const StructOp& A, int bs, const T* val, const T* dinv, const T* b,
+void sweep_cheb(cudaStream_t stream, const StructOp& A, int bs, const T* val, const T* rows, const T* dinv, const T* b,
                 const T* xin, T* out, T* d, T cd, T cr, int sched) {
   const Lat32 lat = lat32_of(A);
+  if (const int lpp = rows ? row_lanes(sched) : 0) {
+    dispatch_rows(bs, A.kind, lpp, [&](auto BS, auto K, auto LPP) {
+      k_cheb_r<BS.value, K.value, LPP.value, T><<<lgrid(grid_for(A.N * LPP.value, 128)), 128, 0, stream>>>(
+          lat, rows, dinv, b, xin, out, d, cd, cr, lbytes());
+    });
+    return;
+  }
   dispatch_bs(bs, [&](auto BS) {
     dispatch_kind_bs<BS.value>(A.kind, [&](auto K) {
       dispatch_sched(sched, [&](auto S) {
@@ -242,6 +398,20 @@ void sweep_cheb(cudaStream_t stream, const StructOp& A, int bs, const T* val, co
 }
 
 template <typename T>
+size_t sweep_row_elems(const StructOp& A, int bs) {
+  size_t n = 0;
+  dispatch_rows(bs, A.kind, 32, [&](auto BS, auto K, auto) { n = (size_t)A.N * BS.value * row_pad<BS.value, K.value>(); });
+  return n;
+}
+
+template <typename T>
+void sweep_pack_rows(cudaStream_t stream, const StructOp& A, int bs, const T* val, T* rows) {
+  dispatch_rows(bs, A.kind, 32, [&](auto BS, auto K, auto) {
+    k_pack_rows<BS.value, K.value, T><<<grid_for((long long)sweep_row_elems<T>(A, bs), 256), 256, 0, stream>>>(A.N, val, rows);
+  });
+}
+
+template <typename T>
 void sweep_cheb_zero(cudaStream_t stream, long long npts, int bs, const T* dinv, const T* b, T* out, T* d, T cr) {
   dispatch_bs(bs, [&](auto BS) {
     k_cheb_zero<BS.value, T><<<lgrid(grid_for(npts, 256)), 256, 0, stream>>>(npts, dinv, b, out, d, cr, lbytes());
@@ -249,10 +419,12 @@ void sweep_cheb_zero(cudaStream_t stream, long long npts, int bs, const T* dinv,
 }
 
 template void sweep_spmv<MHFP_SWEEP_T>(cudaStream_t, const StructOp&, int, const MHFP_SWEEP_T*, const MHFP_SWEEP_T*,
-                                       const MHFP_SWEEP_T*, MHFP_SWEEP_T*, int);
+                                       const MHFP_SWEEP_T*, const MHFP_SWEEP_T*, MHFP_SWEEP_T*, int);
 template void sweep_cheb<MHFP_SWEEP_T>(cudaStream_t, const StructOp&, int, const MHFP_SWEEP_T*, const MHFP_SWEEP_T*,
-                                       const MHFP_SWEEP_T*, const MHFP_SWEEP_T*, MHFP_SWEEP_T*, MHFP_SWEEP_T*,
-                                       MHFP_SWEEP_T, MHFP_SWEEP_T, int);
+                                       const MHFP_SWEEP_T*, const MHFP_SWEEP_T*, const MHFP_SWEEP_T*, MHFP_SWEEP_T*,
+                                       MHFP_SWEEP_T*, MHFP_SWEEP_T, MHFP_SWEEP_T, int);
+template size_t sweep_row_elems<MHFP_SWEEP_T>(const StructOp&, int);
+template void sweep_pack_rows<MHFP_SWEEP_T>(cudaStream_t, const StructOp&, int, const MHFP_SWEEP_T*, MHFP_SWEEP_T*);
 template void sweep_cheb_zero<MHFP_SWEEP_T>(cudaStream_t, long long, int, const MHFP_SWEEP_T*, const MHFP_SWEEP_T*,
                                             MHFP_SWEEP_T*, MHFP_SWEEP_T*, MHFP_SWEEP_T);
 

@@ -132,3 +132,34 @@ def test_float_float_operator_row_families(dims):
         scale = ref[a:b].abs().max()
         assert (y[a:b] - ref[a:b]).abs().max() <= 2.0 ** -38 * scale
     s.close()
+
+
+# row-major sweeps and residuals (a warp or eight lanes per point) as the
+# autotuner and the size rule pick them: box levels of 1 to a few thousand
+# points (a last block that is not full), 1, 3 and 6 unknowns per point
+@pytest.mark.parametrize("near_kernel", [0, 1])
+@pytest.mark.parametrize("precision", [0, 1])
+@pytest.mark.parametrize("dims,autotune", [((12, 10, 4), 0), ((12, 10, 4), 1), ((45, 7, 7), 0)])
+def test_row_major_levels_against_the_oracle(dims, autotune, precision, near_kernel):
+    prob = mi.random_small(*dims, seed=13, jitter=0.15)
+    B = oracle.assemble(prob)
+    from oracle import rbm
+    pc = precond.build(B, "amg_rbm" if near_kernel else "amg", coarse_max=4)
+    s = _solver(prob, autotune=autotune, coarse_max=4, precision=precision, near_kernel=near_kernel)
+    if not autotune:
+        assert 32 in s.hierarchy(0)["schedule"] and 32 in s.hierarchy(1)["schedule"]
+    rng = np.random.default_rng(8)
+    nU, _, nPi = B.sizes
+    tol = 1e-5 if precision else 1e-10
+    for which, n, levels in ((0, nU, pc.u_levels), (1, nPi, pc.pi_levels)):
+        b = rng.standard_normal(n)
+        ref = rbm.vcycle(levels, b) if near_kernel and which == 0 else precond.vcycle(levels, b)
+        got = s.vcycle(which, torch.from_numpy(b).cuda()).cpu().numpy()
+        assert np.abs(got - ref).max() <= tol * np.abs(ref).max()
+    if not precision:
+        for which, levels in ((0, pc.u_levels), (1, pc.pi_levels)):
+            for l, lev in enumerate(levels):
+                x = rng.standard_normal(lev.A.shape[0])
+                y = s.level_apply(which, l, torch.from_numpy(x).cuda()).cpu().numpy()
+                assert np.abs(y - lev.A @ x).max() <= 1e-11 * np.abs(lev.A @ x).max()
+    s.close()
