@@ -186,44 +186,51 @@ struct GsTail {
 // One Arnoldi step's Hessenberg column, by one warp: h = h1 + h2 (j+1
 // entries; h2 null after a single Gram-Schmidt pass), the new subdiagonal
 // ||w|| = sqrt(nrm2); apply the previous rotations, make the new one, update
-// g.  scal[0] = |g_{j+1}|, scal[1] = 1/||w|| (0 on breakdown).  The operands
-// are loaded by the whole warp first: the recurrence itself (2 FP64 steps
-// per rotation) then runs from shared memory.
+// g.  scal[0] = |g_{j+1}|, scal[1] = 1/||w|| (0 on breakdown).
+// The previous rotations are a linear recurrence, a_{i+1} = -s_i a_i + c_i
+// h_{i+1} with a_0 = h_0, of which column entry i is c_i a_i + s_i h_{i+1}: one
+// thread walking it took 0.27 us per rotation (the latency of its FP64
+// chain), so the warp composes the maps a -> M a + K by a scan, 32 at a time.
+// |M| <= 1 throughout.
 __device__ __forceinline__ void givens_step(int j, const GsTail& t, double nrm2) {
-  __shared__ double col[64], c_[64], s_[64];
   const int lane = threadIdx.x & 31;
-  for (int i = lane; i <= j; i += 32) {
-    col[i] = t.h2 ? t.h1[i] + t.h2[i] : t.h1[i];
-    if (i < j) {
-      c_[i] = t.cs[i];
-      s_[i] = t.sn[i];
-    }
-  }
-  const double gj = t.g[j];
-  __syncwarp();
-  if (lane == 0) {
-    const double hn = sqrt(nrm2);
-    double a = col[0];
-    for (int i = 0; i < j; ++i) {
-      const double b = col[i + 1];
-      col[i] = c_[i] * a + s_[i] * b;
-      a = -s_[i] * a + c_[i] * b;
-    }
-    const double den = hypot(a, hn);
-    const double c = den > 0.0 ? a / den : 1.0;
-    const double s = den > 0.0 ? hn / den : 0.0;
-    t.cs[j] = c;
-    t.sn[j] = s;
-    col[j] = den;
-    t.g[j + 1] = -s * gj;
-    t.g[j] = c * gj;
-    t.scal[0] = fabs(s * gj);
-    t.scal[1] = hn > 0.0 ? 1.0 / hn : 0.0;
-  }
-  __syncwarp();
   double* out = t.H + (long long)j * (t.m + 1);
-  for (int i = lane; i <= j; i += 32) out[i] = col[i];
-  if (lane == 0) out[j + 1] = 0.0;
+  auto entry = [&](int i) { return t.h2 ? t.h1[i] + t.h2[i] : t.h1[i]; };
+  const double gj = t.g[j];
+  double a = entry(0);  // a_base, the same in every lane
+  for (int base = 0; base < j; base += 32) {
+    const int i = base + lane;
+    const bool on = i < j;
+    const double c = on ? t.cs[i] : 1.0, s = on ? t.sn[i] : 0.0, h = on ? entry(i + 1) : 0.0;
+    double M = on ? -s : 1.0, K = on ? c * h : 0.0;  // lanes past the column: the identity
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+      const double Mu = __shfl_up_sync(0xffffffffu, M, d), Ku = __shfl_up_sync(0xffffffffu, K, d);
+      if (lane >= d) {
+        K = fma(M, Ku, K);
+        M *= Mu;
+      }
+    }
+    const double next = fma(M, a, K);  // a_{i+1}
+    double ai = __shfl_up_sync(0xffffffffu, next, 1);
+    if (lane == 0) ai = a;
+    if (on) out[i] = c * ai + s * h;
+    a = __shfl_sync(0xffffffffu, next, 31);
+  }
+  // lane 0: the rotation's length, lane 1: ||w||; both with their reciprocal
+  const double len = sqrt(lane == 0 ? fma(a, a, nrm2) : nrm2);
+  const double inv = len > 0.0 ? 1.0 / len : 0.0;
+  const double hn = __shfl_sync(0xffffffffu, len, 1), ihn = __shfl_sync(0xffffffffu, inv, 1);
+  if (lane != 0) return;
+  const double c = len > 0.0 ? a * inv : 1.0, s = len > 0.0 ? hn * inv : 0.0;
+  t.cs[j] = c;
+  t.sn[j] = s;
+  out[j] = len;
+  out[j + 1] = 0.0;
+  t.g[j + 1] = -s * gj;
+  t.g[j] = c * gj;
+  t.scal[0] = fabs(s * gj);
+  t.scal[1] = ihn;
 }
 
 // rows r, r + stride (NR = 2) or r alone (NR = 1): v -= V h, four columns'
@@ -418,13 +425,23 @@ __global__ void k_set_g(int m, double beta, double* __restrict__ g) {
 }
 
 
-// blocks of the Gram-Schmidt kernels: no more than the rows fill
-inline unsigned gs_blocks(long long n, int most) { return std::min<unsigned>(grid_for(n, RED_THREADS), (unsigned)most); }
+// Blocks of the Gram-Schmidt kernels: no more than the rows fill, and fewer
+// on shorter vectors, where the blocks' own reductions and the arrivals at the
+// counter cost more than the rows (microseconds, 13 columns, 152 / 304 / 608
+// blocks: 175,000 rows 10.3 / 12.6 / 16.2 for the dots and 16.4 / 15.9 / 17.6 for
+// the update; 640,000 rows 22.4 / 22.8 / 26.6 and 31.0 / 27.1 / 28.6; 1,884,739
+// rows 57.7 / 55.9 / 56.9 and 117 / 73.8 / 60.4, 912 blocks 75.2).
+inline unsigned gs_dot_blocks(long long n) {
+  return std::min<unsigned>(grid_for(n, RED_THREADS), n < 400000 ? 152u : (n < 4000000 ? 304u : GS_DOT_BLOCKS));
+}
+inline unsigned gs_sub_blocks(long long n) {
+  return std::min<unsigned>(grid_for(n, RED_THREADS), n < 700000 ? 304u : (n < 4000000 ? 608u : GS_BLOCKS));
+}
 
 // hout[0..j] = V^T w; with nrm2 non-null also ||w||^2 into nrm2[0];
 // with skip non-null nothing happens when *skip != 0
 void gs_dots(Ctx& c, int j, double* hout, double* nrm2, const int* skip) {
-  const dim3 grid = lgrid(gs_blocks(c.n, GS_DOT_BLOCKS), j / GS_COLS + 1);
+  const dim3 grid = lgrid(gs_dot_blocks(c.n), j / GS_COLS + 1);
   k_gs_dots<<<grid, RED_THREADS, 0, c.stream>>>(c.n, c.V, j, c.w, c.partials, hout, nrm2, skip,
                                                 (unsigned*)(c.dflag + 2), lbytes());
   MHFP_LAUNCH_CHECK();
@@ -432,7 +449,7 @@ void gs_dots(Ctx& c, int j, double* hout, double* nrm2, const int* skip) {
 
 // w -= V h, then the tail t (see GsTail)
 void gs_sub(Ctx& c, int j, const double* h, const int* skip, const GsTail& t) {
-  k_gemv_sub<<<lgrid(gs_blocks(c.n, GS_BLOCKS)), RED_THREADS, 0, c.stream>>>(
+  k_gemv_sub<<<lgrid(gs_sub_blocks(c.n)), RED_THREADS, 0, c.stream>>>(
       c.n, c.V, j, h, c.w, c.partials + (size_t)c.opt.restart * GS_BLOCKS, skip, (unsigned*)(c.dflag + 1), t,
       lbytes());
   MHFP_LAUNCH_CHECK();
