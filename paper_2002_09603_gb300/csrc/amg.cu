@@ -2521,18 +2521,30 @@ int level_schedule(Ctx& c, std::vector<Level>& H, int l) {
 }
 
 // timed as class 4 (displacement) or 5 (interface pressure)
-void vcycle(Ctx& c, std::vector<Level>& H, const double* b, double* x) {
+void vcycle(Ctx& c, std::vector<Level>& H, const double* b, double* x, bool pre_done) {
   const int cls = (&H == &c.hu) ? 4 : 5;
   timing_begin(c, cls);
-  vcycle_level<double>(c, H, 0, b, x);
+  vcycle_level<double>(c, H, 0, b, x, pre_done);
   timing_end(c, cls, 0.0);
 }
-void vcycle(Ctx& c, std::vector<Level>& H, const float* b, float* x) {
+void vcycle(Ctx& c, std::vector<Level>& H, const float* b, float* x, bool pre_done) {
   const int cls = (&H == &c.hu) ? 4 : 5;
   timing_begin(c, cls);
-  vcycle_level<float>(c, H, 0, b, x);
+  vcycle_level<float>(c, H, 0, b, x, pre_done);
   timing_end(c, cls, 0.0);
 }
+
+namespace {
+template <typename T>
+FirstStep<T> first_step_t(Ctx& c, Level& L, T* x) {
+  if (L.dense_inv) return {};
+  const LV<T> v = view(c, L, T());
+  T* s_buf = (c.opt.cheb_degree % 2 == 1) ? v.y : x;
+  return {v.dinv, (T)(1.0 / cheb_theta(c, L)), step_out(c.opt.cheb_degree, 0, s_buf, s_buf == x ? v.y : x), v.d};
+}
+}  // namespace
+FirstStep<double> first_step(Ctx& c, std::vector<Level>& H, double* x) { return first_step_t<double>(c, H[0], x); }
+FirstStep<float> first_step(Ctx& c, std::vector<Level>& H, float* x) { return first_step_t<float>(c, H[0], x); }
 
 void level_apply(Ctx& c, std::vector<Level>& H, int l, const double* x, double* y) {
   level_spmv_t<double>(c, H[l], x, nullptr, y);

@@ -1064,10 +1064,13 @@ __global__ void __launch_bounds__(256) k_prec_p(FaceTopo32 t, const R* __restric
 // node decoding, every cell's loads issued before the sums
 template <typename R>
 __global__ void __launch_bounds__(256) k_prec_u(FaceTopo32 t, const R* __restrict__ Aup, const R* __restrict__ vu,
-                                                const R* __restrict__ zp, R* __restrict__ tu, long long lb) {
+                                                const R* __restrict__ zp, R* __restrict__ tu, FirstStep<R> fs,
+                                                long long lb) {
   vu = lane_ptr(vu, lb);
   zp = lane_ptr(zp, lb);
   tu = lane_ptr(tu, lb);
+  fs.x = lane_ptr(fs.x, lb);
+  fs.d = lane_ptr(fs.d, lb);
   const unsigned n = blockIdx.x * blockDim.x + threadIdx.x;
   const unsigned nN = (unsigned)(t.nx + 1) * (unsigned)(t.ny + 1) * (unsigned)(t.nz + 1);
   if (n >= nN) return;
@@ -1096,9 +1099,19 @@ __global__ void __launch_bounds__(256) k_prec_u(FaceTopo32 t, const R* __restric
     y1 += av[c][1] * pv[c];
     y2 += av[c][2] * pv[c];
   }
-  tu[3 * n] = vu[3 * n] - y0;
-  tu[3 * n + 1] = vu[3 * n + 1] - y1;
-  tu[3 * n + 2] = vu[3 * n + 2] - y2;
+  const R res[3] = {vu[3 * n] - y0, vu[3 * n + 1] - y1, vu[3 * n + 2] - y2};
+#pragma unroll
+  for (int a = 0; a < 3; ++a) tu[3 * n + a] = res[a];
+  if (fs.dinv) {  // the V-cycle's first smoothing step, as its own kernel would form it from tu
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+      R z = R(0);
+#pragma unroll
+      for (int s = 0; s < 3; ++s) z += fs.dinv[(size_t)(3 * a + s) * nN + n] * res[s];
+      fs.d[3 * n + a] = fs.cr * z;
+      fs.x[3 * n + a] = fs.cr * z;
+    }
+  }
 }
 
 // transposed preconditioner M^T (forward substitution u, p, pi):
@@ -1582,9 +1595,9 @@ void precond_p_step(Ctx& c, const double* vp, const double* zpi, double* zp) {
   MHFP_LAUNCH_CHECK();
 }
 
-void precond_u_rhs(Ctx& c, const double* vu, const double* zp, double* tu) {
+void precond_u_rhs(Ctx& c, const double* vu, const double* zp, double* tu, const FirstStep<double>& fs) {
   const Dims d = dims_of(c);
-  k_prec_u<double><<<lgrid(grid_for(c.nN, 256)), 256, 0, c.stream>>>(topo32(c), c.Aup, vu, zp, tu, lbytes());
+  k_prec_u<double><<<lgrid(grid_for(c.nN, 256)), 256, 0, c.stream>>>(topo32(c), c.Aup, vu, zp, tu, fs, lbytes());
   MHFP_LAUNCH_CHECK();
 }
 
@@ -1595,9 +1608,9 @@ void precond_p_step(Ctx& c, const float* vp, const float* zpi, float* zp) {
   MHFP_LAUNCH_CHECK();
 }
 
-void precond_u_rhs(Ctx& c, const float* vu, const float* zp, float* tu) {
+void precond_u_rhs(Ctx& c, const float* vu, const float* zp, float* tu, const FirstStep<float>& fs) {
   const Dims d = dims_of(c);
-  k_prec_u<float><<<lgrid(grid_for(c.nN, 256)), 256, 0, c.stream>>>(topo32(c), c.Aupf, vu, zp, tu, lbytes());
+  k_prec_u<float><<<lgrid(grid_for(c.nN, 256)), 256, 0, c.stream>>>(topo32(c), c.Aupf, vu, zp, tu, fs, lbytes());
   MHFP_LAUNCH_CHECK();
 }
 

@@ -592,10 +592,18 @@ void apply_operator_arnoldi(Ctx& c, const double* z, const float* zf, double* y,
 void narrow_to_f32(Ctx& c, const double* x, float* y, long long n);  // y = fl32(x)
 // the mixed-precision solve: FP32 preconditioner, float-float Arnoldi operator
 inline bool ff_krylov(const Ctx& c) { return c.opt.precision == 1 && c.opt.formulation == 0 && c.auu_h != nullptr; }
+// the finest displacement level's first Chebyshev step from zero, x = d = cr
+// D^-1 b, for the kernel that forms b (dinv null: none, a dense level)
+template <typename T>
+struct FirstStep {
+  const T* dinv = nullptr;
+  T cr = T(0);
+  T *x = nullptr, *d = nullptr;
+};
 void precond_p_step(Ctx& c, const double* vp, const double* zpi, double* zp);
-void precond_u_rhs(Ctx& c, const double* vu, const double* zp, double* tu);
+void precond_u_rhs(Ctx& c, const double* vu, const double* zp, double* tu, const FirstStep<double>& fs);
 void precond_p_step(Ctx& c, const float* vp, const float* zpi, float* zp);
-void precond_u_rhs(Ctx& c, const float* vu, const float* zp, float* tu);
+void precond_u_rhs(Ctx& c, const float* vu, const float* zp, float* tu, const FirstStep<float>& fs);
 void make_fp32_blocks(Ctx& c);
 void precondT_p_step(Ctx& c, const double* vp, const double* zu, double* zp);
 void precondT_p_step(Ctx& c, const float* vp, const float* zu, float* zp);
@@ -621,8 +629,12 @@ void invalidate_graphs(Ctx& c);
 
 // amg.cu
 void build_hierarchies(Ctx& c);
-void vcycle(Ctx& c, std::vector<Level>& H, const double* b, double* x);
-void vcycle(Ctx& c, std::vector<Level>& H, const float* b, float* x);
+// pre_done: the finest level's first smoothing step was taken where b was
+// formed, into first_step(c, H, x)
+void vcycle(Ctx& c, std::vector<Level>& H, const double* b, double* x, bool pre_done = false);
+void vcycle(Ctx& c, std::vector<Level>& H, const float* b, float* x, bool pre_done = false);
+FirstStep<double> first_step(Ctx& c, std::vector<Level>& H, double* x);
+FirstStep<float> first_step(Ctx& c, std::vector<Level>& H, float* x);
 void level_apply(Ctx& c, std::vector<Level>& H, int l, const double* x, double* y);
 void build_mixed_hierarchies(Ctx& c);
 void chebyshev_from_zero(Ctx& c, std::vector<Level>& H, const double* b, double* x);

@@ -547,8 +547,9 @@ void precond_blocks(Ctx& c, const T* t, T* z, T* work_u, T* work_pi, bool transp
   if (!transpose) {
     vcycle(c, c.hpi, tpi, zpi);
     precond_p_step(c, tp, zpi, zp);
-    precond_u_rhs(c, tu, zp, work_u);
-    vcycle(c, c.hu, (const T*)work_u, zu);
+    const FirstStep<T> fs = first_step(c, c.hu, zu);
+    precond_u_rhs(c, tu, zp, work_u, fs);
+    vcycle(c, c.hu, (const T*)work_u, zu, fs.dinv != nullptr);
   } else {
     vcycle(c, c.hu, tu, zu);
     precondT_p_step(c, tp, zu, zp);
