@@ -305,8 +305,9 @@ mhfp_status mhfp_grad_logk(mhfp_handle h, const double* d_lambda, const double* 
  * depend on kappa and are kept.  No device buffer of the handle is
  * reallocated (the first update allocates its scratch once: the anisotropy
  * ratios, the Galerkin product workspace and the dense-inverse workspace).
- * The captured solve graphs are dropped and captured again by the next
- * solve.  MHFP_ERR_ARG if some exp(theta_T) is not a positive finite
+ * The handle's captured solve graphs stay valid (they read the Chebyshev
+ * coefficients from device memory); batches on the handle do not (see
+ * mhfp_batch_create).  MHFP_ERR_ARG if some exp(theta_T) is not a positive finite
  * permeability (nothing is changed then).  Synchronises the stream. */
 mhfp_status mhfp_update_logk(mhfp_handle h, const double* d_logk);
 

@@ -35,8 +35,9 @@ namespace {
 template <int SPLIT>
 __global__ void __launch_bounds__(SPLIT ? 9 * U64_NODES : U64_NODES_1)
     k_cheb_u0(Lat32 L, const double* __restrict__ val, const double* __restrict__ dinv, const double* __restrict__ b,
-              const double* __restrict__ xin, double* __restrict__ xout, double* __restrict__ d, double cd, double cr,
-              long long lb) {
+              const double* __restrict__ xin, double* __restrict__ xout, double* __restrict__ d,
+              const double* __restrict__ cf, bool first, long long lb) {
+  const double cd = cf[0], cr = cf[1];
   b = lane_ptr(b, lb);
   xin = lane_ptr(xin, lb);
   xout = lane_ptr(xout, lb);
@@ -55,7 +56,7 @@ __global__ void __launch_bounds__(SPLIT ? 9 * U64_NODES : U64_NODES_1)
     double z = 0.0;
 #pragma unroll
     for (int t = 0; t < 3; ++t) z += dinv[(3 * comp + t) * N + n] * rs[t][threadIdx.x];
-    const double dn = (cd != 0.0) ? cd * d[r] + cr * z : cr * z;
+    const double dn = first ? cr * z : cd * d[r] + cr * z;
     d[r] = dn;
     xout[r] = xin[r] + dn;
   } else {
@@ -71,7 +72,7 @@ __global__ void __launch_bounds__(SPLIT ? 9 * U64_NODES : U64_NODES_1)
       double z = 0.0;
 #pragma unroll
       for (int t = 0; t < 3; ++t) z += dinv[(3 * a + t) * N + n] * acc[t];
-      const double dn = (cd != 0.0) ? cd * d[r] + cr * z : cr * z;
+      const double dn = first ? cr * z : cd * d[r] + cr * z;
       d[r] = dn;
       xout[r] = xin[r] + dn;
     }
@@ -185,7 +186,8 @@ template <typename T, int MINB>
 __global__ void __launch_bounds__(256, MINB) k_cheb_u0_sym(Lat L, const T* __restrict__ up,
                                                            const T* __restrict__ dinv, const T* __restrict__ b,
                                                            const T* __restrict__ xin, T* __restrict__ xout,
-                                                           T* __restrict__ d, T cd, T cr, long long lb) {
+                                                           T* __restrict__ d, const T* __restrict__ cf, bool first,
+                                                           long long lb) {
   b = lane_ptr(b, lb);
   xin = lane_ptr(xin, lb);
   xout = lane_ptr(xout, lb);
@@ -197,7 +199,7 @@ __global__ void __launch_bounds__(256, MINB) k_cheb_u0_sym(Lat L, const T* __res
 #pragma unroll
   for (int a = 0; a < 3; ++a) {
     const T z = dinv[(3 * a) * L.N + p] * r[0] + dinv[(3 * a + 1) * L.N + p] * r[1] + dinv[(3 * a + 2) * L.N + p] * r[2];
-    const T dn = (cd != T(0)) ? cd * d[3 * p + a] + cr * z : cr * z;
+    const T dn = first ? cf[1] * z : cf[0] * d[3 * p + a] + cf[1] * z;
     d[3 * p + a] = dn;
     xout[3 * p + a] = (xin ? xin[3 * p + a] : T(0)) + dn;
   }
@@ -270,7 +272,8 @@ struct TmaSweep {
   const float* dinv; // [9][N]
   const float *b, *xin;
   float *xout, *d;
-  float cd, cr;
+  const float* cf;   // {cd, cr} (null: the residual)
+  bool first;
   int* err;
 };
 
@@ -428,7 +431,7 @@ __global__ void __launch_bounds__(TMA_THREADS, 3) k_sym_tma(Lat L, TmaSweep a0, 
           for (int e = 0; e < 3; ++e) {
             const float z = a.dinv[(3 * e) * L.N + p] * r[0] + a.dinv[(3 * e + 1) * L.N + p] * r[1] +
                             a.dinv[(3 * e + 2) * L.N + p] * r[2];
-            const float dn = (a.cd != 0.f) ? a.cd * a.d[3 * p + e] + a.cr * z : a.cr * z;
+            const float dn = a.first ? a.cf[1] * z : a.cf[0] * a.d[3 * p + e] + a.cf[1] * z;
             a.d[3 * p + e] = dn;
             a.xout[3 * p + e] = a.xin[3 * p + e] + dn;
           }
@@ -496,7 +499,7 @@ __global__ void __launch_bounds__(128) k_pack_P(Lat32 F, Lat32 C, const double* 
 template <int BF, int BC, int R, int W, typename T>
 __global__ void __launch_bounds__(256) k_restrict_f(Lat32 F, Lat32 C, const T* __restrict__ Pc,
                                                     const T* __restrict__ r, T* __restrict__ bc,
-                                                    const T* __restrict__ dinvc, T cr, T* __restrict__ xc,
+                                                    const T* __restrict__ dinvc, const T* __restrict__ cfc, T* __restrict__ xc,
                                                     T* __restrict__ dc, long long lb) {
   r = lane_ptr(r, lb);
   bc = lane_ptr(bc, lb);
@@ -569,8 +572,8 @@ __global__ void __launch_bounds__(256) k_restrict_f(Lat32 F, Lat32 C, const T* _
     T z = T(0);
 #pragma unroll
     for (int t = 0; t < BC; ++t) z += dinvc[(unsigned)(lane * BC + t) * (unsigned)C.N + J] * acc[t];
-    dc[BC * J + lane] = cr * z;
-    xc[BC * J + lane] = cr * z;
+    dc[BC * J + lane] = cfc[1] * z;
+    xc[BC * J + lane] = cfc[1] * z;
   }
 }
 
@@ -750,7 +753,8 @@ template <typename T>
 __global__ void __launch_bounds__(256) k_cheb_ell(FaceTopo32 t, const T* __restrict__ val,
                                                   const T* __restrict__ dinv, const T* __restrict__ b,
                                                   const T* __restrict__ xin, T* __restrict__ xout, T* __restrict__ d,
-                                                  T cd, T cr, long long lb) {
+                                                  const T* __restrict__ cf, bool first, long long lb) {
+  const T cd = cf[0], cr = cf[1];
   b = lane_ptr(b, lb);
   xin = lane_ptr(xin, lb);
   xout = lane_ptr(xout, lb);
@@ -764,7 +768,7 @@ __global__ void __launch_bounds__(256) k_cheb_ell(FaceTopo32 t, const T* __restr
 #pragma unroll
     for (int q = 0; q < 11; ++q) r -= val[q * t.nF + f] * xin[col[q]];
   }
-  const T dn = (cd != T(0)) ? cd * d[f] + cr * dinv[f] * r : cr * dinv[f] * r;
+  const T dn = first ? cr * dinv[f] * r : cd * d[f] + cr * dinv[f] * r;
   d[f] = dn;
   xout[f] = (xin ? xin[f] : T(0)) + dn;
 }
@@ -811,7 +815,7 @@ __device__ __forceinline__ int ft_face_cells(const FaceTopo& d, long long f, int
 template <typename T>
 __global__ void __launch_bounds__(256) k_restrict_faces(FaceTopo32 t, const T* __restrict__ pw,
                                                         const T* __restrict__ r, T* __restrict__ bc,
-                                                        const T* __restrict__ dinvc, T cr, T* __restrict__ xc,
+                                                        const T* __restrict__ dinvc, const T* __restrict__ cfc, T* __restrict__ xc,
                                                         T* __restrict__ dc, long long lb) {
   r = lane_ptr(r, lb);
   bc = lane_ptr(bc, lb);
@@ -832,8 +836,8 @@ __global__ void __launch_bounds__(256) k_restrict_faces(FaceTopo32 t, const T* _
   if (dinvc) {  // the cell level's first Chebyshev step from zero, as k_restrict_f
     T z = T(0);
     z += dinvc[Tc] * s;
-    dc[Tc] = cr * z;
-    xc[Tc] = cr * z;
+    dc[Tc] = cfc[1] * z;
+    xc[Tc] = cfc[1] * z;
   }
 }
 
@@ -1663,6 +1667,31 @@ void make_dense_coarse(Ctx& c, Level& L) {
   if (h_err) throw Error{MHFP_ERR_ARG, "singular or indefinite coarsest multigrid level"};
 }
 
+// the Chebyshev recurrence's coefficients on [lmax / ratio, lmax]: step 0 is d
+// = (1 / theta) D^-1 r, step s > 0 is d = cd d + cr D^-1 r
+void write_cheb_coefficients(Ctx& c, Level& L) {
+  constexpr int STEPS = 8;
+  const double lmin = L.lmax / c.opt.cheb_ratio;
+  const double theta = 0.5 * (L.lmax + lmin), delta = 0.5 * (L.lmax - lmin), sigma = theta / delta;
+  double cf[2 * STEPS];
+  float cff[2 * STEPS];
+  double rho = 1.0 / sigma;
+  cf[0] = 0.0;
+  cf[1] = 1.0 / theta;
+  for (int s = 1; s < STEPS; ++s) {
+    const double rn = 1.0 / (2.0 * sigma - rho);
+    cf[2 * s] = rn * rho;
+    cf[2 * s + 1] = 2.0 * rn / delta;
+    rho = rn;
+  }
+  for (int i = 0; i < 2 * STEPS; ++i) cff[i] = (float)cf[i];
+  if (!L.cf) L.cf = dalloc_n<double>(c, 2 * STEPS);
+  if (!L.cff) L.cff = dalloc_n<float>(c, 2 * STEPS);
+  MHFP_CUDA(cudaMemcpyAsync(L.cf, cf, sizeof(cf), cudaMemcpyHostToDevice, c.stream));
+  MHFP_CUDA(cudaMemcpyAsync(L.cff, cff, sizeof(cff), cudaMemcpyHostToDevice, c.stream));
+  MHFP_CUDA(cudaStreamSynchronize(c.stream));  // cf and cff are this call's
+}
+
 void finish_level(Ctx& c, Level& L) {
   if (!L.dinv) L.dinv = dalloc_n<double>(c, (size_t)L.bs * L.bs * L.npts);
   if (L.faces) {
@@ -1682,6 +1711,7 @@ void finish_level(Ctx& c, Level& L) {
     MHFP_LAUNCH_CHECK();
   }
   L.lmax = 1.1 * spectral_radius(c, L);
+  write_cheb_coefficients(c, L);
 }
 
 // the transfer kernels index the prolongator [slot][entry][fine point] in
@@ -1950,13 +1980,13 @@ void make_fp64_transfers(Ctx& c, std::vector<Level>& H) {
 // built by the set-up, or their FP32 copies for the mixed-precision cycle.
 template <typename T>
 struct LV {
-  const T *val, *rows, *dinv, *P, *Pm, *ell, *pw;  // P: coarse-point major, Pm: fine-point major
+  const T *val, *rows, *dinv, *P, *Pm, *ell, *pw, *cf;  // P: coarse-point major, Pm: fine-point major
   T *r, *d, *y;
 };
 LV<double> view(Ctx& c, Level& L, double) {
-  return {L.A.val, L.rowd, L.dinv, L.Pd, L.P, L.ell ? L.ell : c.Cpi, c.pw, L.r, L.d, L.y};
+  return {L.A.val, L.rowd, L.dinv, L.Pd, L.P, L.ell ? L.ell : c.Cpi, c.pw, L.cf, L.r, L.d, L.y};
 }
-LV<float> view(Ctx& c, Level& L, float) { return {L.valf, L.rowf, L.dinvf, L.Pf, L.Pmf, c.Cpif, c.pwf, L.rf, L.df, L.yf}; }
+LV<float> view(Ctx& c, Level& L, float) { return {L.valf, L.rowf, L.dinvf, L.Pf, L.Pmf, c.Cpif, c.pwf, L.cff, L.rf, L.df, L.yf}; }
 double* bvec(Level& L, double) { return L.b; }
 float* bvec(Level& L, float) { return L.bf; }
 double* xvec(Level& L, double) { return L.x; }
@@ -1976,12 +2006,12 @@ void level_spmv_t(Ctx& c, Level& L, const T* x, const T* b, T* y) {
 // one Chebyshev sweep on a lattice level with schedule sched (the first
 // sweep from zero has no stencil work and always runs one point per thread)
 template <typename T>
-void launch_cheb(Ctx& c, Level& L, const LV<T>& v, const T* b, const T* xin, T* out, T cd, T cr, int sched) {
+void launch_cheb(Ctx& c, Level& L, const LV<T>& v, const T* b, const T* xin, T* out, int step, int sched) {
   if (!xin) {
-    sweep_cheb_zero<T>(c.stream, L.A.N, L.bs, v.dinv, b, out, v.d, cr);
+    sweep_cheb_zero<T>(c.stream, L.A.N, L.bs, v.dinv, b, out, v.d, v.cf);
     return;
   }
-  sweep_cheb<T>(c.stream, L.A, L.bs, v.val, v.rows, v.dinv, b, xin, out, v.d, cd, cr, sched);
+  sweep_cheb<T>(c.stream, L.A, L.bs, v.val, v.rows, v.dinv, b, xin, out, v.d, v.cf + 2 * step, step == 0, sched);
 }
 
 // The symmetric FP32 sweep and residual of the finest displacement level
@@ -1997,7 +2027,7 @@ int sym_minb(const Level& L) {
 
 // the bulk-copy-fed variant (schedule 4): persistent CTAs, 4 per SM
 void launch_sym_tma(Ctx& c, const Level& L, bool cheb, const float* b, const float* xin, float* xout, float* d,
-                    float cd, float cr) {
+                    const float* cf, bool first) {
   const Lat lat = lat_of(L.A);
   if (lat.N >= (1LL << 31) - TMA_NB) throw Error{MHFP_ERR_ARG, "level too large for the bulk-copy sweep"};
   const long long nblocks = (lat.N + TMA_NB - 1) / TMA_NB;
@@ -2008,40 +2038,40 @@ void launch_sym_tma(Ctx& c, const Level& L, bool cheb, const float* b, const flo
     MHFP_CUDA(cudaFuncSetAttribute(k_sym_tma<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TMA_SMEM));
     attr = true;
   }
-  TmaSweep a{L.symf, L.dinvf, b, xin, xout, d, cd, cr, c.d_flag};
+  TmaSweep a{L.symf, L.dinvf, b, xin, xout, d, cf, first, c.d_flag};
   if (cheb) k_sym_tma<true><<<lgrid(grid), TMA_THREADS, TMA_SMEM, c.stream>>>(lat, a, lbytes());
   else k_sym_tma<false><<<lgrid(grid), TMA_THREADS, TMA_SMEM, c.stream>>>(lat, a, lbytes());
 }
-void launch_cheb_sym(Ctx& c, const Level& L, const float* b, const float* xin, float* xout, float* d, float cd,
-                     float cr) {
+void launch_cheb_sym(Ctx& c, const Level& L, const float* b, const float* xin, float* xout, float* d, const float* cf,
+                     bool first) {
   const Lat lat = lat_of(L.A);
   if (!xin) {  // the first step from zero has no stencil work
-    sweep_cheb_zero<float>(c.stream, lat.N, 3, L.dinvf, b, xout, d, cr);
+    sweep_cheb_zero<float>(c.stream, lat.N, 3, L.dinvf, b, xout, d, cf);
     MHFP_LAUNCH_CHECK();
     return;
   }
   const int mb = sym_minb(L);
   if (mb == 4)
-    launch_sym_tma(c, L, true, b, xin, xout, d, cd, cr);
+    launch_sym_tma(c, L, true, b, xin, xout, d, cf, first);
   else if (mb == 5)
     k_cheb_u0_sym<float, 5><<<lgrid(grid_for(lat.N, 256)), 256, 0, c.stream>>>(lat, L.symf, L.dinvf, b, xin,
-                                                                                xout, d, cd, cr, lbytes());
+                                                                                xout, d, cf, first, lbytes());
   else if (mb == 7)
     k_cheb_u0_sym<float, 7><<<lgrid(grid_for(lat.N, 256)), 256, 0, c.stream>>>(lat, L.symf, L.dinvf, b, xin,
-                                                                                xout, d, cd, cr, lbytes());
+                                                                                xout, d, cf, first, lbytes());
   else if (mb == 8)
     k_cheb_u0_sym<float, 8><<<lgrid(grid_for(lat.N, 256)), 256, 0, c.stream>>>(lat, L.symf, L.dinvf, b, xin,
-                                                                                xout, d, cd, cr, lbytes());
+                                                                                xout, d, cf, first, lbytes());
   else
     k_cheb_u0_sym<float, 6><<<lgrid(grid_for(lat.N, 256)), 256, 0, c.stream>>>(lat, L.symf, L.dinvf, b, xin,
-                                                                                xout, d, cd, cr, lbytes());
+                                                                                xout, d, cf, first, lbytes());
   MHFP_LAUNCH_CHECK();
 }
 void launch_resid_sym(Ctx& c, const Level& L, const float* x, const float* b, float* y) {
   const Lat lat = lat_of(L.A);
   const int mb = sym_minb(L);
   if (mb == 4)
-    launch_sym_tma(c, L, false, b, x, y, nullptr, 0.f, 0.f);
+    launch_sym_tma(c, L, false, b, x, y, nullptr, nullptr, true);
   else if (mb == 5)
     k_resid_u0_sym<float, 5><<<lgrid(grid_for(lat.N, 256)), 256, 0, c.stream>>>(lat, L.symf, x, b, y,
                                                                                  lbytes());
@@ -2131,7 +2161,7 @@ void autotune_fine_sym(Ctx& c, Level& L) {
   int best_minb = 0;
   for (int minb : {8, 7, 6, 5, 4}) {
     L.tpp = minb;
-    const float us = graph_time_us(c, tune_reps(4.0 * 126 * L.A.N), best, [&] { launch_cheb_sym(c, L, L.bf, L.xf, L.yf, L.df, 0.5f, 0.5f); });
+    const float us = graph_time_us(c, tune_reps(4.0 * 126 * L.A.N), best, [&] { launch_cheb_sym(c, L, L.bf, L.xf, L.yf, L.df, L.cff + 2, false); });
     if (us < best) {
       best = us;
       best_minb = minb;
@@ -2159,7 +2189,7 @@ void autotune_level(Ctx& c, Level& L) {
   const std::vector<int> cand = v.rows ? std::vector<int>{32, 64, 8, 4, 16} : std::vector<int>{1, 4, 8, 16};
   for (int tpp : cand) {
     const float us = graph_time_us(c, tune_reps((double)sizeof(T) * L.A.noff() * L.bs * L.bs * L.A.N), best, [&] {
-      launch_cheb<T>(c, L, v, b, x, v.y, T(0.5), T(0.5), tpp);
+      launch_cheb<T>(c, L, v, b, x, v.y, 1, tpp);
       MHFP_LAUNCH_CHECK();
     });
     if (us < best) {
@@ -2176,12 +2206,6 @@ void autotune_level(Ctx& c, Level& L) {
 // steps write dst and alt in turn, chosen so that the last one writes dst
 // (the first step's output differs from x0 when alt is the buffer that x0
 // is not, or x0 is null).
-// the centre of level L's Chebyshev interval [lmax / ratio, lmax]
-double cheb_theta(const Ctx& c, const Level& L) {
-  const double lmax = L.lmax, lmin = lmax / c.opt.cheb_ratio;
-  return 0.5 * (lmax + lmin);
-}
-
 // output buffer of step s of a smoothing into dst that alternates with alt
 template <typename T>
 T* step_out(int deg, int s, T* dst, T* alt) {
@@ -2197,39 +2221,29 @@ void smooth(Ctx& c, std::vector<Level>& H, int l, const T* b, const T* x0, T* ds
   Level& L = H[l];
   const LV<T> v = view(c, L, T());
   const int deg = c.opt.cheb_degree;
-  const double lmax = L.lmax, lmin = lmax / c.opt.cheb_ratio;
-  const double theta = cheb_theta(c, L), delta = 0.5 * (lmax - lmin), sigma = theta / delta;
-  double rho = 1.0 / sigma;
   const T* xin = first_done ? step_out(deg, 0, dst, alt) : x0;
   for (int s = first_done ? 1 : 0; s < deg; ++s) {
     T* out = step_out(deg, s, dst, alt);
-    double cd = 0.0, cr = 1.0 / theta;
-    if (s > 0) {
-      const double rn = 1.0 / (2.0 * sigma - rho);
-      cd = rn * rho;
-      cr = 2.0 * rn / delta;
-      rho = rn;
-    }
     if (time_it && xin) timing_begin(c, 0);
     if (L.faces) {
       k_cheb_ell<T><<<lgrid(grid_for(L.n, 256)), 256, 0, c.stream>>>(face_topo(c), v.ell, v.dinv, b, xin, out, v.d,
-                                                                     (T)cd, (T)cr, lbytes());
+                                                                     v.cf + 2 * s, s == 0, lbytes());
     } else if (time_it) {
       if constexpr (std::is_same<T, float>::value) {
-        launch_cheb_sym(c, L, b, xin, out, v.d, (T)cd, (T)cr);
+        launch_cheb_sym(c, L, b, xin, out, v.d, v.cf + 2 * s, s == 0);
       } else {
         const Lat32 lat = lat32_of(L.A);
         if (!xin)  // the first step from zero has no stencil work
-          sweep_cheb_zero<T>(c.stream, lat.N, 3, v.dinv, b, out, v.d, (T)cr);
+          sweep_cheb_zero<T>(c.stream, lat.N, 3, v.dinv, b, out, v.d, v.cf);
         else if (lat.N <= U64_SPLIT_NODES)
           k_cheb_u0<1><<<lgrid(grid_for(lat.N, U64_NODES)), dim3(U64_NODES, 9), 0, c.stream>>>(
-              lat, v.val, v.dinv, b, xin, out, v.d, cd, cr, lbytes());
+              lat, v.val, v.dinv, b, xin, out, v.d, v.cf + 2 * s, s == 0, lbytes());
         else
           k_cheb_u0<0><<<lgrid(grid_for(lat.N, U64_NODES_1)), U64_NODES_1, 0, c.stream>>>(
-              lat, v.val, v.dinv, b, xin, out, v.d, cd, cr, lbytes());
+              lat, v.val, v.dinv, b, xin, out, v.d, v.cf + 2 * s, s == 0, lbytes());
       }
     } else {
-      launch_cheb<T>(c, L, v, b, xin, out, (T)cd, (T)cr, L.tpp ? L.tpp : default_schedule(L.A, v.rows != nullptr));
+      launch_cheb<T>(c, L, v, b, xin, out, s, L.tpp ? L.tpp : default_schedule(L.A, v.rows != nullptr));
     }
     MHFP_LAUNCH_CHECK();
     // algorithmic bytes of a Chebyshev sweep: the matrix values (27 blocks
@@ -2278,7 +2292,7 @@ void vcycle_level(Ctx& c, std::vector<Level>& H, int l, const T* b, T* x, bool p
   const int deg = c.opt.cheb_degree;
   T* cs_buf = (deg % 2 == 1) ? cv.y : cx;
   const T* fdinv = fuse ? cv.dinv : nullptr;
-  const T fcr = fuse ? (T)(1.0 / cheb_theta(c, C)) : T(0);
+  const T* fcr = fuse ? cv.cf : nullptr;
   T* fx = fuse ? step_out(deg, 0, cs_buf, cs_buf == cx ? cv.y : cx) : nullptr;
   T* fd = fuse ? cv.d : nullptr;
   if (L.faces) {
@@ -2540,7 +2554,7 @@ FirstStep<T> first_step_t(Ctx& c, Level& L, T* x) {
   if (L.dense_inv) return {};
   const LV<T> v = view(c, L, T());
   T* s_buf = (c.opt.cheb_degree % 2 == 1) ? v.y : x;
-  return {v.dinv, (T)(1.0 / cheb_theta(c, L)), step_out(c.opt.cheb_degree, 0, s_buf, s_buf == x ? v.y : x), v.d};
+  return {v.dinv, v.cf + 1, step_out(c.opt.cheb_degree, 0, s_buf, s_buf == x ? v.y : x), v.d};
 }
 }  // namespace
 FirstStep<double> first_step(Ctx& c, std::vector<Level>& H, double* x) { return first_step_t<double>(c, H[0], x); }

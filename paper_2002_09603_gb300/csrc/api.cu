@@ -507,7 +507,9 @@ mhfp_status mhfp_update_logk(mhfp_handle h, const double* d_logk) {
     if (!c.prepared) throw Error{MHFP_ERR_STATE, "mhfp_setup_precond must come first"};
     if (!d_logk) throw Error{MHFP_ERR_ARG, "bad log-permeability vector"};
     mhfp::update_logk_blocks(c, d_logk);  // validates before changing anything
-    mhfp::invalidate_graphs(c);
+    // every buffer and schedule stays, so the handle's captured solve graphs
+    // stay valid; batches are refused until they are created again
+    ++c.graph_gen;
     mhfp::rebuild_pi_hierarchy(c);
     if (c.opt.precision == 1) mhfp::make_fp32_blocks(c);
     MHFP_CUDA(cudaStreamSynchronize(c.stream));

@@ -1102,14 +1102,16 @@ __global__ void __launch_bounds__(256) k_prec_u(FaceTopo32 t, const R* __restric
   const R res[3] = {vu[3 * n] - y0, vu[3 * n + 1] - y1, vu[3 * n + 2] - y2};
 #pragma unroll
   for (int a = 0; a < 3; ++a) tu[3 * n + a] = res[a];
-  if (fs.dinv) {  // the V-cycle's first smoothing step, as its own kernel would form it from tu
+  if (fs.dinv) {
+    const R cr = *fs.cr;
+    // the V-cycle's first smoothing step, as its own kernel would form it from tu
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
       R z = R(0);
 #pragma unroll
       for (int s = 0; s < 3; ++s) z += fs.dinv[(size_t)(3 * a + s) * nN + n] * res[s];
-      fs.d[3 * n + a] = fs.cr * z;
-      fs.x[3 * n + a] = fs.cr * z;
+      fs.d[3 * n + a] = cr * z;
+      fs.x[3 * n + a] = cr * z;
     }
   }
 }

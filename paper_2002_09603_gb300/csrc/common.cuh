@@ -377,6 +377,11 @@ struct Level {
   StructOp A;                 // lattice operator (unused on the face level)
   double* dinv = nullptr;     // [bs*bs][npts] inverse diagonal blocks
   double lmax = 0.0;
+  // Chebyshev coefficients {cd, cr} of steps 0..7 (the degree's limit is 8) in
+  // device memory, FP64 and FP32: the captured solve graphs read them there, so
+  // that a permeability update, which changes lmax, leaves the graphs valid
+  double* cf = nullptr;
+  float* cff = nullptr;
   // prolongator to the next level (lattice levels only): [p_slots^3][bs*bs][npts]
   // as the set-up builds it (fine-point major; Pmf: FP32, large levels), and coarse-point major
   // as the restriction and the small levels' prolongation read it (Pd; Pf: FP32)
@@ -597,7 +602,7 @@ inline bool ff_krylov(const Ctx& c) { return c.opt.precision == 1 && c.opt.formu
 template <typename T>
 struct FirstStep {
   const T* dinv = nullptr;
-  T cr = T(0);
+  const T* cr = nullptr;  // the step's coefficient, in device memory
   T *x = nullptr, *d = nullptr;
 };
 void precond_p_step(Ctx& c, const double* vp, const double* zpi, double* zp);
@@ -623,8 +628,8 @@ void btp_p_rhs(Ctx& c, const double* vp, const double* zu, const double* zq, dou
 // amg.cu: the interface-pressure hierarchy and the FP32 copies rebuilt in
 // place after a permeability update (same levels, same schedules)
 void rebuild_pi_hierarchy(Ctx& c);
-// krylov.cu: drop the captured CUDA graphs (their kernel arguments hold the
-// old Chebyshev coefficients); the next solve captures them again
+// krylov.cu: drop the captured CUDA graphs (a new Chebyshev degree changes
+// their launches); the next solve captures them again
 void invalidate_graphs(Ctx& c);
 
 // amg.cu

@@ -220,13 +220,13 @@ void sweep_spmv(cudaStream_t stream, const StructOp& A, int bs, const T* val, co
                 T* y, int sched);
 template <typename T>
 void sweep_cheb(cudaStream_t stream, const StructOp& A, int bs, const T* val, const T* rows, const T* dinv, const T* b,
-                const T* xin, T* out, T* d, T cd, T cr, int sched);
+                const T* xin, T* out, T* d, const T* cf, bool first, int sched);
 // row-major copy of a level's values (schedules 32 and 64; null: none)
 template <typename T>
 size_t sweep_row_elems(const StructOp& A, int bs);
 template <typename T>
 void sweep_pack_rows(cudaStream_t stream, const StructOp& A, int bs, const T* val, T* rows);
 template <typename T>
-void sweep_cheb_zero(cudaStream_t stream, long long npts, int bs, const T* dinv, const T* b, T* out, T* d, T cr);
+void sweep_cheb_zero(cudaStream_t stream, long long npts, int bs, const T* dinv, const T* b, T* out, T* d, const T* cf);
 
 }  // namespace mhfp

@@ -87,17 +87,19 @@ __global__ void __launch_bounds__(256) k_spmv_f(Lat32 L, const T* __restrict__ v
   for (int a = 0; a < BS; ++a) y[BS * p + a] = b ? b[BS * p + a] + r[a] : -r[a];
 }
 
-// Chebyshev step: r = b - A xin (r = b when xin is null), d = cd d + cr D^-1 r, xout = xin + d
+// Chebyshev step: r = b - A xin, d = cd d + cr D^-1 r, xout = xin + d with cf = {cd, cr} in device
+// memory; FIRST (cd = 0): d is only written
 template <typename T, int BS>
 __device__ __forceinline__ void cheb_update(unsigned p, unsigned N, const T r[BS], const T* __restrict__ dinv,
-                                            const T* __restrict__ xin, T* __restrict__ xout, T* __restrict__ d, T cd,
-                                            T cr) {
+                                            const T* __restrict__ xin, T* __restrict__ xout, T* __restrict__ d,
+                                            const T* __restrict__ cf, bool first) {
+  const T cd = cf[0], cr = cf[1];
 #pragma unroll
   for (int a = 0; a < BS; ++a) {
     T z = T(0);
 #pragma unroll
     for (int s = 0; s < BS; ++s) z += dinv[(a * BS + s) * N + p] * r[s];
-    const T dn = (cd != T(0)) ? cd * d[BS * p + a] + cr * z : cr * z;
+    const T dn = first ? cr * z : cd * d[BS * p + a] + cr * z;
     d[BS * p + a] = dn;
     xout[BS * p + a] = (xin ? xin[BS * p + a] : T(0)) + dn;
   }
@@ -106,7 +108,8 @@ __device__ __forceinline__ void cheb_update(unsigned p, unsigned N, const T r[BS
 template <int BS, int KIND, typename T>
 __global__ void __launch_bounds__(256) k_cheb_f(Lat32 L, const T* __restrict__ val, const T* __restrict__ dinv,
                                                 const T* __restrict__ b, const T* __restrict__ xin,
-                                                T* __restrict__ xout, T* __restrict__ d, T cd, T cr, long long lb) {
+                                                T* __restrict__ xout, T* __restrict__ d, const T* __restrict__ cf, bool first,
+                                                long long lb) {
   b = lane_ptr(b, lb);
   xin = lane_ptr(xin, lb);
   xout = lane_ptr(xout, lb);
@@ -117,17 +120,18 @@ __global__ void __launch_bounds__(256) k_cheb_f(Lat32 L, const T* __restrict__ v
 #pragma unroll
   for (int a = 0; a < BS; ++a) r[a] = b[BS * p + a];
   coarse_residual<BS, KIND, f_chunk<BS, T>(), T>(L, p, val, xin, r, 0, 1);
-  cheb_update<T, BS>(p, (unsigned)L.N, r, dinv, xin, xout, d, cd, cr);
+  cheb_update<T, BS>(p, (unsigned)L.N, r, dinv, xin, xout, d, cf, first);
 }
 
 // the first Chebyshev step from x = 0: d = cr D^-1 b, xout = d (no stencil)
 template <int BS, typename T>
 __global__ void __launch_bounds__(256) k_cheb_zero(long long npts, const T* __restrict__ dinv,
                                                    const T* __restrict__ b, T* __restrict__ xout, T* __restrict__ d,
-                                                   T cr, long long lb) {
+                                                   const T* __restrict__ cf, long long lb) {
   b = lane_ptr(b, lb);
   xout = lane_ptr(xout, lb);
   d = lane_ptr(d, lb);
+  const T cr = cf[1];
   const long long p = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (p >= npts) return;
   T r[BS];
@@ -190,7 +194,8 @@ __global__ void __launch_bounds__(32 * W) k_spmv_w(Lat32 L, const T* __restrict_
 template <int BS, int KIND, int W, typename T>
 __global__ void __launch_bounds__(32 * W) k_cheb_w(Lat32 L, const T* __restrict__ val, const T* __restrict__ dinv,
                                                    const T* __restrict__ b, const T* __restrict__ xin,
-                                                   T* __restrict__ xout, T* __restrict__ d, T cd, T cr, long long lb) {
+                                                   T* __restrict__ xout, T* __restrict__ d, const T* __restrict__ cf, bool first,
+                                                long long lb) {
   b = lane_ptr(b, lb);
   xin = lane_ptr(xin, lb);
   xout = lane_ptr(xout, lb);
@@ -201,7 +206,7 @@ __global__ void __launch_bounds__(32 * W) k_cheb_w(Lat32 L, const T* __restrict_
   if (!wsplit_residual<BS, KIND, W, T>(L, val, xin, part, p, r)) return;
 #pragma unroll
   for (int a = 0; a < BS; ++a) r[a] += b[BS * p + a];
-  cheb_update<T, BS>(p, (unsigned)L.N, r, dinv, xin, xout, d, cd, cr);
+  cheb_update<T, BS>(p, (unsigned)L.N, r, dinv, xin, xout, d, cf, first);
 }
 
 // Row-major levels: LPP lanes per point on values Ar[point][row a][PP], the
@@ -293,7 +298,8 @@ __global__ void __launch_bounds__(128) k_spmv_r(Lat32 L, const T* __restrict__ A
 template <int BS, int KIND, int LPP, typename T>
 __global__ void __launch_bounds__(128) k_cheb_r(Lat32 L, const T* __restrict__ Ar, const T* __restrict__ dinv,
                                                 const T* __restrict__ b, const T* __restrict__ xin,
-                                                T* __restrict__ xout, T* __restrict__ d, T cd, T cr, long long lb) {
+                                                T* __restrict__ xout, T* __restrict__ d, const T* __restrict__ cf, bool first,
+                                                long long lb) {
   b = lane_ptr(b, lb);
   xin = lane_ptr(xin, lb);
   xout = lane_ptr(xout, lb);
@@ -309,7 +315,8 @@ __global__ void __launch_bounds__(128) k_cheb_r(Lat32 L, const T* __restrict__ A
     di[t] = dinv[(ac * BS + t) * (unsigned)L.N + p];
     bv[t] = b[BS * p + t];
   }
-  if (cd != T(0)) dv = d[BS * p + ac];
+  if (!first) dv = d[BS * p + ac];
+  const T cd = cf[0], cr = cf[1];
   xv = xin[BS * p + ac];
   T r[BS];
   row_product<BS, KIND, LPP, T>(L, p, Ar, xin, r);
@@ -317,7 +324,7 @@ __global__ void __launch_bounds__(128) k_cheb_r(Lat32 L, const T* __restrict__ A
   T z = T(0);
 #pragma unroll
   for (int t = 0; t < BS; ++t) z += di[t] * (bv[t] - r[t]);
-  const T dn = (cd != T(0)) ? cd * dv + cr * z : cr * z;
+  const T dn = first ? cr * z : cd * dv + cr * z;
   d[BS * p + a] = dn;
   xout[BS * p + a] = xv + dn;
 }
@@ -374,12 +381,12 @@ void sweep_spmv(cudaStream_t stream, const StructOp& A, int bs, const T* val, co
 
 template <typename T>
 void sweep_cheb(cudaStream_t stream, const StructOp& A, int bs, const T* val, const T* rows, const T* dinv, const T* b,
-                const T* xin, T* out, T* d, T cd, T cr, int sched) {
+                const T* xin, T* out, T* d, const T* cf, bool first, int sched) {
   const Lat32 lat = lat32_of(A);
   if (const int lpp = rows ? row_lanes(sched) : 0) {
     dispatch_rows(bs, A.kind, lpp, [&](auto BS, auto K, auto LPP) {
       k_cheb_r<BS.value, K.value, LPP.value, T><<<lgrid(grid_for(A.N * LPP.value, 128)), 128, 0, stream>>>(
-          lat, rows, dinv, b, xin, out, d, cd, cr, lbytes());
+          lat, rows, dinv, b, xin, out, d, cf, first, lbytes());
     });
     return;
   }
@@ -387,11 +394,11 @@ void sweep_cheb(cudaStream_t stream, const StructOp& A, int bs, const T* val, co
     dispatch_kind_bs<BS.value>(A.kind, [&](auto K) {
       dispatch_sched(sched, [&](auto S) {
         if constexpr (S.value == 1)
-          k_cheb_f<BS.value, K.value, T><<<lgrid(grid_for(A.N, 256)), 256, 0, stream>>>(lat, val, dinv, b, xin, out, d,
-                                                                                         cd, cr, lbytes());
+          k_cheb_f<BS.value, K.value, T><<<lgrid(grid_for(A.N, 256)), 256, 0, stream>>>(
+              lat, val, dinv, b, xin, out, d, cf, first, lbytes());
         else
           k_cheb_w<BS.value, K.value, S.value, T><<<lgrid(grid_for(A.N, 32)), dim3(32, S.value), 0, stream>>>(
-              lat, val, dinv, b, xin, out, d, cd, cr, lbytes());
+              lat, val, dinv, b, xin, out, d, cf, first, lbytes());
       });
     });
   });
@@ -412,9 +419,10 @@ void sweep_pack_rows(cudaStream_t stream, const StructOp& A, int bs, const T* va
 }
 
 template <typename T>
-void sweep_cheb_zero(cudaStream_t stream, long long npts, int bs, const T* dinv, const T* b, T* out, T* d, T cr) {
+void sweep_cheb_zero(cudaStream_t stream, long long npts, int bs, const T* dinv, const T* b, T* out, T* d,
+                     const T* cf) {
   dispatch_bs(bs, [&](auto BS) {
-    k_cheb_zero<BS.value, T><<<lgrid(grid_for(npts, 256)), 256, 0, stream>>>(npts, dinv, b, out, d, cr, lbytes());
+    k_cheb_zero<BS.value, T><<<lgrid(grid_for(npts, 256)), 256, 0, stream>>>(npts, dinv, b, out, d, cf, lbytes());
   });
 }
 
@@ -422,10 +430,10 @@ template void sweep_spmv<MHFP_SWEEP_T>(cudaStream_t, const StructOp&, int, const
                                        const MHFP_SWEEP_T*, const MHFP_SWEEP_T*, MHFP_SWEEP_T*, int);
 template void sweep_cheb<MHFP_SWEEP_T>(cudaStream_t, const StructOp&, int, const MHFP_SWEEP_T*, const MHFP_SWEEP_T*,
                                        const MHFP_SWEEP_T*, const MHFP_SWEEP_T*, const MHFP_SWEEP_T*, MHFP_SWEEP_T*,
-                                       MHFP_SWEEP_T*, MHFP_SWEEP_T, MHFP_SWEEP_T, int);
+                                       MHFP_SWEEP_T*, const MHFP_SWEEP_T*, bool, int);
 template size_t sweep_row_elems<MHFP_SWEEP_T>(const StructOp&, int);
 template void sweep_pack_rows<MHFP_SWEEP_T>(cudaStream_t, const StructOp&, int, const MHFP_SWEEP_T*, MHFP_SWEEP_T*);
 template void sweep_cheb_zero<MHFP_SWEEP_T>(cudaStream_t, long long, int, const MHFP_SWEEP_T*, const MHFP_SWEEP_T*,
-                                            MHFP_SWEEP_T*, MHFP_SWEEP_T*, MHFP_SWEEP_T);
+                                            MHFP_SWEEP_T*, MHFP_SWEEP_T*, const MHFP_SWEEP_T*);
 
 }  // namespace mhfp

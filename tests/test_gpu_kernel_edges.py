@@ -163,3 +163,24 @@ def test_row_major_levels_against_the_oracle(dims, autotune, precision, near_ker
                 y = s.level_apply(which, l, torch.from_numpy(x).cuda()).cpu().numpy()
                 assert np.abs(y - lev.A @ x).max() <= 1e-11 * np.abs(lev.A @ x).max()
     s.close()
+
+
+@pytest.mark.parametrize("precision,degree", [(0, 1), (0, 3), (1, 1), (1, 2)])
+def test_update_keeps_the_captured_solves(precision, degree):
+    """Solves (both directions) captured before a permeability update give,
+    after it, bit for bit what a handle updated before its first solve gives."""
+    prob = mi.random_small(9, 8, 7, seed=21, jitter=0.1)
+    logk = np.log(prob.kappa[:, 0]) + np.random.default_rng(1).uniform(-2, 2, prob.n_cells)
+    lk = torch.from_numpy(logk).cuda()
+    opts = dict(autotune=0, coarse_max=30, restart=9, precision=precision, cheb_degree=degree)
+    used, fresh = _solver(prob, **opts), _solver(prob, **opts)
+    b = used.build_rhs()
+    used.solve(b, tol=1e-9)
+    used.adjoint_solve(b, tol=1e-6)
+    used.update_logk(lk)
+    fresh.update_logk(lk)
+    for f in ("solve", "adjoint_solve"):
+        (x, sx), (y, sy) = (getattr(s, f)(b, tol=1e-9) for s in (used, fresh))
+        assert torch.equal(x, y) and sx["iterations"] == sy["iterations"]
+    used.close()
+    fresh.close()
