@@ -1539,39 +1539,135 @@ double spectral_radius(Ctx& c, Level& L) {
   return h;
 }
 
-// Gauss-Jordan inverse with partial pivoting (host, FP64), row-major
-// Dense inverse of the coarsest level by Gauss-Jordan elimination on the GPU
-// (FP64, augmented [A | I] of n x 2n, row-major).  The coarse operators are
-// Galerkin products of SPD operators (Dirichlet rows carry a unit diagonal),
-// so elimination needs no pivoting; a pivot that is not positive and finite
-// sets *err and the host reports a singular level.  Column col takes two
-// kernels: the first copies the scaled pivot row and the multipliers, the
-// second updates every row from those copies (no read/write hazard).
-__global__ void k_gj_pivot(int n, int col, const double* __restrict__ M, double* __restrict__ prow,
-                           double* __restrict__ fcol, int* __restrict__ err) {
-  const int w = 2 * n;
-  const double piv = M[(long long)col * w + col];
-  const int t = blockIdx.x * blockDim.x + threadIdx.x;
-  if (t == 0 && !(piv > 0.0 && piv < 1e300)) *err = 1;
-  if (t < w) prow[t] = t < col ? 0.0 : M[(long long)col * w + t] / piv;
-  if (t < n) fcol[t] = M[(long long)t * w + col];
+// Dense inverse of the coarsest level by block Gauss-Jordan elimination in
+// place on the GPU (FP64, row-major).  The coarse operators are Galerkin
+// products of SPD operators (Dirichlet rows carry a unit diagonal): elimination
+// needs no pivoting, and with E the eliminated indices M[j][i] is M[i][j] if
+// both or neither are in E and -M[i][j] otherwise, so only the upper triangle
+// is kept until the end.  A pivot that is not positive and finite sets *err and
+// the host reports a singular level.  GJ_B columns (k0 .. k0 + nb - 1) take
+// three kernels: D = the diagonal block's inverse, the panels, and the rank-GJ_B
+// update of the other tiles; n^3 / 2 FMA in all.  An SM has two FP64 FMA a
+// clock, so even one block's product is long: D takes its reciprocal once per
+// column, and tiles of 32 x 32 spread the update over the chip at the default
+// sizes (n up to 375).  Column by column on [A | I] it took 1.5 n^3 FMA, two
+// launches per column and a pass over the matrix for each: the two levels of a
+// 64^3 set-up with coarse_max 512 (1,536 and 512 unknowns) 24.8 -> 5.9 ms of
+// kernels, that set-up 52 -> 17.4 ms with the launches saved.
+constexpr int GJ_B = 32;                      // columns per step, and the update's tile
+constexpr int GJ_TRI = GJ_B * (GJ_B + 1) / 2;  // entries of D's upper triangle
+
+__global__ void __launch_bounds__(GJ_TRI + 16) k_gj_diag(int n, int k0, const double* __restrict__ M,
+                                                         double* __restrict__ D, int* __restrict__ err) {
+  __shared__ double S[GJ_B][GJ_B + 1], row[GJ_B], inv;
+  const int nb = min(GJ_B, n - k0), t = threadIdx.x;
+  const bool on = t < GJ_TRI;
+  int r = 0, q = t;  // entry t of the triangle: row r, column q >= r
+  if (on)
+    for (; q >= GJ_B; ++r) q += r + 1 - GJ_B;  // row r + 1 starts at its diagonal
+  else
+    q = 0;
+  if (on) S[r][q] = q < nb ? M[(size_t)(k0 + r) * n + k0 + q] : (r == q ? 1.0 : 0.0);
+  __syncthreads();
+  for (int c = 0; c < nb; ++c) {
+    if (t < GJ_B) {
+      // row c times the reciprocal pivot; the eliminated columns' sign flips
+      const double p = S[c][c], ip = 1.0 / p;
+      if (t == 0) {
+        if (!(p > 0.0 && p < 1e300)) *err = 1;
+        inv = ip;
+      }
+      row[t] = (t < c ? -S[t][c] : S[c][t]) * ip;
+    }
+    __syncthreads();
+    double v = 0.0;
+    if (on) {
+      const double fr = r <= c ? S[r][c] : S[c][r];
+      v = r == c ? (q == c ? inv : row[q]) : (q == c ? -fr * inv : fma(-fr, row[q], S[r][q]));
+    }
+    __syncthreads();
+    if (on) S[r][q] = v;
+    __syncthreads();
+  }
+  if (on) D[r * GJ_B + q] = D[q * GJ_B + r] = S[r][q];
 }
 
-__global__ void k_gj_update(int n, int col, double* __restrict__ M, const double* __restrict__ prow,
-                            const double* __restrict__ fcol) {
-  const int w = 2 * n;
-  const int k = col + blockIdx.x * blockDim.x + threadIdx.x;
-  const int r = blockIdx.y;
-  if (k >= w) return;
-  double* m = M + (long long)r * w + k;
-  *m = (r == col) ? prow[k] : *m - fcol[r] * prow[k];
+// V[u][j] = M[k0 + u][j] up to the sign, from the upper triangle, and
+// R[u][j] = (D M_k)[u][j] (D itself in the block's own columns).  A block takes
+// 32 columns and eight rows of R; those of blockIdx.y = 0 write V.
+__global__ void __launch_bounds__(256) k_gj_panel(int n, int k0, const double* __restrict__ M,
+                                                  const double* __restrict__ D, double* __restrict__ R,
+                                                  double* __restrict__ V) {
+  __shared__ double sD[8][GJ_B], sV[GJ_B][GJ_B + 1];
+  const int nb = min(GJ_B, n - k0), j0 = blockIdx.x * GJ_B, u0 = blockIdx.y * 8;
+  const int q = threadIdx.x & 31, w = threadIdx.x >> 5, j = j0 + q;
+  // k0 is a multiple of 32: a block's columns lie left of the pivot block, in
+  // it, or to its right
+  const bool left = j0 < k0, own = j0 == k0;
+  sD[w][q] = D[(u0 + w) * GJ_B + q];
+  for (int x = w; x < GJ_B; x += 8) {
+    if (left) sV[q][x] = q < nb ? M[(size_t)(j0 + x) * n + k0 + q] : 0.0;
+    else sV[x][q] = x < nb && j < n && !own ? M[(size_t)(k0 + x) * n + j] : 0.0;
+  }
+  __syncthreads();
+  if (j >= n) return;
+  if (blockIdx.y == 0)
+    for (int x = w; x < GJ_B; x += 8) V[(size_t)x * n + j] = sV[x][q];
+  double s = 0.0;
+  if (own) {
+    s = sD[w][q];
+  } else {
+#pragma unroll 8
+    for (int x = 0; x < GJ_B; ++x) s = fma(sD[w][x], sV[x][q], s);
+    if (left) s = -s;
+  }
+  R[(size_t)(u0 + w) * n + j] = u0 + w < nb ? s : 0.0;
 }
 
-__global__ void k_gj_extract(int n, const double* __restrict__ M, double* __restrict__ inv) {
-  const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= (long long)n * n) return;
-  const long long r = t / n, cidx = t % n;
-  inv[t] = M[r * 2 * n + n + cidx];
+// upper tiles: rows outside the block M = (0 in the block's columns, M
+// elsewhere) - V^T R, rows of the block M = R
+__global__ void __launch_bounds__(256) k_gj_update(int n, int k0, double* __restrict__ M, const double* __restrict__ R,
+                                                   const double* __restrict__ V) {
+  __shared__ double sV[GJ_B][GJ_B], sR[GJ_B][GJ_B];
+  const int i0 = blockIdx.y * GJ_B, j0 = blockIdx.x * GJ_B;
+  if (i0 > j0) return;
+  const int q = threadIdx.x & 31, w = threadIdx.x >> 5;
+  for (int u = w; u < GJ_B; u += 8) {
+    sV[u][q] = i0 + q < n ? V[(size_t)u * n + i0 + q] : 0.0;
+    sR[u][q] = j0 + q < n ? R[(size_t)u * n + j0 + q] : 0.0;
+  }
+  __syncthreads();
+  double acc[4] = {0.0, 0.0, 0.0, 0.0};  // rows i0 + w + 8 a, column j0 + q
+  if (i0 != k0) {
+#pragma unroll 8
+    for (int u = 0; u < GJ_B; ++u) {
+      const double rv = sR[u][q];
+#pragma unroll
+      for (int a = 0; a < 4; ++a) acc[a] = fma(sV[u][w + 8 * a], rv, acc[a]);
+    }
+  }
+#pragma unroll
+  for (int a = 0; a < 4; ++a) {
+    const int i = i0 + w + 8 * a, j = j0 + q;
+    if (i >= n || j >= n) continue;
+    double* m = M + (size_t)i * n + j;
+    *m = i0 == k0 ? sR[w + 8 * a][q] : (j0 == k0 ? 0.0 : *m) - acc[a];
+  }
+}
+
+// the lower triangle from the upper
+__global__ void __launch_bounds__(256) k_gj_mirror(int n, double* __restrict__ M) {
+  __shared__ double t[GJ_B][GJ_B + 1];
+  const int i0 = blockIdx.y * GJ_B, j0 = blockIdx.x * GJ_B;
+  if (i0 > j0) return;
+  const int q = threadIdx.x & 31, w = threadIdx.x >> 5;
+  for (int x = w; x < GJ_B; x += 8)
+    if (i0 + x < n && j0 + q < n) t[x][q] = M[(size_t)(i0 + x) * n + j0 + q];
+  __syncthreads();
+  for (int x = w; x < GJ_B; x += 8) {
+    const int j = j0 + x, i = i0 + q;  // entry (j, i) below the diagonal
+    if (j < n && i < j) M[(size_t)j * n + i] = t[q][x];
+  }
 }
 
 // Galerkin scratch of the set-up: one buffer for every level of a handle's
@@ -1592,14 +1688,8 @@ double* setup_scratch(Ctx& c, size_t elems) {
   }
   return c.setup_Q;
 }
-// the coarsest level's matrix as the left half of the elimination's [A | I]
-__global__ void k_gj_init(int n, double* __restrict__ M) {
-  const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= (long long)n * 2 * n) return;
-  const long long r = t / (2 * n), cidx = t % (2 * n);
-  M[t] = cidx - n == r ? 1.0 : 0.0;
-}
-// a row's stencil offsets have distinct columns: plain stores
+// the coarsest level's matrix (zeroed before): a row's stencil offsets have
+// distinct columns, so the stores are plain
 __global__ void k_gj_lattice(Lat L, int kind, int no, int bs, const double* __restrict__ val, double* __restrict__ M) {
   const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= L.N * no) return;
@@ -1609,7 +1699,7 @@ __global__ void k_gj_lattice(Lat L, int kind, int no, int bs, const double* __re
   L.ijk(p, i, j, k);
   stencil_offset(kind, o, dx, dy, dz);
   if (!L.in(i + dx, j + dy, k + dz)) return;
-  const long long q = L.id(i + dx, j + dy, k + dz), w = 2 * bs * L.N;
+  const long long q = L.id(i + dx, j + dy, k + dz), w = bs * L.N;
   for (int r = 0; r < bs; ++r)
     for (int s = 0; s < bs; ++s) M[(bs * p + r) * w + bs * q + s] = val[((long long)o * bs * bs + r * bs + s) * L.N + p];
 }
@@ -1617,49 +1707,44 @@ __global__ void k_gj_lattice(Lat L, int kind, int no, int bs, const double* __re
 __global__ void k_gj_faces(int n, const int* __restrict__ col, const double* __restrict__ val, double* __restrict__ M) {
   const int f = blockIdx.x * blockDim.x + threadIdx.x;
   if (f >= n) return;
-  for (int q = 0; q < 11; ++q) M[(long long)f * 2 * n + col[(long long)q * n + f]] += val[(long long)q * n + f];
+  for (int q = 0; q < 11; ++q) M[(long long)f * n + col[(long long)q * n + f]] += val[(long long)q * n + f];
 }
 
-// The dense inverse of the coarsest level into L.dense_inv.  On a rebuild
-// (permeability update) the elimination workspace is the handle's persistent
-// one (allocated once); otherwise it is the set-up's scratch.
+// The dense inverse of the coarsest level, formed in L.dense_inv.  On a
+// rebuild (permeability update) the panels are the handle's persistent ones
+// (allocated once); otherwise they are the set-up's scratch.
 void make_dense_coarse(Ctx& c, Level& L) {
   const int n = (int)L.n;
   const bool rebuild = L.dense_inv != nullptr;
   if (!rebuild) L.dense_inv = dalloc_n<double>(c, (size_t)n * n);
-  double *M, *prow, *fcol;
-  int* err;
-  const size_t elems = (size_t)n * 2 * n + 3 * (size_t)n + 1;
-  double* ws;
-  if (rebuild) {
-    if (c.gj_n < n) {
-      c.gj_M = dalloc_n<double>(c, elems);
-      c.gj_n = n;
-    }
-    ws = c.gj_M;
-  } else {
-    ws = setup_scratch(c, elems);
+  const size_t elems = 2 * (size_t)GJ_B * n + GJ_B * GJ_B + 1;
+  if (rebuild && c.gj_n < n) {
+    c.gj_M = dalloc_n<double>(c, elems);
+    c.gj_n = n;
   }
-  M = ws;
-  prow = M + (size_t)n * 2 * n;
-  fcol = prow + 2 * (size_t)n;
-  err = (int*)(fcol + n);
+  double* R = rebuild ? c.gj_M : setup_scratch(c, elems);
+  double* V = R + (size_t)GJ_B * n;
+  double* D = V + (size_t)GJ_B * n;
+  int* err = (int*)(D + GJ_B * GJ_B);
+  double* M = L.dense_inv;
   MHFP_CUDA(cudaMemsetAsync(err, 0, sizeof(int), c.stream));
-  k_gj_init<<<grid_for((long long)n * 2 * n, 256), 256, 0, c.stream>>>(n, M);
-  MHFP_LAUNCH_CHECK();
+  MHFP_CUDA(cudaMemsetAsync(M, 0, (size_t)n * n * sizeof(double), c.stream));
   if (L.faces)
     k_gj_faces<<<grid_for(n, 128), 128, 0, c.stream>>>(n, c.ell_col, c.Cpi, M);
   else
     k_gj_lattice<<<grid_for(L.A.N * L.A.noff(), 128), 128, 0, c.stream>>>(lat_of(L.A), L.A.kind, L.A.noff(), L.A.bs,
                                                                           L.A.val, M);
   MHFP_LAUNCH_CHECK();
-  for (int col = 0; col < n; ++col) {
-    k_gj_pivot<<<grid_for(2 * n, 256), 256, 0, c.stream>>>(n, col, M, prow, fcol, err);
+  const unsigned tiles = grid_for(n, GJ_B);
+  for (int k0 = 0; k0 < n; k0 += GJ_B) {
+    k_gj_diag<<<1, GJ_TRI + 16, 0, c.stream>>>(n, k0, M, D, err);
     MHFP_LAUNCH_CHECK();
-    k_gj_update<<<dim3(grid_for(2 * n - col, 256), n), 256, 0, c.stream>>>(n, col, M, prow, fcol);
+    k_gj_panel<<<dim3(tiles, GJ_B / 8), 256, 0, c.stream>>>(n, k0, M, D, R, V);
+    MHFP_LAUNCH_CHECK();
+    k_gj_update<<<dim3(tiles, tiles), 256, 0, c.stream>>>(n, k0, M, R, V);
     MHFP_LAUNCH_CHECK();
   }
-  k_gj_extract<<<grid_for((long long)n * n, 256), 256, 0, c.stream>>>(n, M, L.dense_inv);
+  k_gj_mirror<<<dim3(tiles, tiles), 256, 0, c.stream>>>(n, M);
   MHFP_LAUNCH_CHECK();
   int h_err = 0;
   MHFP_CUDA(cudaMemcpyAsync(&h_err, err, sizeof(int), cudaMemcpyDeviceToHost, c.stream));

@@ -184,3 +184,18 @@ def test_update_keeps_the_captured_solves(precision, degree):
         assert torch.equal(x, y) and sx["iterations"] == sy["iterations"]
     used.close()
     fresh.close()
+
+
+# dense coarsest level, eliminated in blocks of 32 columns and updated in
+# tiles of 32: one level of 6 to 420 unknowns, the last block short
+@pytest.mark.parametrize("dims", [(1, 1, 1), (4, 1, 1), (2, 2, 2), (5, 3, 1), (3, 3, 3), (6, 4, 3)])
+def test_dense_level_is_the_inverse(dims):
+    prob = mi.random_small(*dims, seed=17, jitter=0.1)
+    s = _solver(prob, autotune=0, coarse_max=400)
+    rng = np.random.default_rng(2)
+    for which, n in ((0, s.sizes[0]), (1, s.sizes[2])):
+        assert s.hierarchy(which)["levels"] == 1
+        x = torch.from_numpy(rng.standard_normal(n)).cuda()
+        y = s.vcycle(which, s.level_apply(which, 0, x))
+        assert (y - x).abs().max() <= 1e-9 * x.abs().max()  # condition number up to 1.4e4
+    s.close()
