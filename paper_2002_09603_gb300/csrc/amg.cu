@@ -1108,9 +1108,48 @@ __global__ void k_build_Q(Lat F, Lat Cc, const double* __restrict__ val, const d
   for (int q = 0; q < BF * BC; ++q) Q[((long long)s * BF * BC + q) * F.N + p] = out[q];
 }
 
+// The same for the scalar lattices.  Bound by the issue of the index work: most
+// (offset, slot) pairs have no product, and a thread per slot tests all 25 or
+// 125 offsets for each of 64 slots.  Here a thread has the row of slots along x
+// in registers, so an offset's tests on y and z, its coefficient and its
+// addresses are used for the whole row.  96^3, the 25-point level: 3.39 -> 1.50 ms.
+template <int KIND>
+__global__ void __launch_bounds__(256) k_build_Q1(Lat F, Lat Cc, const double* __restrict__ val,
+                                                  const double* __restrict__ P, double* __restrict__ Q) {
+  constexpr int R = St<KIND>::R, NS = (2 + 2 * R) / 3 + 1, NQ = (2 + 4 * R) / 3 + 1;
+  const long long tid = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  if (tid >= F.N * (NQ * NQ)) return;
+  const int s = (int)(tid / F.N);
+  const long long p = tid - (long long)s * F.N;
+  int a, b, c;
+  F.ijk(p, a, b, c);
+  const int I = q_lo(a, R), J = q_lo(b, R) + s % NQ, K = q_lo(c, R) + s / NQ;
+  double acc[NQ];
+#pragma unroll
+  for (int j = 0; j < NQ; ++j) acc[j] = 0.0;
+  if ((unsigned)J < (unsigned)Cc.Ly && (unsigned)K < (unsigned)Cc.Lz) {
+    for (int o = 0; o < St<KIND>::N; ++o) {
+      int dx, dy, dz;
+      St<KIND>::off(o, dx, dy, dz);
+      const int py = J - p_lo(b + dy, R), pz = K - p_lo(c + dz, R);
+      if ((unsigned)py >= (unsigned)NS || (unsigned)pz >= (unsigned)NS) continue;
+      if (!F.in(a + dx, b + dy, c + dz)) continue;
+      const int lx = p_lo(a + dx, R) - I;  // the neighbour's first slot in the row
+      const double v = val[(long long)o * F.N + p];
+      const double* pv = P + (long long)(NS * (py + NS * pz)) * F.N + F.id(a + dx, b + dy, c + dz);
+#pragma unroll
+      for (int j = 0; j < NQ; ++j)
+        if ((unsigned)(j - lx) < (unsigned)NS) acc[j] = fma(v, pv[(long long)(j - lx) * F.N], acc[j]);
+    }
+  }
+#pragma unroll
+  for (int j = 0; j < NQ; ++j)
+    Q[((long long)NQ * s + j) * F.N + p] = (unsigned)(I + j) < (unsigned)Cc.Lx ? acc[j] : 0.0;
+}
+
 // The same for 3 x 3 blocks on the 27-point lattice, bound by the FP64 pipe
-// (125 block products, 3,375 FMA per fine point: 5.1 ms at 96^3).  In the
-// kernel above a warp's lanes have all three residues of the fine x index, so
+// (125 block products, 3,375 FMA per fine point: 5.1 ms at 96^3).  In
+// k_build_Q a warp's lanes have all three residues of the fine x index, so
 // nine (offset, slot) pairs per axis are issued for five that are not zero.
 // Here a warp takes 32 fine points of one residue RHO (a = 3 m + RHO), whose
 // products are known at compile time: x slots of the neighbours 3 n: {n - 1, n},
@@ -1856,8 +1895,12 @@ Level coarsen(Ctx& c, Level& L, Level* into = nullptr) {
           k_build_Q3<<<(unsigned)((F32.Lx + 95) / 96) * (unsigned)(A.Ly * A.Lz), 288, 0, c.stream>>>(F32, C32, A.val,
                                                                                                   L.P, Q);
         } else {
-          k_build_Q<BS.value, BS.value, K.value><<<grid_for(F.N * nq * nq * nq, 256), 256, 0, c.stream>>>(
-              F, Cc, A.val, L.P, Q);
+          // rows of slots once they give every SM a block: 8,000 points of 25
+          // offsets 28 us against 37; 343 points of 125 offsets 60 against 41
+          if (F.N * nq * nq >= 152LL * 256)
+            k_build_Q1<K.value><<<grid_for(F.N * nq * nq, 256), 256, 0, c.stream>>>(F, Cc, A.val, L.P, Q);
+          else
+            k_build_Q<1, 1, K.value><<<grid_for(F.N * nq * nq * nq, 256), 256, 0, c.stream>>>(F, Cc, A.val, L.P, Q);
         }
         MHFP_LAUNCH_CHECK();
       });

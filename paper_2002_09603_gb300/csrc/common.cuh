@@ -671,7 +671,6 @@ void fgmres_advance(Ctx& c, FgState& f);
 void solve_device_graph_launch(Ctx& c, const double* b, double tol, bool transpose);
 void solve_device_graph_finish(Ctx& c, double* x, mhfp_stats* st);
 void apply_precond(Ctx& c, const double* v, double* z, bool transpose = false);
-double device_norm2(Ctx& c, const double* x, long long n);
 void vec_scale(Ctx& c, const double* x, const double* s, bool divide, double* y, long long n);
 
 }  // namespace mhfp

@@ -509,12 +509,6 @@ void ensure_zbasis(Ctx& c) {
   }
 }
 
-double device_norm2(Ctx& c, const double* x, long long n) {
-  ensure_workspace(c);
-  norm2_dev(c, x, n, c.scal + 4);
-  return std::sqrt(read_scalar(c, c.scal + 4));
-}
-
 void vec_scale(Ctx& c, const double* x, const double* s, bool divide, double* y, long long n) {
   k_ewise<<<lgrid(grid_for(n, 256)), 256, 0, c.stream>>>(n, x, s, divide ? 1 : 0, y, lbytes());
   MHFP_LAUNCH_CHECK();

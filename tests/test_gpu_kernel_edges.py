@@ -199,3 +199,18 @@ def test_dense_level_is_the_inverse(dims):
         y = s.vcycle(which, s.level_apply(which, 0, x))
         assert (y - x).abs().max() <= 1e-9 * x.abs().max()  # condition number up to 1.4e4
     s.close()
+
+
+# the second interface-pressure level's Galerkin product, by rows of slots from
+# 2,432 cells on: one line, the first size past it, each residue mod 3 along x
+@pytest.mark.parametrize("dims", [(2600, 1, 1), (19, 16, 8), (23, 9, 12), (45, 8, 7), (20, 13, 10)])
+def test_galerkin_products_by_rows_of_slots(dims):
+    prob = mi.random_small(*dims, seed=29, jitter=0.15)
+    levels = precond.build(oracle.assemble(prob), "amg", coarse_max=60).pi_levels
+    s = _solver(prob, autotune=0, coarse_max=60)
+    rng = np.random.default_rng(4)
+    for l, lev in enumerate(levels[1:-1], 1):
+        x = rng.standard_normal(lev.A.shape[0])
+        y = s.level_apply(1, l, torch.from_numpy(x).cuda()).cpu().numpy()
+        assert np.abs(y - lev.A @ x).max() <= 1e-11 * np.abs(lev.A @ x).max()
+    s.close()
