@@ -375,12 +375,13 @@ def operator_flops(n):
 STENCIL = {"box1": 27, "diamond2": 25, "box2": 125, "faces": 11}
 
 
-def _vcycle_bytes(levels, s, fine_sym):
-    """One V(1,1) cycle with Chebyshev(2) smoothing: per non-last level a
-    zero-start step (D + 3v), three stencil steps (V + D + 5v each), a
+def _vcycle_bytes(levels, s, fine_sym, degree):
+    """One V(1,1) cycle with Chebyshev(degree) smoothing: per non-last level a
+    zero-start step (D + 3v), 2 degree - 1 stencil steps (V + D + 5v each), a
     residual (V + 3v), the restriction and prolongation (prolongator values
-    or face weights plus 3v); the last level is the FP64 dense inverse
-    (n^2 x 8 B) and two vectors."""
+    or face weights plus 3v; of the 2^3 or 3^3 slots a point has, the
+    (5/3)^3 or (7/3)^3 that are not zero by structure); the last level is the
+    FP64 dense inverse (n^2 x 8 B) and two vectors."""
     total = 0.0
     for i, (kind, N, b) in enumerate(levels):
         v, D = b * s * N, b * b * s * N
@@ -390,20 +391,20 @@ def _vcycle_bytes(levels, s, fine_sym):
             break
         K = 14 if (fine_sym and i == 0) else STENCIL[kind]
         V = K * b * b * s * N
-        slots = 8 if kind == "box1" else 27
+        slots = (5 / 3) ** 3 if kind == "box1" else (7 / 3) ** 3
         Pb = (s * N) if kind == "faces" else slots * b * b * s * N
-        total += (D + 3 * v) + 3 * (V + D + 5 * v) + (V + 3 * v) + 2 * (Pb + 3 * v)
+        total += (D + 3 * v) + (2 * degree - 1) * (V + D + 5 * v) + (V + 3 * v) + 2 * (Pb + 3 * v)
     return total
 
 
-def step_bytes(n_mesh, hu_points, hpi_points, precision, m, iters_per_step):
+def step_bytes(n_mesh, hu_points, hpi_points, precision, m, iters_per_step, degree=2):
     """Algorithmic bytes of one time step (right-hand side + FGMRES solve).
 
-    Per Arnoldi step j: the preconditioner (precision conversions, the
+    Per Arnoldi step j: the preconditioner (its scaled input, the
     interface-pressure V-cycle, the two Schur steps, the displacement
     V-cycle), the operator (float-float in the mixed form), one classical
-    Gram-Schmidt pass over the
-    j + 1 basis vectors (dots, update, normalisation) and the Givens step.
+    Gram-Schmidt pass over the j + 1 basis vectors (dots, update,
+    normalisation) and the Givens step.
     Per restart cycle: the residual (operator + norm) and x += Z y."""
     L = n_mesh + 1
     nN, nT = L ** 3, n_mesh ** 3
@@ -413,9 +414,9 @@ def step_bytes(n_mesh, hu_points, hpi_points, precision, m, iters_per_step):
     hu = [("box1", N, 3) for N in hu_points]
     hpi = [("faces", hpi_points[0], 1)] + [("diamond2" if i == 1 else "box2", N, 1)
                                            for i, N in enumerate(hpi_points) if i > 0]
-    conv = (20 + 12) * n if precision == 1 else 24 * n
+    scaled = (8 + s) * n  # D_s^-1 v: the scaling read, the input written
     schur = (6 * s + 3 * s) * nT + nF * s + 24 * s * nT + s * nT + 6 * s * nN
-    prec = conv + _vcycle_bytes(hpi, s, False) + schur + _vcycle_bytes(hu, s, precision == 1)
+    prec = scaled + _vcycle_bytes(hpi, s, False, degree) + schur + _vcycle_bytes(hu, s, precision == 1, degree)
     op = 27 * 9 * 8 * nN + 2 * 24 * 8 * nT + 11 * 8 * nF + 17 * 8 * nT + 16 * n
     # the Arnoldi step's operator: FP64, or float-float words (8 B per
     # coefficient on A_uu's symmetric half) from the FP32 z
@@ -426,7 +427,7 @@ def step_bytes(n_mesh, hu_points, hpi_points, precision, m, iters_per_step):
         steps = min(m, iters_per_step - k)
         total += op + 16 * n            # residual of the cycle and its norm
         for j in range(steps):
-            total += prec + op_arn + (2 * (j + 1) + 4) * 8 * n
+            total += prec + op_arn + (2 * (j + 1) + 5) * 8 * n
         total += (steps + 2) * 8 * n    # x += Z y
         k += steps
     total += op + 16 * n                # true residual at exit
@@ -658,7 +659,8 @@ def run_ours(args):
                        else "fallback 6.8 TB/s"}
     # the whole step against the bandwidth roofline
     mean_iters = statistics.mean(r32["iters"])
-    sb = step_bytes(n_mesh, r32["hu"], r32["hpi"], precisions[-1], r32["restart"], int(round(mean_iters)))
+    sb = step_bytes(n_mesh, r32["hu"], r32["hpi"], precisions[-1], r32["restart"], int(round(mean_iters)),
+                    r32["cheb_degree"])
     step_roof = {"bytes_per_step": sb, "achieved_gbs": sb / (ms * 1e-3) / 1e9, "peak": peak,
                  "frac": sb / (ms * 1e-3) / 1e9 / peak,
                  "model": "algorithmic bytes of every kernel of the step (bench.step_bytes), FP64 coarsest "
@@ -668,7 +670,8 @@ def run_ours(args):
     if r64 is not None and r64 is not r32:
         a64, g64 = _sweep_roofline(r64["kt"], peak)
         t64 = cheb_u0_flops(n_mesh) / (a64 * 1e-3) / 1e12 if r64["kt"]["launches"] else None
-        sb64 = step_bytes(n_mesh, r64["hu"], r64["hpi"], 0, r64["restart"], int(round(statistics.mean(r64["iters"]))))
+        sb64 = step_bytes(n_mesh, r64["hu"], r64["hpi"], 0, r64["restart"], int(round(statistics.mean(r64["iters"]))),
+                          r64["cheb_degree"])
         fp64_plain = {"ms_per_step": r64["ms"], "iterations_per_step": r64["iters"], "setup_ms": r64["setup_ms"],
                       "gpu_launches": r64["launches"], "cheb_degree": r64["cheb_degree"],
                       "sweep_roofline": {"kernel": "k_cheb_u0", "bound": "alu", "achieved": t64, "peak": fpk,
@@ -688,7 +691,7 @@ def run_ours(args):
                  "per_iteration_us": ro["split"],
                  "sweep_frac_of_hbm": go / peak if go else None,
                  "step_frac_of_hbm": step_bytes(64, ro["hu"], ro["hpi"], precisions[-1], ro["restart"],
-                                                int(round(statistics.mean(ro["iters"])))) / (ro["ms"] * 1e-3) / 1e9 / peak,
+                                                int(round(statistics.mean(ro["iters"]))), ro["cheb_degree"]) / (ro["ms"] * 1e-3) / 1e9 / peak,
                  "fp64_plain_ms_per_step": o[0][1]["ms"] if 0 in o and len(precisions) > 1 else None}
         so.close()
 
