@@ -18,6 +18,7 @@
 // on the fine lattice and A_c = P^T Q per coarse point: no atomics, no
 // sparse-matrix hashing.
 #include "lattice.cuh"
+#include "tune.h"
 #include "u64.cuh"
 
 #include <type_traits>
@@ -2217,11 +2218,9 @@ void launch_resid_sym(Ctx& c, const Level& L, const float* x, const float* b, fl
 
 // Device time of one call of `body` (which enqueues kernels on c.stream):
 // `reps` calls captured once into a CUDA graph on a private stream, the
-// graph replayed once to warm up and three times under events, the fastest
-// replay kept.  Timing graph replays leaves out host launch overhead, as in
-// the solve, which runs as graphs.  A candidate that is twice as slow as
-// `best` in its warm-up, or 1.15 times in its first timed replay, is not
-// replayed again.
+// graph uploaded and replayed up to four times under events, the fastest
+// replay kept (best_replay_us).  Timing graph replays leaves out host launch
+// overhead, as in the solve, which runs as graphs.
 template <class F>
 float graph_time_us(Ctx& c, int reps, float best_us, F&& body) {
   cudaStream_t user = c.stream, st = nullptr;
@@ -2248,30 +2247,25 @@ float graph_time_us(Ctx& c, int reps, float best_us, F&& body) {
   g_launches = l0;
   if (e == cudaSuccess) e = cudaGraphInstantiate(&ge, g, 0);
   if (g) cudaGraphDestroy(g);
-  float best = 1e30f;
+  if (e == cudaSuccess) e = cudaGraphUpload(ge, st);  // not in the first replay's time
   cudaEvent_t e0 = nullptr, e1 = nullptr;
   if (e == cudaSuccess) e = cudaEventCreate(&e0);
   if (e == cudaSuccess) e = cudaEventCreate(&e1);
-  for (int it = 0; it < 4 && e == cudaSuccess; ++it) {
-    e = cudaEventRecord(e0, st);
+  const float best = best_replay_us(best_us * reps, [&] {
+    float ms = 0.f;
+    if (e == cudaSuccess) e = cudaEventRecord(e0, st);
     if (e == cudaSuccess) e = cudaGraphLaunch(ge, st);
     if (e == cudaSuccess) e = cudaEventRecord(e1, st);
     if (e == cudaSuccess) e = cudaEventSynchronize(e1);
-    float ms = 0.f;
     if (e == cudaSuccess) e = cudaEventElapsedTime(&ms, e0, e1);
-    if (e == cudaSuccess && it > 0 && ms < best) best = ms;
-    const float us = ms * 1e3f / reps;
-    if (e == cudaSuccess && (it == 0 ? us > 2.f * best_us : us > 1.15f * best_us)) {
-      best = std::min(best, ms);
-      break;
-    }
-  }
+    return 1e3f * ms;
+  });
   if (e0) cudaEventDestroy(e0);
   if (e1) cudaEventDestroy(e1);
   if (ge) cudaGraphExecDestroy(ge);
   cudaStreamDestroy(st);
   MHFP_CUDA(e);
-  return best * 1e3f / reps;
+  return best / reps;
 }
 
 // sweeps per timed replay: about 40 us of them at 3 TB/s, 2 to 5 (ten
@@ -2279,8 +2273,9 @@ float graph_time_us(Ctx& c, int reps, float best_us, F&& body) {
 // a 96^3 set-up and 14 of 34 ms at 45 x 52 x 39)
 int tune_reps(double bytes) { return (int)std::min(5.0, std::max(2.0, 40.0 / (bytes / 3e6))); }
 
-// Set-up autotuner for the finest displacement level in FP32: time the two
-// occupancy variants of the symmetric sweep and keep the faster in L.tpp.
+// Set-up autotuner for the finest displacement level in FP32: time the four
+// occupancy variants of the symmetric sweep and the bulk-copy-fed one and keep
+// the fastest in L.tpp.
 void autotune_fine_sym(Ctx& c, Level& L) {
   MHFP_CUDA(cudaMemsetAsync(L.bf, 0, L.n * sizeof(float), c.stream));
   MHFP_CUDA(cudaMemsetAsync(L.xf, 0, L.n * sizeof(float), c.stream));
