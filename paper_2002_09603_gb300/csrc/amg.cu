@@ -1712,14 +1712,24 @@ __global__ void __launch_bounds__(256) k_gj_mirror(int n, double* __restrict__ M
 
 // Galerkin scratch of the set-up: one buffer for every level of a handle's
 // hierarchies (the first level of the first one needs the most), given back
-// by release_setup_scratch once they are built
+// when the scope that builds them ends, also by an exception
 void release_setup_scratch(Ctx& c) {
   if (!c.setup_Q) return;
-  MHFP_CUDA(cudaStreamSynchronize(c.stream));  // its last kernel may still run
-  dfree(c, c.setup_Q);
+  void* q = c.setup_Q;
   c.setup_Q = nullptr;
   c.setup_Q_elems = 0;
+  MHFP_CUDA(cudaStreamSynchronize(c.stream));  // its last kernel may still run
+  dfree(c, q);
 }
+struct SetupScratch {
+  Ctx& c;
+  ~SetupScratch() {
+    try {
+      release_setup_scratch(c);
+    } catch (...) {  // stays with the handle; the next check reports the device's error
+    }
+  }
+};
 double* setup_scratch(Ctx& c, size_t elems) {
   if (c.setup_Q_elems < elems) {
     release_setup_scratch(c);
@@ -2509,10 +2519,12 @@ void make_fp32(Ctx& c, std::vector<Level>& H, bool fine_sym) {
 }  // namespace
 
 void build_hierarchies(Ctx& c) {
-  if (c.opt.near_kernel == 1) build_u_rbm(c);
-  else build_u(c);
-  build_pi(c);
-  release_setup_scratch(c);
+  {
+    const SetupScratch scratch{c};
+    if (c.opt.near_kernel == 1) build_u_rbm(c);
+    else build_u(c);
+    build_pi(c);
+  }
   if (c.opt.precision == 1) {
     make_fp32(c, c.hu, true);
     make_fp32(c, c.hpi, false);
@@ -2588,11 +2600,9 @@ void rebuild_pi_hierarchy(Ctx& c) {
   }
 }
 
-// The mixed formulation's inner solvers (opt.formulation = 1): the
-// displacement hierarchy as for the hybrid form, A_qq as a single face level
-// (its Chebyshev smoother stands for the paper's incomplete Cholesky), and
-// the smoothed-aggregation hierarchy of C~_p started on the cell lattice.
-void build_mixed_hierarchies(Ctx& c) {
+namespace {
+void build_mixed_levels(Ctx& c) {
+  const SetupScratch scratch{c};
   if (c.opt.near_kernel == 1) build_u_rbm(c);
   else build_u(c);
   c.hq.clear();
@@ -2627,7 +2637,15 @@ void build_mixed_hierarchies(Ctx& c) {
   Level& last = c.hcp.back();
   alloc_work(c, last);
   make_dense_coarse(c, last);
-  release_setup_scratch(c);
+}
+}  // namespace
+
+// The mixed formulation's inner solvers (opt.formulation = 1): the
+// displacement hierarchy as for the hybrid form, A_qq as a single face level
+// (its Chebyshev smoother stands for the paper's incomplete Cholesky), and
+// the smoothed-aggregation hierarchy of C~_p started on the cell lattice.
+void build_mixed_hierarchies(Ctx& c) {
+  build_mixed_levels(c);
   make_fp64_transfers(c, c.hu);
   make_fp64_transfers(c, c.hcp);
   if (c.opt.autotune)
