@@ -31,10 +31,10 @@ namespace mhfp {
 namespace {
 
 // <hot:k_cheb_u0> (bench.py hashes this region to tell whether profiles/traffic.json still applies)
-// Chebyshev step of the finest displacement level in FP64 (the rows and the
-// two forms: u64.cuh): r = b - A xin, d = cd d + cr D^-1 r, xout = xin + d.
-template <int SPLIT>
-__global__ void __launch_bounds__(SPLIT ? 9 * U64_NODES : U64_NODES_1)
+// Chebyshev step of the finest displacement level in FP64 (the rows, the forms
+// and their times: u64.cuh): r = b - A xin, d = cd d + cr D^-1 r, xout = xin + d.
+template <U64Form F>
+__global__ void __launch_bounds__(u64_threads(F), F == U64_ROW ? 13 : 0)
     k_cheb_u0(Lat32 L, const double* __restrict__ val, const double* __restrict__ dinv, const double* __restrict__ b,
               const double* __restrict__ xin, double* __restrict__ xout, double* __restrict__ d,
               const double* __restrict__ cf, bool first, long long lb) {
@@ -44,25 +44,10 @@ __global__ void __launch_bounds__(SPLIT ? 9 * U64_NODES : U64_NODES_1)
   xout = lane_ptr(xout, lb);
   d = lane_ptr(d, lb);
   const long long N = L.N;
-  if (SPLIT) {
-    __shared__ double rs[3][U64_NODES];
-    const unsigned n = blockIdx.x * U64_NODES + threadIdx.x;
-    const int comp = threadIdx.y % 3, s = threadIdx.y / 3;
-    const bool valid = n < (unsigned)N;
-    const double v = u64_row_split(L, n, valid, comp, s, val, xin, nullptr, 0.0);
-    const long long r = 3LL * n + comp;
-    if (s == 0) rs[comp][threadIdx.x] = valid ? b[r] - v : 0.0;
-    __syncthreads();
-    if (!valid || s != 0) return;
-    double z = 0.0;
-#pragma unroll
-    for (int t = 0; t < 3; ++t) z += dinv[(3 * comp + t) * N + n] * rs[t][threadIdx.x];
-    const double dn = first ? cr * z : cd * d[r] + cr * z;
-    d[r] = dn;
-    xout[r] = xin[r] + dn;
-  } else {
-    const unsigned n = blockIdx.x * U64_NODES_1 + threadIdx.x;
-    if (n >= (unsigned)N) return;
+  const unsigned n = blockIdx.x * u64_nodes(F) + threadIdx.x;
+  const bool valid = n < (unsigned)N;
+  if (F == U64_NODE) {
+    if (!valid) return;
     double acc[3] = {0.0, 0.0, 0.0};
     u64_rows(L, n, val, xin, nullptr, 0.0, acc);
 #pragma unroll
@@ -77,6 +62,22 @@ __global__ void __launch_bounds__(SPLIT ? 9 * U64_NODES : U64_NODES_1)
       d[r] = dn;
       xout[r] = xin[r] + dn;
     }
+  } else {
+    __shared__ double rs[3][u64_nodes(F)];
+    const int comp = threadIdx.y % 3, s = threadIdx.y / 3;
+    const long long r = 3LL * n + comp;
+    double v = 0.0;
+    if (F == U64_SPLIT) v = u64_row_split(L, n, valid, comp, s, val, xin, nullptr, 0.0);
+    else if (valid) v = u64_row(L, n, comp, val, xin, nullptr, 0.0);
+    if (s == 0) rs[comp][threadIdx.x] = valid ? b[r] - v : 0.0;
+    __syncthreads();
+    if (!valid || s != 0) return;
+    double z = 0.0;
+#pragma unroll
+    for (int t = 0; t < 3; ++t) z += dinv[(3 * comp + t) * N + n] * rs[t][threadIdx.x];
+    const double dn = first ? cr * z : cd * d[r] + cr * z;
+    d[r] = dn;
+    xout[r] = xin[r] + dn;
   }
 }
 // </hot:k_cheb_u0>
@@ -2368,12 +2369,12 @@ void smooth(Ctx& c, std::vector<Level>& H, int l, const T* b, const T* x0, T* ds
         const Lat32 lat = lat32_of(L.A);
         if (!xin)  // the first step from zero has no stencil work
           sweep_cheb_zero<T>(c.stream, lat.N, 3, v.dinv, b, out, v.d, v.cf);
-        else if (lat.N <= U64_SPLIT_NODES)
-          k_cheb_u0<1><<<lgrid(grid_for(lat.N, U64_NODES)), dim3(U64_NODES, 9), 0, c.stream>>>(
-              lat, v.val, v.dinv, b, xin, out, v.d, v.cf + 2 * s, s == 0, lbytes());
         else
-          k_cheb_u0<0><<<lgrid(grid_for(lat.N, U64_NODES_1)), U64_NODES_1, 0, c.stream>>>(
-              lat, v.val, v.dinv, b, xin, out, v.d, v.cf + 2 * s, s == 0, lbytes());
+          dispatch_u64(lat.N, U64_ROW_STEP, [&](auto F) {
+            constexpr U64Form f = decltype(F)::value;
+            k_cheb_u0<f><<<u64_grid<f>(lat.N), u64_block<f>(), 0, c.stream>>>(
+                lat, v.val, v.dinv, b, xin, out, v.d, v.cf + 2 * s, s == 0, lbytes());
+          });
       }
     } else {
       launch_cheb<T>(c, L, v, b, xin, out, s, L.tpp ? L.tpp : default_schedule(L.A, v.rows != nullptr));

@@ -4,32 +4,45 @@
 //
 // Large levels are bound by the FP64 pipe (243 FMA per node at 608 GFMA/s:
 // 0.40 ns; 1,944 B at 6.8 TB/s: 0.29 ns), small ones by the latency of the
-// stencil's serial chain.  Two forms:
-//  * SPLIT = 0: a thread per node and its three rows; x is read once for nine
-//    products, a pencil (three blocks) of loads ahead of its products.
-//  * SPLIT = 1: nine threads per node, one per (component, stencil plane) and
+// stencil's serial chain.  Three forms, in the order of the number of threads:
+//  * U64_SPLIT: nine threads per node, one per (component, stencil plane) and
 //    27 products each; the planes' partial sums meet in shared memory and are
 //    added in plane order.
-// Measured, microseconds, SPLIT = 1 / SPLIT = 0 / the loop they replace (a
-// thread per node over 27 offsets; for the operator a thread per row):
-//     nodes      residual            Chebyshev step      operator rows
-//       729     4.2 / 13.1 / 24      5.1 / 20.8 / 23.0   4.7 / 14.7 / 11.8
-//     9,261     6.2 / 13.3 / 25      6.9 / 21.4 / 23.5   7.0 / 14.9 / 12.2
-//    68,921    35.9 / 36.1 / 60     40.1 / 55.2 / 56.0  39.9 / 41.4 / 41.7
-//   148,877    72.0 / 72.8 / -      79.9 / 75.4 / 75.1  80.4 / 82.3 / 79.8
-//   274,625     129 / 122  / 196     142 / 146  / 143    144 / 138  / 138
-// 2,146,689     966 / 886  / 1580   1079 / 971  / 961   1083 / 1014 / 1007
-// so levels up to U64_SPLIT_NODES take SPLIT = 1 (the FP64 pipe's time at
-// 2,146,689 nodes: 858, 890 and 943).
+//  * U64_ROW: three threads per node, one per row; the three planes unrolled,
+//    40 registers, so that 16 blocks of 96 threads fit an SM (the Chebyshev
+//    step: 48 and 13, without which it spills).
+//  * U64_NODE: a thread per node and its three rows; x is read once for nine
+//    products.
+// U64_ROW and U64_NODE sum a row in the same order (the same bits).
+// Microseconds, calls in a row / L2 flushed before each; "loop" is what they
+// replace (a thread per node over 27 offsets; for the operator a thread per row):
+//     nodes  residual                     Chebyshev step                      operator rows
+//            SPLIT   NODE    ROW          SPLIT   NODE    ROW     loop        SPLIT   NODE    ROW     loop
+//     9,261  10/14   18/30   -            11/14   29/59   -       39/92       11/14   18/32   -       16/29
+//    54,872  33/37   33/41   35/37        35/39   57/68   37/41   86/103      37/41   37/45   39/37   36/41
+//    68,921  41/47   41/45   41/45        43/49   55/62   45/49   96/105      45/51   45/49   47/45   47/45
+//   117,649  64/67   66/65   60/63        66/71   66/70   65/69   98/107      70/74   72/72   68/71   72/75
+//   274,625  133/139 125/127 125/125      142/147 145/152 133/134 150/152     148/153 140/141 141/141 142/144
+//   531,441  249/254 231/232 233/233      256/261 256/258 248/249 258/263     278/282 260/260 263/264 263/264
+//   912,673  419/424 386/387 393/393      446/450 424/424 416/417 443/446     468/473 434/436 445/445 439/441
+// 2,146,689  943/949 856/858 873/875      1003    932/933 928/930 942/948     1053    967/968 986/987 974/977
+// (the step in a solve, where the vectors lie elsewhere: 274,625 nodes 150 NODE,
+// 130 ROW, 145 loop; 2,146,689 nodes 932, 944 and 929).  So U64_SPLIT up to
+// U64_SPLIT_NODES, where it and the row form change places, U64_NODE for rows
+// and residuals from U64_ROW_ROWS nodes on and for the step from U64_ROW_STEP
+// on, U64_ROW between (the FP64 pipe's time at 2,146,689 nodes: 858, 890 and 943).
 #pragma once
 #include "lattice.cuh"
 
 namespace mhfp {
 namespace {
 
-constexpr long long U64_SPLIT_NODES = 120000;
-constexpr int U64_NODES = 32;      // nodes per block, SPLIT = 1 (288 threads)
-constexpr int U64_NODES_1 = 128;   // nodes and threads per block, SPLIT = 0
+enum U64Form { U64_NODE, U64_SPLIT, U64_ROW };
+constexpr long long U64_SPLIT_NODES = 60000, U64_ROW_ROWS = 450000, U64_ROW_STEP = 1500000;
+constexpr int u64_nodes(U64Form f) { return f == U64_NODE ? 128 : 32; }  // nodes per block
+constexpr int u64_parts(U64Form f) { return f == U64_SPLIT ? 9 : (f == U64_ROW ? 3 : 1); }  // threads per node
+constexpr int u64_threads(U64Form f) { return u64_nodes(f) * u64_parts(f); }
+constexpr int u64_blocks(U64Form f) { return f == U64_ROW ? 16 : 0; }  // per SM, at least (0: not asked for)
 
 // out = so ? so[r] * (bsub ? bsub[r] - y : y) : (bsub ? bsub[r] - y : y)
 __device__ __forceinline__ double finish(double y, long long r, const double* so, const double* bsub) {
@@ -114,12 +127,12 @@ __device__ __forceinline__ void u64_rows(const Lat32& L, unsigned n, const doubl
   }
 }
 
-// SPLIT = 1: row (node, component) of the same; the planes' parts joined in
+// U64_SPLIT: row (node, component) of the same; the planes' parts joined in
 // plane 0, where the sum is returned.  Every thread of the block calls it.
 __device__ __forceinline__ double u64_row_split(const Lat32& L, unsigned n, bool valid, int comp, int s,
                                                 const double* __restrict__ A, const double* __restrict__ x,
                                                 const double* __restrict__ Aup, double cup) {
-  __shared__ double part[2][3][U64_NODES];
+  __shared__ double part[2][3][u64_nodes(U64_SPLIT)];
   double acc[1] = {0.0};
   if (valid) {
     int i, j, k;
@@ -133,26 +146,46 @@ __device__ __forceinline__ double u64_row_split(const Lat32& L, unsigned n, bool
   return s == 0 ? (acc[0] + part[0][comp][threadIdx.x]) + part[1][comp][threadIdx.x] : 0.0;
 }
 
+// U64_ROW: row (node, component) by one thread
+__device__ __forceinline__ double u64_row(const Lat32& L, unsigned n, int comp, const double* __restrict__ A,
+                                          const double* __restrict__ x, const double* __restrict__ Aup, double cup) {
+  double acc[1] = {0.0};
+  int i, j, k;
+  L.ijk(n, i, j, k);
+#pragma unroll
+  for (int dz = -1; dz <= 1; ++dz)
+#pragma unroll
+    for (int dy = -1; dy <= 1; ++dy) u64_pencil<1>(L, n, i, j, k, dy, dz, comp, A, x, acc);
+  if (Aup) {
+#pragma unroll 1
+    for (int uz = 0; uz < 2; ++uz) u64_cells<1>(L, i, j, k, uz, comp, Aup, x + 3LL * L.N, cup, acc);
+  }
+  return acc[0];
+}
+
 // y = b - A x (y = A x when b is null); with Aup the operator's u rows, y =
 // finish(A_uu x_u + cup A_up x_p) with so and b
-template <int SPLIT>
-__global__ void __launch_bounds__(SPLIT ? 9 * U64_NODES : U64_NODES_1)
+template <U64Form F>
+__global__ void __launch_bounds__(u64_threads(F), u64_blocks(F))
     k_u64(Lat32 L, const double* __restrict__ A, const double* __restrict__ Aup, double cup,
           const double* __restrict__ x, const double* __restrict__ so, const double* __restrict__ b,
           double* __restrict__ y, long long lb) {
   x = lane_ptr(x, lb);
   b = lane_ptr(b, lb);
   y = lane_ptr(y, lb);
-  if (SPLIT) {
-    const unsigned n = blockIdx.x * U64_NODES + threadIdx.x;
+  const unsigned n = blockIdx.x * u64_nodes(F) + threadIdx.x;
+  const bool valid = n < (unsigned)L.N;
+  if (F == U64_SPLIT) {
     const int comp = threadIdx.y % 3, s = threadIdx.y / 3;
-    const bool valid = n < (unsigned)L.N;
     const double v = u64_row_split(L, n, valid, comp, s, A, x, Aup, cup);
     const long long r = 3LL * n + comp;
     if (valid && s == 0) y[r] = finish(v, r, so, b);
+  } else if (F == U64_ROW) {
+    if (!valid) return;
+    const long long r = 3LL * n + threadIdx.y;
+    y[r] = finish(u64_row(L, n, threadIdx.y, A, x, Aup, cup), r, so, b);
   } else {
-    const unsigned n = blockIdx.x * U64_NODES_1 + threadIdx.x;
-    if (n >= (unsigned)L.N) return;
+    if (!valid) return;
     double acc[3] = {0.0, 0.0, 0.0};
     u64_rows(L, n, A, x, Aup, cup, acc);
 #pragma unroll
@@ -160,12 +193,25 @@ __global__ void __launch_bounds__(SPLIT ? 9 * U64_NODES : U64_NODES_1)
   }
 }
 
+// f(form) with the form for N nodes, `row` the first size past the row form's
+template <class F>
+void dispatch_u64(long long N, long long row, F&& f) {
+  if (N <= U64_SPLIT_NODES) f(std::integral_constant<U64Form, U64_SPLIT>{});
+  else if (N < row) f(std::integral_constant<U64Form, U64_ROW>{});
+  else f(std::integral_constant<U64Form, U64_NODE>{});
+}
+
+template <U64Form F>
+dim3 u64_grid(long long N) { return lgrid(grid_for(N, u64_nodes(F))); }
+template <U64Form F>
+dim3 u64_block() { return dim3(u64_nodes(F), u64_parts(F)); }
+
 template <class... Args>
 void launch_u64(cudaStream_t stream, const Lat32& L, Args... args) {
-  if (L.N <= U64_SPLIT_NODES)
-    k_u64<1><<<lgrid(grid_for(L.N, U64_NODES)), dim3(U64_NODES, 9), 0, stream>>>(L, args..., lbytes());
-  else
-    k_u64<0><<<lgrid(grid_for(L.N, U64_NODES_1)), U64_NODES_1, 0, stream>>>(L, args..., lbytes());
+  dispatch_u64(L.N, U64_ROW_ROWS, [&](auto F) {
+    constexpr U64Form f = decltype(F)::value;
+    k_u64<f><<<u64_grid<f>(L.N), u64_block<f>(), 0, stream>>>(L, args..., lbytes());
+  });
 }
 
 }  // namespace

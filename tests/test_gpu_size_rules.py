@@ -1,0 +1,62 @@
+"""The forms that the rules on sizes choose above the other tests' meshes,
+against the FP64 oracle (tolerances as in test_gpu_parity): one mesh of 68,880
+nodes and 63,960 cells with odd sides."""
+import numpy as np
+import pytest
+
+import mhfp_inputs as mi
+import oracle
+from oracle import precond, system
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _built():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import __graft_entry__
+    __graft_entry__.build()
+
+
+@pytest.fixture(scope="module")
+def mesh(_built):
+    prob = mi.random_small(41, 40, 39, seed=11, jitter=0.2)
+    return prob, oracle.assemble(prob)
+
+
+@pytest.fixture(scope="module")
+def oracle_pc(mesh):
+    return precond.build(mesh[1], "amg")
+
+
+def _solver(prob, **opts):
+    from paper_2002_09603_gb300 import default_options, prepare
+    o = default_options()
+    for k, v in opts.items():
+        setattr(o, k, v)
+    return prepare(prob, o)
+
+
+def _vcycle_close(s, which, ref, b, tol):
+    got = s.vcycle(which, torch.from_numpy(b).cuda()).cpu().numpy()
+    assert np.abs(got - ref).max() <= tol * np.abs(ref).max()
+
+
+# FP64 displacement rows by a thread per row (60,001 nodes and up): both
+# operators, and the sweeps and the residual of the V-cycle
+def test_fp64_rows_by_a_thread_per_row(mesh, oracle_pc):
+    prob, B = mesh
+    s = _solver(prob, autotune=0)
+    A = system.system_matrix(B)
+    rng = np.random.default_rng(4)
+    x, b = rng.standard_normal(s.n), rng.standard_normal(s.sizes[0])
+    xd = torch.from_numpy(x).cuda()
+    for f, M in ((s.apply_operator, A), (s.apply_operator_t, A.T)):
+        y, ref, o = f(xd).cpu().numpy(), M @ x, 0
+        for n in B.sizes:
+            assert np.abs(y[o:o + n] - ref[o:o + n]).max() <= 1e-12 * np.abs(ref[o:o + n]).max()
+            o += n
+    _vcycle_close(s, 0, precond.vcycle(oracle_pc.u_levels, b), b, 1e-10)
+    s.close()
