@@ -1,0 +1,35 @@
+"""Device functions and kernels called directly, by small CUDA programs that are
+compiled here (each says in its header what it compares with what)."""
+import os
+import subprocess
+import tempfile
+
+import pytest
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+HERE = os.path.dirname(os.path.abspath(__file__))
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _built():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import __graft_entry__
+    __graft_entry__.build()
+
+
+def _run(source, *flags):
+    from paper_2002_09603_gb300 import build
+    with tempfile.TemporaryDirectory() as d:
+        exe = os.path.join(d, "check")
+        r = subprocess.run([build.nvcc(), "-std=c++17", "-O2", "--expt-relaxed-constexpr", *build.ARCH,
+                            os.path.join(HERE, source), "-o", exe, *flags],
+                           capture_output=True, text=True, timeout=300)
+        assert r.returncode == 0, r.stderr[-2000:]
+        r = subprocess.run([exe], capture_output=True, text=True, timeout=300)
+        assert r.returncode == 0 and r.stdout.strip() == "ok", r.stdout[-2000:] + r.stderr[-2000:]
+
+
+def test_conversions_over_every_branch():
+    _run("conversion_check.cu")
