@@ -33,3 +33,9 @@ def _run(source, *flags):
 
 def test_conversions_over_every_branch():
     _run("conversion_check.cu")
+
+
+def test_sweeps_under_every_schedule():
+    from paper_2002_09603_gb300 import LIB_PATH
+    lib = os.path.dirname(os.path.abspath(LIB_PATH))
+    _run("sweep_check.cu", "-L" + lib, "-lmhfp", "-Xlinker", "-rpath=" + lib)
