@@ -1536,7 +1536,7 @@ void level_spmv(Ctx& c, Level& L, const double* x, const double* b, double* y) {
     launch_u64(c.stream, lat32_of(L.A), (const double*)L.A.val, (const double*)nullptr, 0.0, x,
                (const double*)nullptr, b, y);
   } else {
-    launch_spmv<double>(c, L.A, L.bs, L.A.val, L.rowd, x, b, y, default_schedule(L.A, L.rowd != nullptr));
+    launch_spmv<double>(c, L.A, L.bs, L.A.val, L.rowd, x, b, y, default_schedule(L.A, L.rowd != nullptr, false));
   }
   MHFP_LAUNCH_CHECK();
 }
@@ -2138,7 +2138,7 @@ void level_spmv_t(Ctx& c, Level& L, const T* x, const T* b, T* y) {
   if (L.faces) {
     k_spmv_ell<T><<<lgrid(grid_for(L.n, 256)), 256, 0, c.stream>>>(face_topo(c), v.ell, x, b, y, lbytes());
   } else {
-    launch_spmv<T>(c, L.A, L.bs, v.val, v.rows, x, b, y, L.tpp ? L.tpp : default_schedule(L.A, v.rows != nullptr));
+    launch_spmv<T>(c, L.A, L.bs, v.val, v.rows, x, b, y, L.tpp ? L.tpp : default_schedule(L.A, v.rows != nullptr, sizeof(T) == 4));
   }
   MHFP_LAUNCH_CHECK();
 }
@@ -2318,7 +2318,7 @@ void autotune_level(Ctx& c, Level& L) {
   MHFP_CUDA(cudaMemsetAsync(x, 0, L.n * sizeof(T), c.stream));
   MHFP_CUDA(cudaMemsetAsync(v.d, 0, L.n * sizeof(T), c.stream));
   float best = 1e30f;
-  int best_tpp = default_schedule(L.A, v.rows != nullptr);
+  int best_tpp = default_schedule(L.A, v.rows != nullptr, sizeof(T) == 4);
   // likely winners first: a candidate that has lost is dropped early
   const std::vector<int> cand = v.rows ? std::vector<int>{32, 64, 8, 4, 16} : std::vector<int>{1, 4, 8, 16};
   for (int tpp : cand) {
@@ -2377,7 +2377,7 @@ void smooth(Ctx& c, std::vector<Level>& H, int l, const T* b, const T* x0, T* ds
           });
       }
     } else {
-      launch_cheb<T>(c, L, v, b, xin, out, s, L.tpp ? L.tpp : default_schedule(L.A, v.rows != nullptr));
+      launch_cheb<T>(c, L, v, b, xin, out, s, L.tpp ? L.tpp : default_schedule(L.A, v.rows != nullptr, sizeof(T) == 4));
     }
     MHFP_LAUNCH_CHECK();
     // algorithmic bytes of a Chebyshev sweep: the matrix values (27 blocks
@@ -2673,7 +2673,8 @@ void chebyshev_from_zero(Ctx& c, std::vector<Level>& H, const double* b, double*
 int level_schedule(Ctx& c, std::vector<Level>& H, int l) {
   const Level& L = H[l];
   if (&H == &c.hu && l == 0) return L.symf ? sym_minb(L) : 0;  // FP64: the full-storage k_cheb_u0
-  return L.tpp ? L.tpp : default_schedule(L.A, (c.opt.precision == 1 ? (void*)L.rowf : (void*)L.rowd) != nullptr);
+  const bool fp32 = c.opt.precision == 1;
+  return L.tpp ? L.tpp : default_schedule(L.A, (fp32 ? (void*)L.rowf : (void*)L.rowd) != nullptr, fp32);
 }
 
 // timed as class 4 (displacement) or 5 (interface pressure)

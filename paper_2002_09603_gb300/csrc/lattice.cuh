@@ -180,23 +180,24 @@ inline Lat32 lat32_of(const StructOp& A) {
 // or eight lanes, per point on row-major values, which box levels have up to
 // the size where a split schedule is as fast (row_level).  The set-up
 // autotuner times all that apply.  Without it: row-major levels take a warp
-// per point up to 2,048 points and eight lanes above (27-point 3 x 3 levels
-// eight warps), other scalar levels of 64K points and up one point per thread
-// and the rest eight warps.  Microseconds of a Chebyshev step, best split /
-// warp per point / eight lanes:
-//   125-point FP32:  1,000 5.1 / 2.0 / 2.4; 10,648 5.8 / 4.5 / 3.6; 32,768 6.4 / 10 / 7.1
-//   125-point FP64:  1,000 11.6 / 2.7 / 3.5; 10,648 15.3 / 11.6 / 6.0; 32,768 19 / 32 / 14
-//   3 x 3 FP32:      1,000 2.9 / 2.0 / 4.0;  3,375 3.1 / 2.7 / 4.2;   10,648 4.2 / 5.2 / 5.4
-//   3 x 3 FP64:      343 5.8 / 3.2 / 5.2;    3,375 6.2 / 9.2 / 6.2
-//   6 x 6 FP32:      216 6.0 / 3.0 / 7.6;    4,096 8.4 / 4.7 / 8.4;   10,648 9.3 / 8.3 / 9.7
-//   6 x 6 FP64:      216 14.9 / 5.3 / 9.2;   4,096 15.9 / 22 / 13.4
+// per point up to 2,048 points, and in FP32 with 3 or 6 unknowns per point at
+// any size; above, scalar and 6 x 6 levels take eight lanes and 3 x 3 levels
+// eight warps; other scalar levels of 64K points and up one point per thread
+// and the rest eight warps.  Microseconds of a Chebyshev step, eight warps / best
+// split / warp per point / eight lanes:
+//   125-point FP32:  1,000 5.4 / 5.0 / 1.9 / 2.4;    10,648 5.9 / 5.8 / 4.5 / 3.5;    32,768 10.9 / 6.3 / 10.6 / 7.0
+//   125-point FP64:  1,000 11.6 / 11.6 / 2.7 / 3.7;  10,648 21.0 / 15.4 / 10.8 / 5.9; 32,768 46.9 / 19.0 / 29.2 / 13.2
+//   3 x 3 FP32:      1,000 3.6 / 3.1 / 2.0 / 3.6;    2,744 3.7 / 3.2 / 2.6 / 3.8;     4,096 3.8 / 3.2 / 3.0 / 3.9
+//   3 x 3 FP64:      1,000 6.0 / 6.0 / 4.1 / 5.4;    2,744 6.3 / 6.3 / 7.5 / 6.4;     4,096 6.4 / 6.4 / 10.1 / 6.6
+//   6 x 6 FP32:      2,744 8.7 / 8.2 / 3.8 / 8.3;    8,000 10.1 / 9.3 / 6.8 / 9.0;    16,384 17.6 / 15.6 / 12.5 / 13.2
+//   6 x 6 FP64:      1,728 15.4 / 15.4 / 10.1 / 10.3; 4,096 15.9 / 15.9 / 21.7 / 13.5; 16,384 89 / 62 / 79 / 48
 inline bool row_level(const StructOp& A) {
   if (A.kind == ST_DIAMOND2) return false;
   return A.N <= (A.bs == 1 ? 32768 : (A.bs == 3 ? 4096 : 16384));
 }
 inline int row_lanes(int sched) { return sched == 32 ? 32 : (sched == 64 ? 8 : 0); }
-inline int default_schedule(const StructOp& A, bool rows) {
-  if (rows) return A.N <= 2048 ? 32 : (A.bs == 3 ? 8 : 64);
+inline int default_schedule(const StructOp& A, bool rows, bool fp32) {
+  if (rows) return A.N <= 2048 || (fp32 && A.bs > 1) ? 32 : (A.bs == 3 ? 8 : 64);
   return (A.bs == 1 && A.N >= 65536) ? 1 : 8;
 }
 
