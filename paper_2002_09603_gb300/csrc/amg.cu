@@ -2438,12 +2438,16 @@ void vcycle_level(Ctx& c, std::vector<Level>& H, int l, const T* b, T* x, bool p
       constexpr int R = transfer_r<BF.value>();
       // four warps per coarse point where one each would leave SMs idle, and
       // for the blocks of the rigid-body modes (one box point per lane)
-      if (C.A.N < RESTRICT_WIDE || BF.value * BC.value > 9)
-        k_restrict_f<BF.value, BC.value, R, 4, T><<<lgrid(grid_for(C.A.N, 2)), 256, 0, c.stream>>>(
+      auto launch = [&](auto W) {
+        k_restrict_f<BF.value, BC.value, R, W.value, T><<<lgrid(grid_for(C.A.N, 8 / W.value)), 256, 0, c.stream>>>(
             F, Cc, v.P, v.r, cb, fdinv, fcr, fx, fd, lbytes());
-      else
-        k_restrict_f<BF.value, BC.value, R, 1, T><<<lgrid(grid_for(C.A.N, 8)), 256, 0, c.stream>>>(
-            F, Cc, v.P, v.r, cb, fdinv, fcr, fx, fd, lbytes());
+      };
+      if constexpr (BF.value * BC.value > 9) {
+        launch(std::integral_constant<int, 4>{});
+      } else {
+        if (C.A.N < RESTRICT_WIDE) launch(std::integral_constant<int, 4>{});
+        else launch(std::integral_constant<int, 1>{});
+      }
     });
   }
   MHFP_LAUNCH_CHECK();
@@ -2454,15 +2458,15 @@ void vcycle_level(Ctx& c, std::vector<Level>& H, int l, const T* b, T* x, bool p
     const Lat32 F = lat32_of(L.A), Cc = lat32_of(C.A);
     dispatch_pair(L.bs, C.bs, [&](auto BF, auto BC) {
       constexpr int R = transfer_r<BF.value>();
-      if (L.A.N >= PROLONG_WIDE && BF.value == 1)
-        k_prolong_s<R, T><<<lgrid(grid_for(L.A.N, 256)), 256, 0, c.stream>>>(F, Cc, v.P, cx, s_buf, lbytes());
-      else if (L.A.N >= PROLONG_WIDE)
-        k_prolong_f<BF.value, BC.value, R, T>
-            <<<lgrid(grid_for(L.A.N, 32)), dim3(32, Box<R>::ns * Box<R>::ns), 0, c.stream>>>(F, Cc, v.Pm, cx, s_buf,
-                                                                                             lbytes());
-      else
+      if (L.A.N < PROLONG_WIDE)
         k_prolong_w<BF.value, BC.value, R, T>
             <<<lgrid(grid_for(L.A.N, 32)), dim3(32, Box<R>::ns * Box<R>::ns), 0, c.stream>>>(F, Cc, v.P, cx, s_buf,
+                                                                                             lbytes());
+      else if constexpr (BF.value == 1)
+        k_prolong_s<R, T><<<lgrid(grid_for(L.A.N, 256)), 256, 0, c.stream>>>(F, Cc, v.P, cx, s_buf, lbytes());
+      else
+        k_prolong_f<BF.value, BC.value, R, T>
+            <<<lgrid(grid_for(L.A.N, 32)), dim3(32, Box<R>::ns * Box<R>::ns), 0, c.stream>>>(F, Cc, v.Pm, cx, s_buf,
                                                                                              lbytes());
     });
   }

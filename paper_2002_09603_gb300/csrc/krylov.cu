@@ -463,12 +463,6 @@ void norm2_dev(Ctx& c, const double* x, long long n, double* dst) {
   MHFP_LAUNCH_CHECK();
 }
 
-double read_scalar(Ctx& c, const double* dsrc) {
-  MHFP_CUDA(cudaMemcpyAsync(c.host_scal, dsrc, sizeof(double), cudaMemcpyDeviceToHost, c.stream));
-  MHFP_CUDA(cudaStreamSynchronize(c.stream));
-  return c.host_scal[0];
-}
-
 }  // namespace
 
 void ensure_workspace(Ctx& c) {
