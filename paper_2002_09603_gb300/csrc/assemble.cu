@@ -806,11 +806,13 @@ __device__ __forceinline__ void ff_mac(float& sh, float& sl, float ah, float al,
 // One launch for all rows: blocks of 256 rows take the five row families (u
 // nodes, cells, x-, y- and z-faces; about as many blocks each) in turn, so
 // that the families sweep the mesh in z together and what two of them read
-// (A_up by the u and p rows, A_ppi by the p and pi rows, z by all) comes from
-// HBM once and from L2 the second time.  Bound by L2: about 9.6 TB/s of
-// coefficients (A_uu's lower blocks are read a second time there) against
-// 3.47 GB from HBM.  128^3: 762 us, 787 us as three launches (497 + 120 + 170);
-// 64^3: 112 and 114 us; 83 x 64 x 71: 150 and 157 us.
+// (A_up by the u and p rows, A_ppi by the p and pi rows, z by all) can come
+// from L2 the second time.  One pass over every coefficient is 3.47 GB at 128^3,
+// with A_up and A_ppi read twice 3.97 GB; at 64^3 DRAM carries 501 MB, between
+// one pass (441) and two reads of both (504; as three launches 522).  Bound by
+// L1 and L2 requests, about 9.6 TB/s of coefficients (A_uu's lower blocks are
+// read a second time there).  128^3: 762 us, 787 us as three launches (497 +
+// 120 + 170); 64^3: 112 and 114 us; 83 x 64 x 71: 150 and 157 us.
 struct FfOp {
   int Lx, Ly, Lz;              // nodes per axis
   long long nN, nT;
@@ -1759,13 +1761,10 @@ void apply_operator_arnoldi(Ctx& c, const double* z, const float* zf, double* y,
   const long long most = std::max(std::max(c.nN, c.nFx), std::max(c.nFy, c.nF - c.nFx - c.nFy));
   k_apply_ff<<<lgrid(5 * grid_for(most, 256)), 256, 0, c.stream>>>(o, zf, y, lbytes());
   MHFP_LAUNCH_CHECK();
-  // algorithmic bytes, every coefficient a hi + lo pair (8 B): A_uu's
-  // symmetric half (126 per node) and A_up (24 per cell) by the u rows, A_up
-  // again, the p block (1 + 3) and A_ppi (6) by the p rows, A_ppi (6 per
-  // cell) and A_pipi (11 per face) by the pi rows; z read in FP32, y written
-  // in FP64
-  const double bytes = 8.0 * (126.0 * c.nN + (24.0 + 24.0 + 4.0 + 6.0 + 6.0) * c.nT + 11.0 * c.nF) + 4.0 * c.n +
-                       8.0 * c.n;
+  // algorithmic bytes, every coefficient a hi + lo pair (8 B) and read once:
+  // A_uu's symmetric half (126 per node), A_up (24 per cell), the p block (1 + 3),
+  // A_ppi (6 per cell) and A_pipi (11 per face); z read in FP32, y written in FP64
+  const double bytes = 8.0 * (126.0 * c.nN + (24.0 + 4.0 + 6.0) * c.nT + 11.0 * c.nF) + 4.0 * c.n + 8.0 * c.n;
   timing_end(c, 6, bytes);
 }
 

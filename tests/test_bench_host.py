@@ -68,3 +68,9 @@ def test_oracle_leg_runs_on_spawned_processes():
         assert [s[0] for s in st] == [3, 4] and wall > 0
         assert all(it > 0 and sec > 0 for _, _, it, sec in st)
         assert st[1][1] == sum(bench.make_problem_sizes_n("lognormal32", 4))
+
+
+def test_float_float_operator_bytes_count_each_coefficient_once():
+    # one cell: 8 nodes x 126, 24 + 4 + 6, 6 faces x 11 pairs of 8 B; 31 unknowns
+    assert bench.ff_operator_bytes(1) == 8 * (8 * 126 + 34 + 66) + 12 * 31
+    assert bench.ff_operator_bytes(64) == pytest.approx(441.0e6, rel=1e-3)

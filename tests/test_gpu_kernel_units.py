@@ -39,3 +39,20 @@ def test_sweeps_under_every_schedule():
     from paper_2002_09603_gb300 import LIB_PATH
     lib = os.path.dirname(os.path.abspath(LIB_PATH))
     _run("sweep_check.cu", "-L" + lib, "-lmhfp", "-Xlinker", "-rpath=" + lib)
+
+
+def test_registered_bytes_of_the_float_float_operator():
+    import bench
+    import mhfp_inputs as mi
+    from paper_2002_09603_gb300 import default_options, prepare
+    o = default_options()
+    o.precision, o.autotune = 1, 0
+    s = prepare(mi.random_small(5, 5, 5, seed=3), o)
+    x = torch.ones(s.n, dtype=torch.float64, device="cuda")
+    s.timing(True)
+    s.apply_operator_ff(x)
+    torch.cuda.synchronize()
+    t = s.timing_read(6)
+    s.timing(False)
+    assert t["launches"] == 1 and t["bytes_per_launch"] == bench.ff_operator_bytes(5)
+    s.close()
