@@ -12,14 +12,13 @@ namespace mhfp {
 // set-ups, 16 for the first of a process).  A candidate that is 1.15 times as
 // slow as `best_us` in the two replays after it has lost; one slow replay, as
 // the host or another client of the device causes it, does not drop a close
-// candidate.  Any other is replayed a fourth time.
+// candidate.  Any other is replayed a fourth time unless those two agree.
 template <class Replay>
 float best_replay_us(float best_us, Replay&& replay) {
   const float warm = replay();
   if (warm > 2.f * best_us) return warm;
-  float best = replay();
-  best = std::min(best, replay());
-  return best > 1.15f * best_us ? best : std::min(best, replay());
+  const float a = replay(), b = replay(), best = std::min(a, b);
+  return best > 1.15f * best_us || std::max(a, b) <= 1.05f * best ? best : std::min(best, replay());
 }
 
 }  // namespace mhfp
