@@ -1159,7 +1159,7 @@ __global__ void __launch_bounds__(256) k_build_Q1(Lat F, Lat Cc, const double* _
 // Jy slot) of a line's 96 points, so that the three residues share lines in
 // L1; a lane keeps up to three x slots of 3 x 3 sums.  Slots that are zero by
 // structure are not written (k_rap does not read them).  96^3, finest level:
-// 17.3 ms before, 6.9 ms.
+// 17.3 ms before, 6.5 ms (the FP64 pipe active 0.97 of the time).
 template <int RHO>
 __device__ __forceinline__ void q3_line(const Lat32& F, unsigned p, int a, int dy, int dz, int py, int pz,
                                         const double* __restrict__ val, const double* __restrict__ P,
@@ -1244,7 +1244,10 @@ __global__ void __launch_bounds__(288, 2) k_build_Q3(Lat32 F, Lat32 C, const dou
 // A_c[J, J+oc] = sum_{a in box(J)} P[a, J]^T Q[a, J+oc]   (BC x BC blocks).
 // A_c is symmetric: the centre and the offsets after it are formed, the rest
 // are their transposes (half the products; the stored operator is exactly
-// symmetric).  RAP_FIGURES
+// symmetric).  Bound by the FP64 pipe on large levels (96^3: the finest
+// displacement level 1.65 ms, the pipe active 0.88 of the time, the 25-point
+// level 1.0 ms, 0.83); all levels, every offset formed -> this: 5.5 -> 2.1 ms
+// (displacement) and 2.6 -> 1.1 ms (interface pressure).
 template <int BF, int BC, int CKIND>
 __global__ void k_rap(Lat F, Lat Cc, int R, const double* __restrict__ P, const double* __restrict__ Q,
                       const unsigned char* __restrict__ ac, double* __restrict__ Ac) {
@@ -2370,7 +2373,7 @@ void smooth(Ctx& c, std::vector<Level>& H, int l, const T* b, const T* x0, T* ds
         if (!xin)  // the first step from zero has no stencil work
           sweep_cheb_zero<T>(c.stream, lat.N, 3, v.dinv, b, out, v.d, v.cf);
         else
-          dispatch_u64(lat.N, U64_ROW_STEP, [&](auto F) {
+          dispatch_u64(lat.N, U64_SPLIT_NODES, U64_ROW_STEP, [&](auto F) {
             constexpr U64Form f = decltype(F)::value;
             k_cheb_u0<f><<<u64_grid<f>(lat.N), u64_block<f>(), 0, c.stream>>>(
                 lat, v.val, v.dinv, b, xin, out, v.d, v.cf + 2 * s, s == 0, lbytes());
@@ -2541,7 +2544,7 @@ void build_hierarchies(Ctx& c) {
   }
   if (c.opt.autotune) {
     // the finest displacement level runs k_cheb_u0 (FP64) or the symmetric
-    // FP32 sweep, whose two occupancy variants are timed; tune the others
+    // FP32 sweep, whose five variants are timed; tune the others
     // (schedules fixed by the options are not tuned)
     if (c.opt.precision == 1 && !c.hu[0].dense_inv && !c.opt.fine_blocks) autotune_fine_sym(c, c.hu[0]);
     for (auto* H : {&c.hu, &c.hpi})

@@ -28,9 +28,12 @@
 // 2,146,689  943/949 856/858 873/875      1003    932/933 928/930 942/948     1053    967/968 986/987 974/977
 // (the step in a solve, where the vectors lie elsewhere: 274,625 nodes 150 NODE,
 // 130 ROW, 145 loop; 2,146,689 nodes 932, 944 and 929).  So U64_SPLIT up to
-// U64_SPLIT_NODES, where it and the row form change places, U64_NODE for rows
-// and residuals from U64_ROW_ROWS nodes on and for the step from U64_ROW_STEP
-// on, U64_ROW between (the FP64 pipe's time at 2,146,689 nodes: 858, 890 and 943).
+// U64_SPLIT_NODES, for the operator up to U64_SPLIT_ROWS (its matrix is seldom
+// in L2 when it is applied, that of a sweep or residual often is); above, the
+// step takes U64_ROW up to U64_ROW_STEP, the operator up to U64_SPLIT_NODES,
+// and everything else is U64_NODE (393,120 nodes, both operators, the
+// float-float one and the norm in turn: 987 us, 995 with U64_ROW).  The FP64
+// pipe's time at 2,146,689 nodes: 858, 890 and 943.
 #pragma once
 #include "lattice.cuh"
 
@@ -38,7 +41,7 @@ namespace mhfp {
 namespace {
 
 enum U64Form { U64_NODE, U64_SPLIT, U64_ROW };
-constexpr long long U64_SPLIT_NODES = 60000, U64_ROW_ROWS = 450000, U64_ROW_STEP = 1500000;
+constexpr long long U64_SPLIT_NODES = 120000, U64_SPLIT_ROWS = 60000, U64_ROW_STEP = 1500000;
 constexpr int u64_nodes(U64Form f) { return f == U64_NODE ? 128 : 32; }  // nodes per block
 constexpr int u64_parts(U64Form f) { return f == U64_SPLIT ? 9 : (f == U64_ROW ? 3 : 1); }  // threads per node
 constexpr int u64_threads(U64Form f) { return u64_nodes(f) * u64_parts(f); }
@@ -193,11 +196,11 @@ __global__ void __launch_bounds__(u64_threads(F), u64_blocks(F))
   }
 }
 
-// f(form) with the form for N nodes, `row` the first size past the row form's
+// f(form): U64_SPLIT up to `split` nodes, U64_ROW up to `row`, U64_NODE above
 template <class F>
-void dispatch_u64(long long N, long long row, F&& f) {
-  if (N <= U64_SPLIT_NODES) f(std::integral_constant<U64Form, U64_SPLIT>{});
-  else if (N < row) f(std::integral_constant<U64Form, U64_ROW>{});
+void dispatch_u64(long long N, long long split, long long row, F&& f) {
+  if (N <= split) f(std::integral_constant<U64Form, U64_SPLIT>{});
+  else if (N <= row) f(std::integral_constant<U64Form, U64_ROW>{});
   else f(std::integral_constant<U64Form, U64_NODE>{});
 }
 
@@ -206,11 +209,12 @@ dim3 u64_grid(long long N) { return lgrid(grid_for(N, u64_nodes(F))); }
 template <U64Form F>
 dim3 u64_block() { return dim3(u64_nodes(F), u64_parts(F)); }
 
+// the operator's u rows (Aup given) or a product or residual
 template <class... Args>
-void launch_u64(cudaStream_t stream, const Lat32& L, Args... args) {
-  dispatch_u64(L.N, U64_ROW_ROWS, [&](auto F) {
+void launch_u64(cudaStream_t stream, const Lat32& L, const double* A, const double* Aup, Args... args) {
+  dispatch_u64(L.N, Aup ? U64_SPLIT_ROWS : U64_SPLIT_NODES, U64_SPLIT_NODES, [&](auto F) {
     constexpr U64Form f = decltype(F)::value;
-    k_u64<f><<<u64_grid<f>(L.N), u64_block<f>(), 0, stream>>>(L, args..., lbytes());
+    k_u64<f><<<u64_grid<f>(L.N), u64_block<f>(), 0, stream>>>(L, A, Aup, args..., lbytes());
   });
 }
 

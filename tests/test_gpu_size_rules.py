@@ -49,8 +49,9 @@ def _vcycle_close(s, which, ref, b, tol):
     assert np.abs(got - ref).max() <= tol * np.abs(ref).max()
 
 
-# FP64 displacement rows by a thread per row (60,001 nodes and up): both
-# operators, and the sweeps and the residual of the V-cycle
+# FP64 displacement rows: both operators by a thread per row, the V-cycle's steps
+# and residual by nine threads per node (its steps by a thread per row: the 64^3
+# V-cycle of test_gpu_fullsize)
 def test_fp64_rows_by_a_thread_per_row(mesh, oracle_pc):
     prob, B = mesh
     s = _solver(prob, autotune=0)
