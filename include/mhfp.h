@@ -99,10 +99,10 @@ typedef struct {
                         /* coarse level's smoother at set-up (one point per    */
                         /* thread, the stencil offsets split over 4, 8 or 16   */
                         /* warps, or a warp or eight lanes per point on row-   */
-                        /* major values) and the two occupancy variants of the */
-                        /* finest FP32 displacement sweep, and keep the        */
-                        /* fastest (schedule only: the same products, summed   */
-                        /* in a schedule-dependent fixed order)                */
+                        /* major values) and the five variants of the finest   */
+                        /* FP32 displacement sweep (see fine_blocks), and keep */
+                        /* the fastest (schedule only: the same products,      */
+                        /* summed in a schedule-dependent fixed order)         */
   int reorth;           /* Gram-Schmidt of each Arnoldi step (the paper names  */
                         /* GMRES in PETSc, Section 5, and no orthogonalisation)*/
                         /* 1 (default): classical Gram-Schmidt, repeated once  */
@@ -160,10 +160,12 @@ typedef struct {
                         /* levels with the rigid-body modes, 1 for pi)         */
   double lmax[8];       /* 1.1 * rho(D^-1 A) per level (0 on the last level)   */
   int schedule[8];      /* launch schedule of the level's sweeps: 1 = one point */
-                        /* per thread, 4/8/16 = offsets split over that many    */
-                        /* warps, 32/64 = a warp / eight lanes per point on     */
-                        /* row-major values (small levels); finest FP32 displacement level: fine_blocks  */
-                        /* (4, 6 or 8); 0 = not a lattice sweep                */
+                        /* per thread, 4/8/16 = offsets split over that many   */
+                        /* warps, 32/64 = a warp / eight lanes per point on    */
+                        /* row-major values (small levels; taken by the size   */
+                        /* rule or the autotuner, not an option); finest FP32  */
+                        /* displacement level: fine_blocks (4 to 8); 0 = not a */
+                        /* lattice sweep                                       */
   double sweep_us[8];   /* set-up autotuner's time of one sweep under that     */
                         /* schedule, microseconds (0 when not timed)           */
   int cheb_degree;      /* Chebyshev degree of the smoothers in use            */

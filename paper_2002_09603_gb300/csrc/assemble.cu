@@ -96,7 +96,8 @@ __device__ __forceinline__ void load_cell_coords(const Dims& d, const double* __
 // is one full row segment; warp q first forms the gradients at Gauss point q
 // in shared memory, then warp a takes the pairs (a, a + d mod 8), d = 0..3,
 // and d = 4 for a < 4 (nine pairs per scheduler).  96^3 cells: 49.5 ms before
-// (one warp per cell, a store per lane and row), 7.93 ms now (0.92 of the FP64 pipe).
+// (one warp per cell, a store per lane and row), 7.9 ms now (the FP64 pipe
+// active 0.94 of the time).
 constexpr int Q1_CELLS = 32;
 // row of entry (i, j) of the element matrices, stored as upper triangles
 // [300][cells] (half the bytes to allocate, write and give back: about 2 ms of

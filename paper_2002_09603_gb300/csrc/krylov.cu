@@ -34,12 +34,9 @@ __device__ __forceinline__ double block_sum(double v, double* sh) {
 // per thread, many rows in flight, independent FMA chains.
 constexpr int GS_BLOCKS = 1216;   // 8 x 152 SMs
 constexpr int GS_COLS = 8;        // columns per block in the dot kernel (w is read once per 8 columns)
-constexpr int GS_DOT_BLOCKS = 608;  // 4 x 152 SMs: about 12 rows per thread, so the
-                                    // block reductions' FP64 adds stay small
+constexpr int GS_DOT_BLOCKS = 608;  // 4 x 152 SMs at most (gs_dot_blocks): the fewer the
+                                    // blocks, the fewer FP64 adds in their reductions
 
-// partials[c][block] = sum over this block's rows of V[:,c] . w for the
-// GS_COLS columns of blockIdx.y; block column 0 also sums w . w into slot
-// `ncols` when with_norm.  Skipped entirely when skip && *skip.
 // Sum of a[0..7] over the warp by a transposed butterfly: each exchange
 // halves the number of live columns per lane, so the eight sums cost 7 + 2
 // FP64 adds and shuffles per lane instead of 40.  Lane 4q + r (r = 0..3)

@@ -54,6 +54,8 @@ def test_element_kernels_at_tile_edges(dims):
 # FP64 rows of the displacement level: 32 nodes per block (operator, sweeps,
 # residual), 256 per block in the allocation-free norm; at most 300,000 nodes
 # here (the form above that runs in the 128^3 test)
+# (the lines are U64_SPLIT_ROWS, U64_SPLIT_NODES and NA_SPLIT_NODES, 60,000 to
+# 120,000; the form between runs in test_gpu_size_rules)
 @pytest.mark.parametrize("dims", [(7, 1, 1), (10, 1, 2), (1, 3, 15), (15, 3, 3), (4, 5, 9)])
 def test_fp64_rows_at_tile_edges(dims):
     prob = mi.random_small(*dims, seed=11, jitter=0.2)
@@ -96,6 +98,7 @@ def test_arnoldi_vectors_at_edges(dims, restart, reorth, precision):
     s.close()
 
 
+# (through the library's vectors; the functions alone, over every branch: test_gpu_kernel_units)
 def test_conversions_match_the_instructions():
     """The integer-pipe FP32 <-> FP64 conversions (vectors that the mixed form
     rounds and widens) bit for bit, over every exponent, ties, signed zeros,
@@ -137,6 +140,7 @@ def test_float_float_operator_row_families(dims):
 # row-major sweeps and residuals (a warp or eight lanes per point) as the
 # autotuner and the size rule pick them: box levels of 1 to a few thousand
 # points (a last block that is not full), 1, 3 and 6 unknowns per point
+# (every schedule by itself, eight lanes among them: test_gpu_kernel_units)
 @pytest.mark.parametrize("near_kernel", [0, 1])
 @pytest.mark.parametrize("precision", [0, 1])
 @pytest.mark.parametrize("dims,autotune", [((12, 10, 4), 0), ((12, 10, 4), 1), ((45, 7, 7), 0)])
