@@ -1807,28 +1807,36 @@ void make_dense_coarse(Ctx& c, Level& L) {
 }
 
 // the Chebyshev recurrence's coefficients on [lmax / ratio, lmax]: step 0 is d
-// = (1 / theta) D^-1 r, step s > 0 is d = cd d + cr D^-1 r
+// = (1 / theta) D^-1 r, step s > 0 is d = cd d + cr D^-1 r.  They travel as a
+// kernel argument: no copy from host memory that the stream would have to be
+// waited for, in every level of a set-up and of a permeability update.
+constexpr int CHEB_STEPS = 8;
+struct ChebCoefficients {
+  double v[2 * CHEB_STEPS];
+};
+__global__ void k_cheb_coefficients(ChebCoefficients h, double* __restrict__ cf, float* __restrict__ cff) {
+  const int i = threadIdx.x;
+  cf[i] = h.v[i];
+  cff[i] = narrow(h.v[i]);
+}
+
 void write_cheb_coefficients(Ctx& c, Level& L) {
-  constexpr int STEPS = 8;
   const double lmin = L.lmax / c.opt.cheb_ratio;
   const double theta = 0.5 * (L.lmax + lmin), delta = 0.5 * (L.lmax - lmin), sigma = theta / delta;
-  double cf[2 * STEPS];
-  float cff[2 * STEPS];
+  ChebCoefficients h;
   double rho = 1.0 / sigma;
-  cf[0] = 0.0;
-  cf[1] = 1.0 / theta;
-  for (int s = 1; s < STEPS; ++s) {
+  h.v[0] = 0.0;
+  h.v[1] = 1.0 / theta;
+  for (int s = 1; s < CHEB_STEPS; ++s) {
     const double rn = 1.0 / (2.0 * sigma - rho);
-    cf[2 * s] = rn * rho;
-    cf[2 * s + 1] = 2.0 * rn / delta;
+    h.v[2 * s] = rn * rho;
+    h.v[2 * s + 1] = 2.0 * rn / delta;
     rho = rn;
   }
-  for (int i = 0; i < 2 * STEPS; ++i) cff[i] = (float)cf[i];
-  if (!L.cf) L.cf = dalloc_n<double>(c, 2 * STEPS);
-  if (!L.cff) L.cff = dalloc_n<float>(c, 2 * STEPS);
-  MHFP_CUDA(cudaMemcpyAsync(L.cf, cf, sizeof(cf), cudaMemcpyHostToDevice, c.stream));
-  MHFP_CUDA(cudaMemcpyAsync(L.cff, cff, sizeof(cff), cudaMemcpyHostToDevice, c.stream));
-  MHFP_CUDA(cudaStreamSynchronize(c.stream));  // cf and cff are this call's
+  if (!L.cf) L.cf = dalloc_n<double>(c, 2 * CHEB_STEPS);
+  if (!L.cff) L.cff = dalloc_n<float>(c, 2 * CHEB_STEPS);
+  k_cheb_coefficients<<<1, 2 * CHEB_STEPS, 0, c.stream>>>(h, L.cf, L.cff);
+  MHFP_LAUNCH_CHECK();
 }
 
 void finish_level(Ctx& c, Level& L) {
