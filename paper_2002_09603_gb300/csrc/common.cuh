@@ -543,7 +543,7 @@ struct Ctx {
   long long solve_step_kernels[2] = {0, 0};   // kernels of one Arnoldi step
   int solve_pending = 0;
   std::chrono::steady_clock::time_point solve_t0;
-  int graph_gen = 0;                     // bumped whenever captured graphs are dropped
+  int graph_gen = 0;                     // bumped when captured graphs are dropped and by a permeability update: older batches are stale
   DevCtl* ctl = nullptr;                 // device control block
   DevCtl* host_ctl = nullptr;            // pinned copy
   double *bcur = nullptr, *xcur = nullptr;
